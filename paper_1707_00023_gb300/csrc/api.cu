@@ -11,6 +11,7 @@
 #include <thread>
 #include <vector>
 
+#include "kx_cdense.cuh"
 #include "kx_internal.cuh"
 
 using namespace kx;
@@ -524,6 +525,7 @@ kx_status create_impl(const kx_desc* desc, const double* eps_cell, const uint8_t
       {(void**)&c->d_tmp, (size_t)c->n * c->esize},
       {(void**)&c->d_tmp2, (size_t)c->n * c->esize},
       {(void**)&c->d_expm_ws, (size_t)(MMAX + 1) * MMAX * MAXF * sizeof(double)},
+      {(void**)&c->d_cd_ws, (size_t)std::max(2, B) * CD_WS * sizeof(double)},
       {(void**)&c->d_zre, (size_t)d.max_freqs * c->n * c->esize},
       {(void**)&c->d_zim, (size_t)d.max_freqs * c->n * c->esize},
       {(void**)&c->d_swT, (size_t)c->n * c->esize},
@@ -675,7 +677,7 @@ kx_status krylov_expm_destroy(kx_ctx* c) {
   cudaStreamSynchronize(c->stream);
   void* ptrs[] = {c->d_inv_eps, c->d_sig2, c->d_eps_cell, c->d_V, c->d_aug, c->d_H, c->d_scale,
                   c->d_part, c->d_counter, c->d_u, c->d_state, c->d_rho, c->d_coef, c->d_coefd,
-                  c->d_omegas, c->d_small, c->d_tmp, c->d_tmp2, c->d_expm_ws, c->d_zre, c->d_zim,
+                  c->d_omegas, c->d_small, c->d_tmp, c->d_tmp2, c->d_expm_ws, c->d_cd_ws, c->d_zre, c->d_zim,
                   c->d_ckpt, c->d_adj_Q, c->d_adj_alpha, c->d_adj_omg, c->d_adj_cw, c->d_adj_sn,
                   c->d_gauss, c->d_rst_b, c->d_rst_smp, c->d_rst_mats, c->d_rst_u, c->d_rst_res,
                   c->d_rst_state, c->d_rst_yp, c->d_swT, c->d_swpart, c->d_swG, c->d_swco};

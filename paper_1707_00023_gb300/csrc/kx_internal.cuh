@@ -220,6 +220,7 @@ struct kx_ctx {
   void* d_tmp;              // one extra vector
   void* d_tmp2;             // one extra vector
   double* d_expm_ws;        // projected exponential workspace
+  double* d_cd_ws;          // cluster-wide dense work (kx_cdense.cuh), one piece a slot, two at least
   // adjoint workspace (max_checkpoints > 0)
   void* d_ckpt = nullptr;   // max_checkpoints states of the forward solution
   double* d_adj_Q = nullptr;      // per-E-node time integrals
