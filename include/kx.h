@@ -91,7 +91,7 @@ typedef struct {
                           otherwise batch >= 2); one per time sub-step       */
   int rst_samples;    /* time samples of [0, T] per frequency kept by the
                          restart-in-dimension method (0: method unavailable);
-                         the workspace is max_freqs * rst_samples * 72
+                         the workspace is max_freqs * rst_samples * 104
                          bytes plus max_freqs output-plane accumulators      */
   int pml;            /* 0: lossy layer (above).  1: the paper's perfectly
                          matched layer (2D, layer_axis 0 only; Sect. 2.1,

@@ -582,6 +582,9 @@ kx_status create_impl(const kx_desc* desc, const double* eps_cell, const uint8_t
         {(void**)&c->d_rst_b, (size_t)d.max_freqs * d.rst_samples * RST_P * sizeof(double)},
         {(void**)&c->d_rst_smp, (size_t)d.max_freqs * (d.rst_samples + 1) * 3 * sizeof(double)},
         {(void**)&c->d_rst_mats, (size_t)RST_MATS * sizeof(double)},
+        {(void**)&c->d_rst_fu,
+         (size_t)d.max_freqs * ((size_t)(d.rst_samples + RST_L - 1) / RST_L) * MMAX * sizeof(double)},
+        {(void**)&c->d_rst_cnt, (size_t)MAXF * sizeof(unsigned)},
         {(void**)&c->d_rst_u, (size_t)MAXF * MMAX * sizeof(double)},
         {(void**)&c->d_rst_res, (size_t)MAXF * sizeof(double)},
         {(void**)&c->d_rst_state, (size_t)MAXF * sizeof(int)},
@@ -679,7 +682,7 @@ kx_status krylov_expm_destroy(kx_ctx* c) {
                   c->d_part, c->d_counter, c->d_u, c->d_state, c->d_rho, c->d_coef, c->d_coefd,
                   c->d_omegas, c->d_small, c->d_tmp, c->d_tmp2, c->d_expm_ws, c->d_cd_ws, c->d_zre, c->d_zim,
                   c->d_ckpt, c->d_adj_Q, c->d_adj_alpha, c->d_adj_omg, c->d_adj_cw, c->d_adj_sn,
-                  c->d_gauss, c->d_rst_b, c->d_rst_smp, c->d_rst_mats, c->d_rst_u, c->d_rst_res,
+                  c->d_gauss, c->d_rst_b, c->d_rst_smp, c->d_rst_mats, c->d_rst_fu, c->d_rst_cnt, c->d_rst_u, c->d_rst_res,
                   c->d_rst_state, c->d_rst_yp, c->d_swT, c->d_swpart, c->d_swG, c->d_swco};
   for (void* p : ptrs)
     if (p) cudaFree(p);

@@ -125,16 +125,15 @@ __host__ __device__ __forceinline__ int64_t plane_node(const Geo& g, int axis, i
 }
 
 // Restart in Krylov dimension: polynomial degree + 1 of the interpolated
-// source on one sample interval, and the layout (in doubles) of the per-
-// restart set-up record: E = exp(-d H_m) (MMAX x MMAX, row-major), the
-// interval responses W_j (RST_P x MMAX), the last rows of H_m and H_m^2, and
-// the scalars h_{m+1,m}, (H_m)_{m,1}, m.
+// source on one sample interval, intervals a chunk of the march (rstdim.cu),
+// and the layout (in doubles) of the per-restart tables: E^L (MMAX x MMAX,
+// row-major), the sources' responses at a chunk's end (L RST_P x MMAX) and the
+// sampling rows ((MMAX + L RST_P) x 3 L).
 constexpr int RST_P = 6;
-constexpr int RST_OFF_W = MMAX * MMAX;
-constexpr int RST_OFF_R1 = RST_OFF_W + RST_P * MMAX;
-constexpr int RST_OFF_R2 = RST_OFF_R1 + MMAX;
-constexpr int RST_OFF_SC = RST_OFF_R2 + MMAX;
-constexpr int RST_MATS = RST_OFF_SC + 8;
+constexpr int RST_L = 16;
+constexpr int RST_OFF_Z = MMAX * MMAX;
+constexpr int RST_OFF_R = RST_OFF_Z + RST_L * RST_P * MMAX;
+constexpr int RST_MATS = RST_OFF_R + (MMAX + RST_L * RST_P) * 3 * RST_L;
 
 // Single-sweep Arnoldi (sweep.cu): reduced partial columns of the last
 // pass, and the coefficients the next sweep applies.  One record per slot.
@@ -235,7 +234,9 @@ struct kx_ctx {
   // restart in Krylov dimension (rst_samples > 0)
   double* d_rst_b = nullptr;     // 2 x max_freqs x rst_samples x RST_P source coefficients
   double* d_rst_smp = nullptr;   // max_freqs x (rst_samples + 1) x 3 alphahat samples
-  double* d_rst_mats = nullptr;  // set-up record of the current restart
+  double* d_rst_mats = nullptr;  // tables of the current restart
+  double* d_rst_fu = nullptr;    // max_freqs x chunks x MMAX: the chunks' sources, then their u
+  unsigned* d_rst_cnt = nullptr; // MAXF block counters of the sampling
   double* d_rst_u = nullptr;     // MAXF x MMAX projected solutions u(T)
   double* d_rst_res = nullptr;   // MAXF residual maxima
   int* d_rst_state = nullptr;    // MAXF: 0 active, 1 stops after this restart, 2 stopped

@@ -21,11 +21,12 @@
 //   alphahat'' = -h e_m^T (H_m^2 u - alpha H_m e_1 + alpha' e_1).
 //
 //   k_rst_source   restart 1's source ||g|| sin(W t) as interval coefficients.
-//   k_rst_setup    one CTA: E and the W_j from one exponential of the
+//   k_rst_setup    one cluster: E and the W_j from one exponential of the
 //                  (m+6)-square matrix [[-d H_m, e_1 e_1^T], [0, J]] (J the
-//                  6x6 shift; its top right block holds phi_1..phi_6 (-d H_m) e_1).
-//   k_rst_cascade  one CTA per frequency: the Nt interval maps, E held in
-//                  registers; a fifth warp samples alphahat and its first two
+//                  6x6 shift; its top right block holds phi_1..phi_6 (-d H_m) e_1),
+//                  and the tables that advance a chunk of 16 intervals at once.
+//   k_rst_drive, k_rst_march, k_rst_sample
+//                  the Nt interval maps in chunks; alphahat and its first two
 //                  derivatives at every grid point.
 //   k_rst_coef     the next restart's interval coefficients from those
 //                  samples (all intervals in parallel).
@@ -34,8 +35,8 @@
 #include <atomic>
 #include <cmath>
 
+#include "kx_cdense.cuh"
 #include "kx_internal.cuh"
-#include "kx_dense.cuh"
 #include "kx_reduce.cuh"
 
 namespace kx {
@@ -80,240 +81,363 @@ kx_status launch_rst_source(kx_ctx* c, cudaStream_t st, int nfreq, double beta, 
 }
 
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_rst_setup(const double* __restrict__ H, int ldh,
-                                                   const SlotState* st, double d, double* mats,
-                                                   double* gbuf, int* status) {
+// Set-up of one restart, one cluster (kx_cdense.cuh): E and the W_j from one
+// exponential of order m + 6, then the chunk tables by doubling.  With G =
+// E^P known (P = 1, 2, 4, 8), the blocks hold their rows of G and stage all of
+// it:  E^2P = G G,  Z_{P+l} = G Z_l (Z_l = E^l W, l < P),  R_{P+l} = R_l G
+// (R_l = C E^l, C the three sampling rows); one cluster barrier a doubling.
+// On one block (the exponential alone, 64 dependent pivots of its solve) the
+// set-up took 1060 us at m = 64.
+constexpr int RST_ZC = RST_L * RST_P;                   // columns of [Z_0 .. Z_{L-1}]
+constexpr int RST_O = 3 * RST_L;                        // sampled values of a chunk
+constexpr int RST_SMEM = CD_SMEM + MMAX * CD_LD * (int)sizeof(double);
+static_assert(RST_L == 16, "four doublings");
+static_assert(RST_ZC / 2 <= CD_LD && RST_O <= MMAX, "the half-filled tables fit the shared operands");
+
+__global__ void __launch_bounds__(CD_THREADS) k_rst_setup(const double* __restrict__ H, int ldh, const SlotState* st,
+                                                          double d, double* mats, double* ws, int* status) {
+  extern __shared__ __align__(16) double sm[];
   __shared__ double red[32];
-  __shared__ double lv[MMAX + RST_P + 2];
-  __shared__ int piv;
+  const int rank = cl_rank(), tid = threadIdx.x;
   const int md = st->m_done;
-  if (md < 1 || st->status) {
-    // the Arnoldi process's own status (a non-finite value, a bounded wait
-    // that ran out), else no step completed
-    if (threadIdx.x == 0) *status = st->status ? st->status : KX_ENONFINITE;
-    return;
-  }
-  // the six (m+6)-square work matrices live in global memory (L1/L2
-  // resident): a large shared-memory request would keep this CTA off every
-  // SM that runs the Arnoldi passes, which this kernel overlaps
   const int n = md + RST_P;
-  double* buf[6];
-  for (int q = 0; q < 6; ++q) buf[q] = gbuf + (size_t)q * n * n;
-  for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) {
-    const int r = idx / n, c = idx - r * n;
-    double v = 0.0;
-    if (r < md && c < md) v = (r <= c + 1) ? -d * H[r + (int64_t)c * ldh] : 0.0;
-    else if (r == 0 && c == md) v = 1.0;
-    else if (r >= md && c == r + 1) v = 1.0;
-    buf[0][idx] = v;
-  }
-  __syncthreads();
-  double* X = cta_expm(buf, n, red, lv, &piv);
-  if (!X) {
-    if (threadIdx.x == 0) *status = KX_ENONFINITE;
+  // (m+6)-square [[-d H_m, e_1 e_1^T], [0, J]], J the shift
+  auto entry = [&](int r, int c) {
+    if (r < md && c < md) return r <= c + 1 ? -d * H[r + (int64_t)c * ldh] : 0.0;
+    return (r == 0 && c == md) || (r >= md && c == r + 1) ? 1.0 : 0.0;
+  };
+  int q = 0, s = 0;
+  const bool ok = md >= 1 && !st->status;
+  if (!ok || !cd_plan(cd_norm1(n, red, entry), 1, &q, &s)) {
+    // the Arnoldi process's own status (a non-finite value, a bounded wait
+    // that ran out), else no step completed or a non-finite matrix
+    if (rank == 0 && tid == 0) *status = st->status ? st->status : KX_ENONFINITE;
     return;
   }
-  for (int idx = threadIdx.x; idx < MMAX * MMAX; idx += blockDim.x) {
-    const int r = idx / MMAX, c = idx - r * MMAX;
-    mats[idx] = (r < md && c < md) ? X[r * n + c] : 0.0;
-  }
-  for (int idx = threadIdx.x; idx < RST_P * MMAX; idx += blockDim.x) {
-    const int j = idx / MMAX, r = idx - j * MMAX;
-    double fact = 1.0;
-    for (int q = 2; q <= j; ++q) fact *= q;
-    mats[RST_OFF_W + idx] = (r < md) ? d * fact * X[r * n + md + j] : 0.0;
-  }
-  // last rows of H_m and H_m^2 (row m-1 of H_m is nonzero in columns m-2, m-1)
+  const CdShared sh = cd_shared(sm);
+  double* Zs = sm + CD_SMEM / sizeof(double);
+  const CdRows w = cd_rows(n, rank);
+  const int R = max(0, min(w.R, md - w.r0));   // own rows among the first md
+  const double sc = ldexp(1.0, -s);
+  double* P = cd_expm(sh, ws, n, w, q, s, [&](int r, int c) { return sc * entry(r, c); });
+  double* Q = P == sh.S[3] ? sh.S[4] : sh.S[3];
+  double* gE = ws + 2 * CD_MAT;                // E^P, two in turn
+  double* gZ = ws + 4 * CD_MAT;                // Z, row stride RST_ZC
+  double* gR = gZ + MMAX * RST_ZC;             // R, row stride MMAX
+  static_assert(4 * CD_MAT + MMAX * RST_ZC + RST_O * MMAX <= CD_WS, "the workspace holds the tables");
+  // C: last rows of -h I, h H_m and -h H_m^2 (nonzero in the last three columns)
+  const double h = st->done ? 0.0 : H[md + (int64_t)(md - 1) * ldh];
   const int lr = md - 1;
-  for (int c = threadIdx.x; c < MMAX; c += blockDim.x) {
-    double r1 = 0.0, r2 = 0.0;
-    if (c < md) {
-      if (lr <= c + 1) r1 = H[lr + (int64_t)c * ldh];
-      for (int k = max(0, lr - 1); k < md; ++k)
-        if (k <= c + 1) r2 += H[lr + (int64_t)k * ldh] * H[k + (int64_t)c * ldh];
-    }
-    mats[RST_OFF_R1 + c] = r1;
-    mats[RST_OFF_R2 + c] = r2;
+  auto crow = [&](int comp, int c) {
+    if (c < lr - 2) return 0.0;
+    if (comp == 0) return c == lr ? -h : 0.0;
+    if (comp == 1) return c >= lr - 1 ? h * H[lr + (int64_t)c * ldh] : 0.0;
+    double v = 0.0;
+    for (int k = max(0, lr - 1); k < md; ++k)
+      if (k <= c + 1) v += H[lr + (int64_t)k * ldh] * H[k + (int64_t)c * ldh];
+    return -h * v;
+  };
+  for (int o = tid; o < R * md; o += CD_THREADS) {
+    const int r = o / md, c = o - r * md;
+    gE[(w.r0 + r) * CD_LD + c] = P[r * CD_LD + c];
   }
-  if (threadIdx.x == 0) {
-    mats[RST_OFF_SC + 0] = st->done ? 0.0 : H[md + (int64_t)(md - 1) * ldh];
-    mats[RST_OFF_SC + 1] = (lr <= 1) ? H[lr] : 0.0;
-    mats[RST_OFF_SC + 2] = (double)md;
+  for (int o = tid; o < R * RST_P; o += CD_THREADS) {
+    const int r = o / RST_P, j = o - r * RST_P;
+    double f = d;
+    for (int k = 2; k <= j; ++k) f *= k;
+    gZ[(w.r0 + r) * RST_ZC + j] = f * P[r * CD_LD + md + j];
+  }
+  if (rank == 0)
+    for (int o = tid; o < 3 * md; o += CD_THREADS) {
+      const int comp = o / md, c = o - comp * md;
+      gR[comp * MMAX + c] = crow(comp, c);
+    }
+  cl_sync();
+  for (int k = 0; (1 << k) < RST_L; ++k) {
+    const int half = 1 << k;
+    const double* cur = gE + (k & 1) * CD_MAT;
+    double* nxt = gE + ((k & 1) ^ 1) * CD_MAT;
+    cd_load(sh.B, cur, md, md);
+    for (int o = tid; o < md * half * (RST_P / 2); o += CD_THREADS) {
+      const int r = o / (half * (RST_P / 2)), c = 2 * (o - r * (half * (RST_P / 2)));
+      *reinterpret_cast<double2*>(Zs + r * CD_LD + c) = __ldcg(reinterpret_cast<const double2*>(gZ + r * RST_ZC + c));
+    }
+    // this block's share of the sampling rows
+    const int per = (3 * half + CD_CTAS - 1) / CD_CTAS;
+    const int s0 = min(3 * half, rank * per), ns = min(3 * half, s0 + per) - s0;
+    for (int o = tid; o < ns * md; o += CD_THREADS) {
+      const int r = o / md, c = o - r * md;
+      sh.S[0][r * CD_LD + c] = __ldcg(gR + (s0 + r) * MMAX + c);
+    }
+    __syncthreads();
+    cd_mm(P, sh.B, R, md, md, [&](int r, int c, double v) {
+      Q[r * CD_LD + c] = v;
+      nxt[(w.r0 + r) * CD_LD + c] = v;
+    });
+    cd_mm(P, Zs, R, md, half * RST_P,
+          [&](int r, int c, double v) { gZ[(w.r0 + r) * RST_ZC + half * RST_P + c] = v; });
+    cd_mm(sh.S[0], sh.B, ns, md, md, [&](int r, int c, double v) { gR[(3 * half + s0 + r) * MMAX + c] = v; });
+    cl_sync();
+    double* t = P;
+    P = Q;
+    Q = t;
+  }
+  // the tables of the marching kernels, zero past the basis' size
+  const double* EL = gE;                       // E^16 after four doublings
+  const int t0 = rank * CD_THREADS + tid, nt = CD_CTAS * CD_THREADS;
+  for (int o = t0; o < MMAX * MMAX; o += nt) {
+    const int r = o / MMAX, c = o % MMAX;
+    mats[o] = r < md && c < md ? __ldcg(EL + r * CD_LD + c) : 0.0;
+  }
+  for (int o = t0; o < RST_ZC * MMAX; o += nt) {
+    const int k = o / MMAX, r = o % MMAX, qq = k / RST_P, j = k % RST_P;
+    mats[RST_OFF_Z + o] = r < md ? __ldcg(gZ + r * RST_ZC + (RST_L - 1 - qq) * RST_P + j) : 0.0;
+  }
+  const double hm0 = lr <= 1 ? H[lr] : 0.0, del = md == 1 ? 1.0 : 0.0;
+  for (int o = t0; o < (MMAX + RST_ZC) * RST_O; o += nt) {
+    const int k = o / RST_O, c = o % RST_O, r = c / 3, comp = c % 3;
+    double v = 0.0;
+    if (k < MMAX) {
+      if (k < md) v = __ldcg(gR + c * MMAX + k);
+    } else {
+      const int qq = (k - MMAX) / RST_P, j = (k - MMAX) % RST_P;
+      if (qq < r) {
+        for (int i = max(0, lr - 2); i <= lr; ++i)
+          v = fma(crow(comp, i), __ldcg(gZ + i * RST_ZC + (r - 1 - qq) * RST_P + j), v);
+      } else if (qq == r) {
+        // alphahat' and alphahat'' carry the source and its slope (b_1 = d alpha')
+        if (j == 0) v = comp == 1 ? -h * del : (comp == 2 ? h * hm0 : 0.0);
+        if (j == 1 && comp == 2) v = -h * del / d;
+      }
+    }
+    mats[RST_OFF_R + o] = v;
   }
 }
 
 kx_status launch_rst_setup(kx_ctx* c, cudaStream_t st, int slot, double d) {
   Slot<float> s = make_slot<float>(c, slot);
   int* status = reinterpret_cast<int*>(c->d_small + 64);
+  static SmemOptIn attr{};
+  const kx_status so = smem_opt_in(c, attr, (const void*)k_rst_setup, RST_SMEM);
+  if (so != KX_OK) return so;
   time_begin(c);
-  k_rst_setup<<<1, 256, 0, st>>>(s.H, c->m + 1, s.st, d, c->d_rst_mats,
-                                                            c->d_expm_ws, status);
+  launch_cluster(k_rst_setup, 1, RST_SMEM, st, (const double*)s.H, c->m + 1, (const SlotState*)s.st, d, c->d_rst_mats,
+                 c->d_cd_ws, status);
   time_end(c, KX_K_PROJ, 0.0);
   KX_CHECK_LAUNCH(c);
   return KX_OK;
 }
 
 // ---------------------------------------------------------------------------
-// One CTA per frequency.  Threads 0..127 apply the interval map, two per
-// row r = tid / 2, columns q + 2k (q = tid % 2) with E's entries in
-// registers; each adds half of the source responses b_j W_j[r] before the
-// pair's sum.  Threads 128..159 (the sampling warp) read u_i meanwhile and
-// write alphahat, d alphahat / dt and d2 alphahat / dt2 at t_i (lanes 0, 1,
-// 2, each five FMAs: the last rows of H_m and H_m^2 touch only u's last
-// three entries).  u is double-buffered in shared memory, one barrier per
-// interval.  On this GPU a double-precision warp instruction costs the same
-// issue time whatever its active lanes, so the interval's FP64 instruction
-// count per warp is what the layout minimises.
-constexpr int RST_MV = 2 * MMAX;
-constexpr int RST_THREADS = RST_MV + 32;
+// The march over the Nt intervals, in chunks of L = RST_L.  Done interval by
+// interval it is Nt dependent products with E, one block a frequency: 4.5k
+// double-precision FMAs an interval on one SM's slow pipe, 3.2 ms for Nt =
+// 2160.  Over a chunk starting at u_c,
+//   u_{c+1}        = E^L u_c + F_c,   F_c = sum_q Z_{L-1-q} b_q,
+//   s_r (r < L)    = R_r u_c + sum_{q<r} C Z_{r-1-q} b_q + D b_r
+// (s the samples alphahat, alphahat', alphahat''; D the source's own share),
+// so only the short recursion over chunks is serial:
+//   k_rst_drive    F_c of every chunk and frequency (a 64 x 6L product)
+//   k_rst_march    u_{c+1} = E^L u_c + F_c, one block a frequency
+//   k_rst_sample   the samples of every chunk (a 3L x (64 + 6L) product)
+// about 860 FMAs an interval, all but 256 of them spread over the GPU.  L = 16
+// balances the serial part (64^2 / L an interval) against the samples' share
+// (grows with L) and the tables' set-up (log L products).
+// The first chunk may be short: it starts pad = Nt_chunks L - Nt intervals
+// early with u = 0 and no source, so every chunk is treated alike.
+constexpr int RST_CB = 4;   // chunks a block of the parallel kernels
 
-__global__ void __launch_bounds__(RST_THREADS) k_rst_cascade(const double* __restrict__ mats,
-                                                            const double* __restrict__ b,
-                                                            double* __restrict__ smp, int Nt, double d,
-                                                            double tol_abs, int* fstate, double* resid,
-                                                            double* u_out) {
+__device__ __forceinline__ int rst_chunks(int Nt) { return (Nt + RST_L - 1) / RST_L; }
+
+// The source coefficients of chunks c0 .. c0 + RST_CB - 1 to shared memory.
+__device__ __forceinline__ void rst_load_b(double* sb, const double* __restrict__ bf, int c0, int nch, int pad) {
+  for (int o = threadIdx.x; o < RST_CB * RST_ZC; o += blockDim.x) {
+    const int64_t k = (int64_t)c0 * RST_ZC + o - (int64_t)pad * RST_P;
+    sb[o] = (c0 + o / RST_ZC < nch && k >= 0) ? bf[k] : 0.0;
+  }
+}
+
+__global__ void __launch_bounds__(RST_CB * MMAX) k_rst_drive(const double* __restrict__ mats,
+                                                            const double* __restrict__ b, double* __restrict__ fu,
+                                                            int Nt, const int* __restrict__ fstate) {
+  const int f = blockIdx.y;
+  if (fstate[f] != 0) return;
+  __shared__ double sb[RST_CB * RST_ZC];
+  const int nch = rst_chunks(Nt), c0 = blockIdx.x * RST_CB;
+  rst_load_b(sb, b + (int64_t)f * Nt * RST_P, c0, nch, nch * RST_L - Nt);
+  __syncthreads();
+  const int r = threadIdx.x % MMAX, ci = threadIdx.x / MMAX;
+  const double* z = mats + RST_OFF_Z + r;
+  const double* x = sb + ci * RST_ZC;
+  double a0 = 0.0, a1 = 0.0;
+#pragma unroll 8
+  for (int k = 0; k < RST_ZC; k += 2) {
+    a0 = fma(z[k * MMAX], x[k], a0);
+    a1 = fma(z[(k + 1) * MMAX], x[k + 1], a1);
+  }
+  if (c0 + ci < nch) fu[((int64_t)f * nch + c0 + ci) * MMAX + r] = a0 + a1;
+}
+
+// Two threads a row, E^L's entries in registers (2048 issue clocks of the
+// double-precision pipe a chunk, which is what bounds it); the next F's are
+// loaded RST_AHEAD chunks before their use.  F_c is replaced by u_c.
+constexpr int RST_MV = 2 * MMAX;
+constexpr int RST_AHEAD = 4;
+
+__global__ void __launch_bounds__(RST_MV) k_rst_march(const double* __restrict__ mats, double* __restrict__ fu, int Nt,
+                                                     int* fstate, double* resid, unsigned* cnt, double* u_out) {
   const int f = blockIdx.x;
   const int tid = threadIdx.x;
   __shared__ int s_state;
   __shared__ double u[2][MMAX];
   if (tid == 0) s_state = fstate[f];
-  for (int i = tid; i < 2 * MMAX; i += blockDim.x) (&u[0][0])[i] = 0.0;
+  if (tid < MMAX) u[0][tid] = 0.0;
   __syncthreads();
   if (s_state != 0) {
     if (tid == 0 && s_state == 1) fstate[f] = 2;
     return;
   }
-  const int md = (int)mats[RST_OFF_SC + 2];
-  const double h = mats[RST_OFF_SC + 0];
-  const double hm0 = mats[RST_OFF_SC + 1];
+  if (tid == 0) {
+    resid[f] = 0.0;
+    cnt[f] = 0u;
+  }
+  const int nch = rst_chunks(Nt);
+  const int r = tid >> 1, q = tid & 1;
+  double* ff = fu + (int64_t)f * nch * MMAX + r;
+  double Er[32];
+#pragma unroll
+  for (int k = 0; k < 32; ++k) Er[k] = mats[r * MMAX + q + 2 * k];
+  double fn[RST_AHEAD];
+#pragma unroll
+  for (int t = 0; t < RST_AHEAD; ++t) fn[t] = (q == 0 && t < nch) ? ff[t * MMAX] : 0.0;
+  double mine = 0.0;
+  for (int c0 = 0; c0 < nch; c0 += RST_AHEAD) {
+#pragma unroll
+    for (int t = 0; t < RST_AHEAD; ++t) {
+      const int c = c0 + t;
+      if (c < nch) {
+        const double* uc = u[t & 1];
+        double s0 = 0.0, s1 = 0.0;
+#pragma unroll
+        for (int k = 0; k < 32; k += 2) {
+          s0 = fma(Er[k], uc[q + 2 * k], s0);
+          s1 = fma(Er[k + 1], uc[q + 2 * k + 2], s1);
+        }
+        double sum = s0 + s1;
+        sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+        if (q == 0) {
+          sum += fn[t];
+          ff[(int64_t)c * MMAX] = mine;
+          if (c + RST_AHEAD < nch) fn[t] = ff[(int64_t)(c + RST_AHEAD) * MMAX];
+          u[(t & 1) ^ 1][r] = sum;
+          mine = sum;
+        }
+        __syncthreads();
+      }
+    }
+  }
+  static_assert(RST_AHEAD % 2 == 0, "the buffer of u alternates with t");
+  if (q == 0) u_out[(int64_t)f * MMAX + r] = mine;
+}
+
+// One thread a sampled value of a chunk; the warp stops at its latest
+// sample's sources.  The last block of a frequency to finish takes the
+// stopping test from the maximum (of non-negative doubles, whose bits order
+// as integers: the same whatever the blocks' order).
+__global__ void __launch_bounds__(RST_CB * RST_O) k_rst_sample(const double* __restrict__ mats,
+                                                              const double* __restrict__ b,
+                                                              const double* __restrict__ fu, double* __restrict__ smp,
+                                                              int Nt, double tol_abs, int* fstate, double* resid,
+                                                              unsigned* cnt, const double* __restrict__ u_end) {
+  const int f = blockIdx.y;
+  if (fstate[f] != 0) return;
+  __shared__ double sb[RST_CB * RST_ZC], su[RST_CB * MMAX];
+  __shared__ double red[RST_CB * RST_O / 32];
+  const int tid = threadIdx.x;
+  const int nch = rst_chunks(Nt), c0 = blockIdx.x * RST_CB, pad = nch * RST_L - Nt;
   const double* bf = b + (int64_t)f * Nt * RST_P;
   double* sf = smp + (int64_t)f * (Nt + 1) * 3;
-  const bool mv = tid < RST_MV;
-  const int r = tid >> 1, q = tid & 1, lane = tid & 31;
-  const bool samp = !mv && lane < 3;
-  double Er[32], Wr[3];
-  if (mv) {
-#pragma unroll
-    for (int k = 0; k < 32; ++k) {
-      const int c = q + 2 * k;
-      Er[k] = (r < md && c < md) ? mats[r * MMAX + c] : 0.0;
-    }
-#pragma unroll
-    for (int t = 0; t < 3; ++t) Wr[t] = r < md ? mats[RST_OFF_W + (q + 2 * t) * MMAX + r] : 0.0;
+  rst_load_b(sb, bf, c0, nch, pad);
+  for (int o = tid; o < RST_CB * MMAX; o += blockDim.x)
+    su[o] = c0 + o / MMAX < nch ? fu[((int64_t)f * nch + c0) * MMAX + o] : 0.0;
+  __syncthreads();
+  const int o = tid % RST_O, ci = tid / RST_O, r = o / 3, comp = o % 3;
+  const double* t = mats + RST_OFF_R + o;
+  const double* x = su + ci * MMAX;
+  double a0 = 0.0, a1 = 0.0;
+#pragma unroll 8
+  for (int k = 0; k < MMAX; k += 2) {
+    a0 = fma(t[k * RST_O], x[k], a0);
+    a1 = fma(t[(k + 1) * RST_O], x[k + 1], a1);
   }
-  // sampler lane l: value = c0 u[i0] + c1 u[i1] + c2 u[i2] + c3 alpha + c4 (d alpha'),
-  //   l = 0: alphahat = -h u_m
-  //   l = 1: alphahat' = h (H_m u)_m - h [m = 1] alpha
-  //   l = 2: alphahat'' = -h (H_m^2 u)_m + h (H_m)_{m,1} alpha - h [m = 1] alpha'
-  int i0 = 0, i1 = 0, i2 = 0;
-  double c0 = 0.0, c1 = 0.0, c2 = 0.0, c3 = 0.0, c4 = 0.0;
-  if (samp) {
-    const double* R1 = mats + RST_OFF_R1;
-    const double* R2 = mats + RST_OFF_R2;
-    const double del = md == 1 ? 1.0 : 0.0;
-    i2 = md - 1;
-    i1 = md >= 2 ? md - 2 : 0;
-    i0 = md >= 3 ? md - 3 : 0;
-    if (lane == 0) {
-      c2 = -h;
-    } else if (lane == 1) {
-      c0 = md >= 3 ? h * R1[md - 3] : 0.0;
-      c1 = md >= 2 ? h * R1[md - 2] : 0.0;
-      c2 = h * R1[md - 1];
-      c3 = -h * del;
-    } else {
-      c0 = md >= 3 ? -h * R2[md - 3] : 0.0;
-      c1 = md >= 2 ? -h * R2[md - 2] : 0.0;
-      c2 = -h * R2[md - 1];
-      c3 = h * hm0;
-      c4 = -h * del / d;
-    }
+  t += MMAX * RST_O;
+  x = sb + ci * RST_ZC;
+  const int lim = (__reduce_max_sync(0xffffffffu, r) + 1) * RST_P;
+#pragma unroll 6
+  for (int k = 0; k < lim; k += 2) {
+    a0 = fma(t[k * RST_O], x[k], a0);
+    a1 = fma(t[(k + 1) * RST_O], x[k + 1], a1);
   }
-  // this thread's source coefficients of the current interval: b_q, b_{q+2},
-  // b_{q+4} (map threads) or b_0, b_1 (sampler lanes)
-  double bc[3] = {0.0, 0.0, 0.0};
-  if (mv) {
-#pragma unroll
-    for (int t = 0; t < 3; ++t) bc[t] = bf[q + 2 * t];
-  } else if (samp) {
-    bc[0] = bf[0];
-    bc[1] = bf[1];
-  }
+  const int i = (c0 + ci) * RST_L - pad + r;
   double mx = 0.0;
-  int cur = 0;
-  for (int i = 0; i < Nt; ++i) {
-    const bool pre = (i + 1 < Nt);
-    double bn[3] = {0.0, 0.0, 0.0};
-    if (pre) {
-      const double* nx = bf + (int64_t)(i + 1) * RST_P;
-      if (mv) {
-#pragma unroll
-        for (int t = 0; t < 3; ++t) bn[t] = nx[q + 2 * t];
-      } else if (samp) {
-        bn[0] = nx[0];
-        bn[1] = nx[1];
-      }
-    }
-    if (mv) {
-      double s0 = 0.0, s1 = 0.0;
-#pragma unroll
-      for (int k = 0; k < 32; k += 2) {
-        s0 = fma(Er[k], u[cur][q + 2 * k], s0);
-        s1 = fma(Er[k + 1], u[cur][q + 2 * k + 2], s1);
-      }
-      s0 = fma(bc[0], Wr[0], s0);
-      s1 = fma(bc[1], Wr[1], s1);
-      s0 = fma(bc[2], Wr[2], s0);
-      double sum = s0 + s1;
-      sum += __shfl_xor_sync(0xffffffffu, sum, 1);
-      if (q == 0 && r < md) u[cur ^ 1][r] = sum;
-    } else if (samp) {
-      double v = c0 * u[cur][i0];
-      v = fma(c1, u[cur][i1], v);
-      v = fma(c2, u[cur][i2], v);
-      v = fma(c3, bc[0], v);
-      v = fma(c4, bc[1], v);
-      sf[(int64_t)i * 3 + lane] = v;
-      if (lane == 0) mx = fmax(mx, fabs(v));
-    }
-    if (pre) {
-#pragma unroll
-      for (int t = 0; t < 3; ++t) bc[t] = bn[t];
-    }
-    __syncthreads();
-    cur ^= 1;
+  if (c0 + ci < nch && i >= 0) {
+    const double v = a0 + a1;
+    sf[(int64_t)i * 3 + comp] = v;
+    if (comp == 0) mx = fabs(v);
   }
-  // u[cur] = u(T): the last sample (source value and d-scaled slope from the
-  // last interval's polynomial at theta = 1), the maximum, the stopping test
-  if (samp) {
+  if (blockIdx.x == gridDim.x - 1 && tid < 3) {
+    // t = T: source value and d-scaled slope from the last interval's
+    // polynomial at theta = 1 (the rows of r = 0 give C and D)
     const double* last = bf + (int64_t)(Nt - 1) * RST_P;
     double al = 0.0, dal = 0.0;
-#pragma unroll
     for (int j = 0; j < RST_P; ++j) {
       al += last[j];
       dal += j * last[j];
     }
-    double v = c0 * u[cur][i0];
-    v = fma(c1, u[cur][i1], v);
-    v = fma(c2, u[cur][i2], v);
-    v = fma(c3, al, v);
-    v = fma(c4, dal, v);
-    sf[(int64_t)Nt * 3 + lane] = v;
-    if (lane == 0) {
-      mx = fmax(mx, fabs(v));
-      resid[f] = mx;
-      if (!isfinite(mx)) fstate[f] = 3;            // reported by the host
-      else if (mx <= tol_abs) fstate[f] = 1;       // stops after this restart's combination
-    }
+    const double* tc = mats + RST_OFF_R + tid;
+    double v = 0.0;
+    for (int k = 0; k < MMAX; ++k) v = fma(tc[k * RST_O], u_end[(int64_t)f * MMAX + k], v);
+    v = fma(tc[MMAX * RST_O], al, v);
+    v = fma(tc[(MMAX + 1) * RST_O], dal, v);
+    sf[(int64_t)Nt * 3 + tid] = v;
+    if (tid == 0) mx = fabs(v) > mx || !(v == v) ? fabs(v) : mx;
   }
-  for (int i = tid; i < MMAX; i += blockDim.x) u_out[(int64_t)f * MMAX + i] = i < md ? u[cur][i] : 0.0;
+  // the largest bits (a NaN's order above every number's)
+  unsigned long long m = (unsigned long long)__double_as_longlong(mx);
+  for (int s = 16; s > 0; s >>= 1) {
+    const unsigned long long y = __shfl_xor_sync(0xffffffffu, m, s);
+    m = y > m ? y : m;
+  }
+  if ((tid & 31) == 0) red[tid >> 5] = __longlong_as_double((long long)m);
+  __syncthreads();
+  if (tid != 0) return;
+  for (int wq = 0; wq < RST_CB * RST_O / 32; ++wq) {
+    const unsigned long long y = (unsigned long long)__double_as_longlong(red[wq]);
+    m = y > m ? y : m;
+  }
+  unsigned long long* rb = reinterpret_cast<unsigned long long*>(resid) + f;
+  atomicMax(rb, m);
+  __threadfence();
+  if (atomicAdd(cnt + f, 1u) != gridDim.x - 1) return;
+  __threadfence();
+  const double all = __longlong_as_double((long long)atomicMax(rb, 0ull));
+  if (!isfinite(all)) fstate[f] = 3;            // reported by the host
+  else if (all <= tol_abs) fstate[f] = 1;       // stops after this restart's combination
 }
 
 kx_status launch_rst_cascade(kx_ctx* c, cudaStream_t st, int nfreq, const double* b, int Nt, double d,
                              double tol_abs) {
+  (void)d;
+  const int nch = (Nt + RST_L - 1) / RST_L;
+  const dim3 grid((nch + RST_CB - 1) / RST_CB, nfreq);
   time_begin(c);
-  k_rst_cascade<<<nfreq, RST_THREADS, 0, st>>>(c->d_rst_mats, b, c->d_rst_smp, Nt, d, tol_abs, c->d_rst_state,
-                                               c->d_rst_res, c->d_rst_u);
+  k_rst_drive<<<grid, RST_CB * MMAX, 0, st>>>(c->d_rst_mats, b, c->d_rst_fu, Nt, c->d_rst_state);
+  KX_CHECK_LAUNCH(c);
+  k_rst_march<<<nfreq, RST_MV, 0, st>>>(c->d_rst_mats, c->d_rst_fu, Nt, c->d_rst_state, c->d_rst_res, c->d_rst_cnt,
+                                       c->d_rst_u);
+  KX_CHECK_LAUNCH(c);
+  k_rst_sample<<<grid, RST_CB * RST_O, 0, st>>>(c->d_rst_mats, b, c->d_rst_fu, c->d_rst_smp, Nt, tol_abs,
+                                               c->d_rst_state, c->d_rst_res, c->d_rst_cnt, c->d_rst_u);
   time_end(c, KX_K_CASCADE, 0.0);
   KX_CHECK_LAUNCH(c);
   return KX_OK;
