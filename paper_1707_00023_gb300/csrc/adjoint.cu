@@ -19,9 +19,10 @@
 #include <cmath>
 #include <vector>
 
-#include "kx_dense.cuh"
 #include <atomic>
 
+#include "kx_cdense.cuh"
+#include "kx_eft.cuh"
 #include "kx_internal.cuh"
 
 namespace kx {
@@ -59,220 +60,239 @@ __global__ void k_adj_seed(Geo g, int axis, int idx, const T* __restrict__ y, T*
   }
 }
 
-// y = M x for an m x m row-major matrix, four threads per row.
-__device__ void cta_mv(const double* __restrict__ M, const double* x, double* y, int m) {
-  const int r = threadIdx.x >> 2, part = threadIdx.x & 3;
-  double s = 0.0;
-  if (r < m)
-    for (int c = part; c < m; c += 4) s = fma(M[r * m + c], x[c], s);
-  s += __shfl_xor_sync(0xffffffffu, s, 1);
-  s += __shfl_xor_sync(0xffffffffu, s, 2);
-  __syncthreads();
-  if (r < m && part == 0) y[r] = s;
-  __syncthreads();
+// exp(-delta H_m) of the forward basis (cluster 0, slot 0) and the adjoint
+// basis (cluster 1, slot 1), rows with stride CD_LD in the cluster's global
+// matrix ADJ_E (kx_cdense.cuh).
+constexpr int ADJ_E = 2 * CD_MAT;
+
+__global__ void __launch_bounds__(CD_THREADS) k_adj_expm(SlotSet<float> ss, int ldh, double delta, double* ws,
+                                                         int* status) {
+  extern __shared__ __align__(16) double sm[];
+  __shared__ double red[32];
+  const int which = blockIdx.x / CD_CTAS, rank = cl_rank();
+  const Slot<float> sl = slot_at(ss, which);
+  const double* H = sl.H;
+  const int m = sl.st->m_done;
+  if (m <= 0 || sl.st->beta == 0.0) return;   // zero state: no coefficients are formed
+  auto entry = [&](int r, int c) { return r <= c + 1 ? H[r + (int64_t)c * ldh] : 0.0; };
+  int q = 0, s = 0;
+  if (!cd_plan(delta * cd_norm1(m, red, entry), 1, &q, &s)) {
+    if (rank == 0 && threadIdx.x == 0) *status = KX_ENONFINITE;
+    return;
+  }
+  const CdRows w = cd_rows(m, rank);
+  const double sc = -ldexp(delta, -s);
+  double* g = ws + (size_t)which * CD_WS;
+  const double* E = cd_expm(cd_shared(sm), g, m, w, q, s, [&](int r, int c) { return sc * entry(r, c); });
+  for (int o = threadIdx.x; o < w.R * m; o += CD_THREADS) {
+    const int r = o / m, c = o - r * m;
+    g[ADJ_E + (w.r0 + r) * CD_LD + c] = E[r * CD_LD + c];
+  }
 }
 
-// Projected quadrature coefficients of one sub-step.  Block 0 works on the
-// forward basis (slot 0), block 1 on the adjoint basis (slot 1).
+// M x with M's entries in registers, four threads a row (columns part + 4 k);
+// the sum in every lane of the row's four.
+__device__ __forceinline__ double adj_row(const double* Mr, const double* x, int part) {
+  double a = 0.0, b = 0.0;
+#pragma unroll
+  for (int k = 0; k < 16; k += 2) {
+    a = fma(Mr[k], x[part + 4 * k], a);
+    b = fma(Mr[k + 1], x[part + 4 * k + 4], b);
+  }
+  a += b;
+  a += __shfl_xor_sync(0xffffffffu, a, 1);
+  a += __shfl_xor_sync(0xffffffffu, a, 2);
+  return a;
+}
+
+// Projected quadrature coefficients of one sub-step, one block for each
+// Gauss node j (blockIdx.x) and basis (blockIdx.y: 0 forward, slot 0; 1
+// adjoint, slot 1).
 //   nodes s_q = (i + x_j) delta, q = i * P + j, delta = tau / nsub
 //   alpha[q][r] = scale_V[r] (H_V u(s_q))_r,  r <= m_V   (A y at s_q)
+//   alpha[q][MMAX + 1] = sin(W (t_k + s_q))              (the source's factor)
 //   omg[q][r]   = scale_W[r] w(tau - s_q)_r,  r < m_W    (lambda at s_q)
-//   cw[q] = delta * wg[j],  sn[q] = sin(W (t_k + s_q))
-//   slot 1's u = w(tau)   (lambda at t_k, for the next sub-step)
-__global__ void __launch_bounds__(256) k_adj_coeffs(SlotSet<float> ss, int ldh, double tau, int nsub,
-                                                    const double* __restrict__ xg,
-                                                    const double* __restrict__ wg, double omega,
-                                                    double tk, double* __restrict__ Eg,
-                                                    float* __restrict__ alpha, float* __restrict__ omg,
-                                                    float* __restrict__ cw, float* __restrict__ sn,
-                                                    int* status) {
-  extern __shared__ double sm[];
-  __shared__ double red[32];
-  __shared__ double lv[72];
-  __shared__ int piv;
-  __shared__ double z[2][72], acc[72];
-  const int which = blockIdx.x;
+//   cw[q] = delta * wg[j]
+//   block (P, 1): slot 1's u = w(tau)   (lambda at t_k, for the next sub-step)
+// The start exp(-x_j delta H) beta e_1 by its Taylor series, then nsub
+// products with E = exp(-delta H).  Marching the eight nodes one after the
+// other on one block, with the exponential before them, took 2.0 ms at m =
+// 64, tau = 12; each product is bound by the double-precision pipe (1.2 us).
+constexpr int ADJ_A = MMAX + 2;   // stored alpha rows a node
+
+__global__ void __launch_bounds__(256) k_adj_march(SlotSet<float> ss, int ldh, double tau, int nsub,
+                                                   const double* __restrict__ xg, const double* __restrict__ wg,
+                                                   double omega, double tk, const double* __restrict__ ws,
+                                                   double* __restrict__ alpha, double* __restrict__ omg,
+                                                   double* __restrict__ cw) {
+  const int which = blockIdx.y, j = blockIdx.x, tid = threadIdx.x;
+  const bool end = j == GAUSS_P;
+  if (end && which == 0) return;
+  __shared__ double z[2][MMAX], scl[MMAX + 1], red[32];
   const Slot<float> sl = slot_at(ss, which);
   const double* H = sl.H;
   const int m = sl.st->m_done;
   const double beta = sl.st->beta;
   const double delta = tau / nsub;
-  double* E = Eg + (size_t)which * MMAX * MMAX;
-  if (m <= 0 || beta == 0.0) {
+  const bool zero = m <= 0 || beta == 0.0;
+  if (!end && which == 0)
+    for (int i = tid; i < nsub; i += blockDim.x) {
+      cw[i * GAUSS_P + j] = delta * wg[j];
+      alpha[(size_t)(i * GAUSS_P + j) * ADJ_A + MMAX + 1] = sin(omega * (tk + (i + xg[j]) * delta));
+    }
+  if (zero) {
     // zero state: every coefficient vanishes
-    for (int q = threadIdx.x; q < nsub * GAUSS_P; q += blockDim.x) {
-      for (int r = 0; r <= MMAX; ++r) {
-        if (which == 0) alpha[(size_t)q * (MMAX + 1) + r] = 0.f;
-        else if (r < MMAX) omg[(size_t)q * MMAX + r] = 0.f;
-      }
-      if (which == 0) {
-        const int i = q / GAUSS_P, j = q % GAUSS_P;
-        cw[q] = (float)(delta * wg[j]);
-        sn[q] = (float)sin(omega * (tk + (i + xg[j]) * delta));
-      }
+    if (end) {
+      if (tid < ldh - 1) sl.u[tid] = 0.0;
+      return;
     }
-    if (which == 1 && threadIdx.x < ldh - 1) sl.u[threadIdx.x] = 0.0;
-    return;
-  }
-  // E = exp(-delta H_m)
-  double* buf[6];
-  for (int q = 0; q < 6; ++q) buf[q] = sm + (size_t)q * m * m;
-  for (int idx = threadIdx.x; idx < m * m; idx += blockDim.x) {
-    const int r = idx / m, c = idx - r * m;
-    buf[0][idx] = (r <= c + 1) ? -delta * H[r + (int64_t)c * ldh] : 0.0;
-  }
-  __syncthreads();
-  double* X = cta_expm(buf, m, red, lv, &piv);
-  if (!X) {
-    if (threadIdx.x == 0) *status = KX_ENONFINITE;
-    return;
-  }
-  for (int idx = threadIdx.x; idx < m * m; idx += blockDim.x) E[idx] = X[idx];
-  // H_m row-major in shared memory for the Taylor steps (buf[1] is free now)
-  double* Hs = buf[0] == X ? buf[1] : buf[0];
-  for (int idx = threadIdx.x; idx < m * m; idx += blockDim.x) {
-    const int r = idx / m, c = idx - r * m;
-    Hs[idx] = (r <= c + 1) ? H[r + (int64_t)c * ldh] : 0.0;
-  }
-  __syncthreads();
-  const double hnext = H[m + (int64_t)(m - 1) * ldh];
-  for (int j = 0; j < GAUSS_P; ++j) {
-    // z = exp(-x_j delta H) beta e_1 by its Taylor series (|x_j delta H| small)
-    const double h = -xg[j] * delta;
-    for (int r = threadIdx.x; r < m; r += blockDim.x) {
-      z[0][r] = r == 0 ? beta : 0.0;
-      acc[r] = z[0][r];
-    }
-    __syncthreads();
-    int cur = 0;
-    for (int kk = 1; kk <= 60; ++kk) {
-      cta_mv(Hs, z[cur], z[cur ^ 1], m);
-      cur ^= 1;
-      double nrm = 0.0, tot = 0.0;
-      for (int r = threadIdx.x; r < m; r += blockDim.x) {
-        z[cur][r] *= h / kk;
-        acc[r] += z[cur][r];
-      }
-      __syncthreads();
-      if (threadIdx.x < 32) {
-        for (int r = threadIdx.x; r < m; r += 32) {
-          nrm = fmax(nrm, fabs(z[cur][r]));
-          tot = fmax(tot, fabs(acc[r]));
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-          nrm = fmax(nrm, __shfl_xor_sync(0xffffffffu, nrm, o));
-          tot = fmax(tot, __shfl_xor_sync(0xffffffffu, tot, o));
-        }
-        if (threadIdx.x == 0) red[0] = (nrm <= 1e-18 * tot) ? 1.0 : 0.0;
-      }
-      __syncthreads();
-      if (red[0] != 0.0) break;
-      __syncthreads();
-    }
-    // march the sub-intervals: value at (i + x_j) delta is E^i z
-    for (int r = threadIdx.x; r < m; r += blockDim.x) z[0][r] = acc[r];
-    __syncthreads();
-    cur = 0;
     for (int i = 0; i < nsub; ++i) {
-      if (i > 0) {
-        cta_mv(E, z[cur], z[cur ^ 1], m);
-        cur ^= 1;
-      }
+      const size_t q = (size_t)i * GAUSS_P + j;
+      if (which == 0 && tid <= MMAX) alpha[q * ADJ_A + tid] = 0.0;
+      if (which == 1 && tid < MMAX) omg[q * MMAX + tid] = 0.0;
+    }
+    return;
+  }
+  const int r = tid >> 2, part = tid & 3;
+  const double* E = ws + (size_t)which * CD_WS + ADJ_E;
+  double Er[16], Hr[16];
+#pragma unroll
+  for (int k = 0; k < 16; ++k) {
+    const int c = part + 4 * k;
+    Er[k] = r < m && c < m ? E[r * CD_LD + c] : 0.0;
+    Hr[k] = r < m && c < m && r <= c + 1 ? H[r + (int64_t)c * ldh] : 0.0;
+  }
+  if (tid < MMAX) z[0][tid] = tid == 0 ? beta : 0.0;
+  if (tid <= m) scl[tid] = sl.scale[tid];
+  double hn = 0.0;   // ||H||_inf bounds the Taylor terms
+  {
+    double a = 0.0;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) a += fabs(Hr[k]);
+    a += __shfl_xor_sync(0xffffffffu, a, 1);
+    a += __shfl_xor_sync(0xffffffffu, a, 2);
+    for (int o = 16; o > 2; o >>= 1) a = fmax(a, __shfl_xor_sync(0xffffffffu, a, o));
+    if ((tid & 31) == 0) red[tid >> 5] = a;
+    __syncthreads();
+    for (int q = 0; q < 8; ++q) hn = fmax(hn, red[q]);
+  }
+  int cur = 0;
+  if (!end) {
+    const double h = -xg[j] * delta;
+    int terms = 0;
+    for (double t = 1.0; t > 1e-18 && terms < 60; t *= fabs(h) * hn / terms) ++terms;
+    double acc = r == 0 ? beta : 0.0;
+    for (int kk = 1; kk <= terms; ++kk) {
+      const double v = adj_row(Hr, z[cur], part) * (h / kk);
+      acc += v;
+      if (part == 0) z[cur ^ 1][r] = v;
+      __syncthreads();
+      cur ^= 1;
+    }
+    if (part == 0) z[cur ^ 1][r] = acc;   // rows past m stay zero
+    __syncthreads();
+    cur ^= 1;
+  }
+  const double hnext = H[m + (int64_t)(m - 1) * ldh];
+  // value at (i + x_j) delta is E^i z
+  for (int i = 0; i < nsub; ++i) {
+    if (!end) {
       const double* u = z[cur];
       if (which == 0) {
-        const int q = i * GAUSS_P + j;
         // alpha = scale .* (Hbar u), Hbar the (m+1) x m Hessenberg matrix
-        for (int r = threadIdx.x; r <= m; r += blockDim.x) {
-          double s = 0.0;
-          if (r < m) {
-            for (int c = max(r - 1, 0); c < m; ++c) s = fma(Hs[r * m + c], u[c], s);
-          } else {
-            s = hnext * u[m - 1];
-          }
-          alpha[(size_t)q * (MMAX + 1) + r] = (float)(sl.scale[r] * s);
-        }
-        for (int r = m + 1 + threadIdx.x; r <= MMAX; r += blockDim.x) alpha[(size_t)q * (MMAX + 1) + r] = 0.f;
-        if (threadIdx.x == 0) {
-          cw[q] = (float)(delta * wg[j]);
-          sn[q] = (float)sin(omega * (tk + (i + xg[j]) * delta));
-        }
-      } else {
+        double* al = alpha + (size_t)(i * GAUSS_P + j) * ADJ_A;
+        const double v = adj_row(Hr, u, part);
+        if (part == 0) al[r] = r < m ? scl[r] * v : (r == m ? scl[m] * hnext * u[m - 1] : 0.0);
+        if (tid == 0) al[MMAX] = m == MMAX ? scl[m] * hnext * u[m - 1] : 0.0;
+      } else if (tid < MMAX) {
         // lambda at t_k + s_q needs w(tau - s_q): tau - s_q = (nsub-1-i + x_{P-1-j}) delta
-        const int q = (nsub - 1 - i) * GAUSS_P + (GAUSS_P - 1 - j);
-        for (int r = threadIdx.x; r < MMAX; r += blockDim.x)
-          omg[(size_t)q * MMAX + r] = r < m ? (float)(sl.scale[r] * u[r]) : 0.f;
+        omg[(size_t)((nsub - 1 - i) * GAUSS_P + (GAUSS_P - 1 - j)) * MMAX + tid] = tid < m ? scl[tid] * u[tid] : 0.0;
       }
-      __syncthreads();
+      if (i == nsub - 1) break;
     }
-  }
-  if (which == 1) {
-    // w(tau) = E^nsub beta e_1 for the update lambda(t_k) = W w(tau)
-    for (int r = threadIdx.x; r < m; r += blockDim.x) z[0][r] = r == 0 ? beta : 0.0;
+    const double v = adj_row(Er, z[cur], part);
+    if (part == 0) z[cur ^ 1][r] = v;
     __syncthreads();
-    int cur = 0;
-    for (int i = 0; i < nsub; ++i) {
-      cta_mv(E, z[cur], z[cur ^ 1], m);
-      cur ^= 1;
-    }
-    for (int r = threadIdx.x; r < m; r += blockDim.x) sl.u[r] = z[cur][r];
+    cur ^= 1;
+  }
+  // w(tau) = E^nsub beta e_1 for the update lambda(t_k) = W w(tau)
+  if (end && tid < m) sl.u[tid] = z[cur][tid];
+}
+
+// The quadrature over the sub-step's nodes, done once on the coefficients:
+//   M_{i,k} = sum_q cw_q alpha_{q,i} omg_{q,k}
+// (row MMAX + 1: the source's factor), as float pairs hi + lo.  One block a row.
+__global__ void __launch_bounds__(256) k_adj_moments(const double* __restrict__ alpha, const double* __restrict__ omg,
+                                                     const double* __restrict__ cw, int nq, float* __restrict__ M) {
+  extern __shared__ __align__(16) double wq[];   // nq
+  __shared__ double part[4][MMAX];
+  const int i = blockIdx.x, tid = threadIdx.x, k = tid & (MMAX - 1), g = tid / MMAX;
+  for (int q = tid; q < nq; q += blockDim.x) wq[q] = cw[q] * alpha[(size_t)q * ADJ_A + i];
+  __syncthreads();
+  double a = 0.0;
+  for (int q = g; q < nq; q += 4) a = fma(wq[q], omg[(size_t)q * MMAX + k], a);
+  part[g][k] = a;
+  __syncthreads();
+  if (g == 0) {
+    a = (part[0][k] + part[1][k]) + (part[2][k] + part[3][k]);
+    const float hi = (float)a;
+    M[i * MMAX + k] = hi;
+    M[(ADJ_A + i) * MMAX + k] = (float)(a - (double)hi);
   }
 }
 
-// Q_e += sum_q cw_q (sum_i alpha_q,i V_i,e + sn_q g_e) (sum_i omg_q,i W_i,e) / eps_e
-// over the E nodes e, in chunks of 32 quadrature nodes staged in shared memory.
+// Q_e += (sum_{i,k} V_{i,e} M_{i,k} W_{k,e} + g_e sum_k M_{MMAX+1,k} W_{k,e}) / eps_e
+// over the E nodes e: the quadrature of (A y)_e lambda_e on the sub-step.  One
+// thread a node, W's column of the node in registers, M in shared memory.
+// With M formed first a node costs 66 x 64 products whatever the number of
+// quadrature nodes; evaluating both factors at every node took 129 FMAs a
+// node and quadrature point (240 of them at tau = 12: 667 us at 48^3).  The
+// entries of M cancel where the factors at a node did not, so the sums carry
+// their rounding errors (hi + lo, kx_eft.cuh) and M is a float pair: five
+// packed operations for two products.
 template <typename T>
-__global__ void __launch_bounds__(NTHREADS) k_adj_accum(Geo g, const T* __restrict__ V, const T* __restrict__ W,
-                                                       int64_t ld, int mV, int mW, const T* __restrict__ gsrc,
-                                                       const T* __restrict__ ie, int nq,
-                                                       const float* __restrict__ alpha,
-                                                       const float* __restrict__ omg,
-                                                       const float* __restrict__ cw,
-                                                       const float* __restrict__ sn, double* __restrict__ Q) {
-  constexpr int CH = 32;
-  __shared__ float sa[CH][MMAX + 1];
-  __shared__ float so[CH][MMAX];
-  __shared__ float scw[CH], ssn[CH];
+__global__ void __launch_bounds__(128) k_adj_accum(Geo g, const T* __restrict__ V, const T* __restrict__ W,
+                                                  int64_t ld, int mV, int mW, const T* __restrict__ gsrc,
+                                                  const T* __restrict__ ie, const float* __restrict__ M,
+                                                  double* __restrict__ Q) {
+  __shared__ __align__(16) float sM[2 * ADJ_A * MMAX];
+  for (int o = threadIdx.x; o < 2 * ADJ_A * MMAX; o += blockDim.x) sM[o] = M[o];
+  __syncthreads();
   const int64_t nE = (int64_t)g.ne * g.ncell;
   const int64_t off = (int64_t)g.nh * g.ncell;
-  const int64_t rounds = (nE + blockDim.x - 1) / blockDim.x;
-  for (int64_t r0 = blockIdx.x; r0 < rounds; r0 += gridDim.x) {
-    const int64_t e = r0 * blockDim.x + threadIdx.x;
-    const bool act = e < nE;
-    double qacc = 0.0;
-    const T ge = act ? gsrc[off + e] : T(0);
-    for (int q0 = 0; q0 < nq; q0 += CH) {
-      const int nc = min(CH, nq - q0);
-      __syncthreads();
-      for (int t = threadIdx.x; t < nc * (MMAX + 1); t += blockDim.x)
-        sa[t / (MMAX + 1)][t % (MMAX + 1)] = alpha[(size_t)(q0 + t / (MMAX + 1)) * (MMAX + 1) + t % (MMAX + 1)];
-      for (int t = threadIdx.x; t < nc * MMAX; t += blockDim.x)
-        so[t / MMAX][t % MMAX] = omg[(size_t)(q0 + t / MMAX) * MMAX + t % MMAX];
-      for (int t = threadIdx.x; t < nc; t += blockDim.x) {
-        scw[t] = cw[q0 + t];
-        ssn[t] = sn[q0 + t];
-      }
-      __syncthreads();
-      if (!act) continue;
-      float a[CH], b[CH];
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nE; e += (int64_t)gridDim.x * blockDim.x) {
+    float2 w[MMAX / 2];
 #pragma unroll
-      for (int t = 0; t < CH; ++t) { a[t] = 0.f; b[t] = 0.f; }
-      for (int i = 0; i <= mV; ++i) {
-        const float v = (float)V[(int64_t)i * ld + off + e];
-#pragma unroll
-        for (int t = 0; t < CH; ++t) a[t] = fmaf(sa[t][i], v, a[t]);
-      }
-      for (int i = 0; i < mW; ++i) {
-        const float w = (float)W[(int64_t)i * ld + off + e];
-#pragma unroll
-        for (int t = 0; t < CH; ++t) b[t] = fmaf(so[t][i], w, b[t]);
-      }
-      float part = 0.f;
-#pragma unroll
-      for (int t = 0; t < CH; ++t)
-        if (t < nc) part = fmaf(scw[t] * fmaf(ssn[t], (float)ge, a[t]), b[t], part);
-      qacc += (double)part;
+    for (int k = 0; k < MMAX / 2; ++k) {
+      w[k].x = 2 * k < mW ? (float)W[(int64_t)(2 * k) * ld + off + e] : 0.f;
+      w[k].y = 2 * k + 1 < mW ? (float)W[(int64_t)(2 * k + 1) * ld + off + e] : 0.f;
     }
-    if (act) Q[e] += qacc * (double)ie[e];
+    float qh = 0.f, ql = 0.f;
+#pragma unroll 1
+    for (int i = 0; i <= mV + 1; ++i) {
+      const int row = i <= mV ? i : MMAX + 1;
+      const float v = i <= mV ? (float)V[(int64_t)i * ld + off + e] : (float)gsrc[off + e];
+      const float4* mh = reinterpret_cast<const float4*>(sM + row * MMAX);
+      const float4* ml = reinterpret_cast<const float4*>(sM + (ADJ_A + row) * MMAX);
+      float2 h0 = make_float2(0.f, 0.f), h1 = h0, l0 = h0, l1 = h0;
+#pragma unroll
+      for (int k = 0; k < MMAX / 4; ++k) {
+        const float4 x = mh[k], y = ml[k];
+        l0 = __ffma2_rn(make_float2(y.x, y.y), w[2 * k], l0);
+        l1 = __ffma2_rn(make_float2(y.z, y.w), w[2 * k + 1], l1);
+        sub_fma2(h0, l0, make_float2(x.x, x.y), w[2 * k]);
+        sub_fma2(h1, l1, make_float2(x.z, x.w), w[2 * k + 1]);
+      }
+      // t = h + l: the four partial sums added with their errors
+      float th = 0.f, tl = (l0.x + l0.y) + (l1.x + l1.y);
+      sub_fma(th, tl, 1.f, h0.x);
+      add_two(th, tl, h0.y);
+      add_two(th, tl, h1.x);
+      add_two(th, tl, h1.y);
+      ql = fmaf(v, tl, ql);
+      sub_fma(qh, ql, v, th);
+    }
+    Q[e] += ((double)qh + (double)ql) * (double)ie[e];
   }
 }
 
@@ -321,30 +341,36 @@ kx_status launch_adj_substep(kx_ctx* c, double tau, double omega, double tk, con
   }
   const int m = c->m;
   static SmemOptIn attr{};
-  const kx_status so = smem_opt_in(c, attr, (const void*)k_adj_coeffs, expm_smem_bytes(MMAX + 2));
+  const kx_status so = smem_opt_in(c, attr, (const void*)k_adj_expm, CD_SMEM);
   if (so != KX_OK) return so;
   int* status = reinterpret_cast<int*>(c->d_small + 64);
+  const SlotSet<float> ss = make_slotset<float>(c, 0);
+  const int nq = nsub * GAUSS_P;
   time_begin(c);
-  k_adj_coeffs<<<2, 256, expm_smem_bytes(m), c->stream>>>(
-      make_slotset<float>(c, 0), m + 1, tau, nsub, c->d_gauss, c->d_gauss + GAUSS_P, omega, tk,
-      c->d_expm_ws, c->d_adj_alpha, c->d_adj_omg, c->d_adj_cw, c->d_adj_sn, status);
+  launch_cluster(k_adj_expm, 2, CD_SMEM, c->stream, ss, m + 1, tau / nsub, c->d_cd_ws, status);
+  KX_CHECK_LAUNCH(c);
+  k_adj_march<<<dim3(GAUSS_P + 1, 2), 256, 0, c->stream>>>(ss, m + 1, tau, nsub, c->d_gauss, c->d_gauss + GAUSS_P,
+                                                           omega, tk, c->d_cd_ws, c->d_adj_alpha, c->d_adj_omg,
+                                                           c->d_adj_cw);
+  KX_CHECK_LAUNCH(c);
+  k_adj_moments<<<ADJ_A, 256, nq * sizeof(double), c->stream>>>(c->d_adj_alpha, c->d_adj_omg, c->d_adj_cw, nq,
+                                                               c->d_adj_M);
   time_end(c, KX_K_PROJ, 0.0);
   KX_CHECK_LAUNCH(c);
-  const int nq = nsub * GAUSS_P;
   const int64_t nE = (int64_t)c->geo.ne * c->geo.ncell;
-  const int blocks = (int)std::min<int64_t>((nE + NTHREADS - 1) / NTHREADS, (int64_t)c->nsm * 4);
+  const int blocks = (int)std::min<int64_t>((nE + 127) / 128, (int64_t)c->nsm * 8);
   const int64_t sV = (int64_t)(m + 1) * c->ld;
   // the basis sizes are read back by the host after each Arnoldi run
   const int mV = c->h_state[0].m_done, mW = c->h_state[1].m_done;
   time_begin(c);
   if (c->d.precision == KX_FP64) {
-    k_adj_accum<double><<<blocks, NTHREADS, 0, c->stream>>>(
+    k_adj_accum<double><<<blocks, 128, 0, c->stream>>>(
         c->geo, (const double*)c->d_V, (const double*)c->d_V + sV, c->ld, mV, mW, (const double*)g,
-        (const double*)c->d_inv_eps, nq, c->d_adj_alpha, c->d_adj_omg, c->d_adj_cw, c->d_adj_sn, c->d_adj_Q);
+        (const double*)c->d_inv_eps, c->d_adj_M, c->d_adj_Q);
   } else {
-    k_adj_accum<float><<<blocks, NTHREADS, 0, c->stream>>>(
+    k_adj_accum<float><<<blocks, 128, 0, c->stream>>>(
         c->geo, (const float*)c->d_V, (const float*)c->d_V + sV, c->ld, mV, mW, (const float*)g,
-        (const float*)c->d_inv_eps, nq, c->d_adj_alpha, c->d_adj_omg, c->d_adj_cw, c->d_adj_sn, c->d_adj_Q);
+        (const float*)c->d_inv_eps, c->d_adj_M, c->d_adj_Q);
   }
   time_end(c, KX_K_ZUPDATE, (double)(mV + 1 + mW) * nE * c->esize);
   KX_CHECK_LAUNCH(c);

@@ -524,7 +524,7 @@ kx_status create_impl(const kx_desc* desc, const double* eps_cell, const uint8_t
       {(void**)&c->d_small, (size_t)256 * sizeof(double)},
       {(void**)&c->d_tmp, (size_t)c->n * c->esize},
       {(void**)&c->d_tmp2, (size_t)c->n * c->esize},
-      {(void**)&c->d_expm_ws, (size_t)(MMAX + 1) * MMAX * MAXF * sizeof(double)},
+      {(void**)&c->d_expm_ws, (size_t)((MMAX + 1) * MMAX + MMAX * MAXF) * sizeof(double)},
       {(void**)&c->d_cd_ws, (size_t)std::max(2, B) * CD_WS * sizeof(double)},
       {(void**)&c->d_zre, (size_t)d.max_freqs * c->n * c->esize},
       {(void**)&c->d_zim, (size_t)d.max_freqs * c->n * c->esize},
@@ -548,10 +548,10 @@ kx_status create_impl(const kx_desc* desc, const double* eps_cell, const uint8_t
     Alloc adj[] = {
         {(void**)&c->d_ckpt, (size_t)d.max_checkpoints * c->ld * c->esize},
         {(void**)&c->d_adj_Q, (size_t)nE * sizeof(double)},
-        {(void**)&c->d_adj_alpha, (size_t)c->adj_nq_max * (MMAX + 1) * sizeof(float)},
-        {(void**)&c->d_adj_omg, (size_t)c->adj_nq_max * MMAX * sizeof(float)},
-        {(void**)&c->d_adj_cw, (size_t)c->adj_nq_max * sizeof(float)},
-        {(void**)&c->d_adj_sn, (size_t)c->adj_nq_max * sizeof(float)},
+        {(void**)&c->d_adj_alpha, (size_t)c->adj_nq_max * (MMAX + 2) * sizeof(double)},
+        {(void**)&c->d_adj_omg, (size_t)c->adj_nq_max * MMAX * sizeof(double)},
+        {(void**)&c->d_adj_cw, (size_t)c->adj_nq_max * sizeof(double)},
+        {(void**)&c->d_adj_M, (size_t)2 * (MMAX + 2) * MMAX * sizeof(float)},
         {(void**)&c->d_gauss, (size_t)2 * P * sizeof(double)},
     };
     for (auto& a : adj) {
@@ -681,7 +681,7 @@ kx_status krylov_expm_destroy(kx_ctx* c) {
   void* ptrs[] = {c->d_inv_eps, c->d_sig2, c->d_eps_cell, c->d_V, c->d_aug, c->d_H, c->d_scale,
                   c->d_part, c->d_counter, c->d_u, c->d_state, c->d_rho, c->d_coef, c->d_coefd,
                   c->d_omegas, c->d_small, c->d_tmp, c->d_tmp2, c->d_expm_ws, c->d_cd_ws, c->d_zre, c->d_zim,
-                  c->d_ckpt, c->d_adj_Q, c->d_adj_alpha, c->d_adj_omg, c->d_adj_cw, c->d_adj_sn,
+                  c->d_ckpt, c->d_adj_Q, c->d_adj_alpha, c->d_adj_omg, c->d_adj_cw, c->d_adj_M,
                   c->d_gauss, c->d_rst_b, c->d_rst_smp, c->d_rst_mats, c->d_rst_fu, c->d_rst_cnt, c->d_rst_u, c->d_rst_res,
                   c->d_rst_state, c->d_rst_yp, c->d_swT, c->d_swpart, c->d_swG, c->d_swco};
   for (void* p : ptrs)

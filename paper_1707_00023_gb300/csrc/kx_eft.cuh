@@ -25,7 +25,15 @@ __device__ __forceinline__ void sub_fma(float& hi, float& lo, float nc, float v)
   hi = s;
 }
 
-// The same on two lanes at a time in packed FP32x2 operations (a - b as
+// hi + lo <- hi + lo + x (Knuth's TwoSum)
+__device__ __forceinline__ void add_two(float& hi, float& lo, float x) {
+  const float s = hi + x;
+  const float z = s - hi;
+  lo += (hi - (s - z)) + (x - z);
+  hi = s;
+}
+
+// sub_fma on two lanes at a time in packed FP32x2 operations (a - b as
 // fma(b, -1, a), exact before its one rounding).
 __device__ __forceinline__ void sub_fma2(float2& hi, float2& lo, float2 nc, float2 v) {
   const float2 m1 = make_float2(-1.f, -1.f);

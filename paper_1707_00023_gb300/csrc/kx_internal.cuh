@@ -218,15 +218,15 @@ struct kx_ctx {
   double* h_small;          // pinned
   void* d_tmp;              // one extra vector
   void* d_tmp2;             // one extra vector
-  double* d_expm_ws;        // projected exponential workspace
+  double* d_expm_ws;        // expm_phi_project's matrix and results
   double* d_cd_ws;          // cluster-wide dense work (kx_cdense.cuh), one piece a slot, two at least
   // adjoint workspace (max_checkpoints > 0)
   void* d_ckpt = nullptr;   // max_checkpoints states of the forward solution
   double* d_adj_Q = nullptr;      // per-E-node time integrals
-  float* d_adj_alpha = nullptr;   // quadrature coefficients
-  float* d_adj_omg = nullptr;
-  float* d_adj_cw = nullptr;
-  float* d_adj_sn = nullptr;
+  double* d_adj_alpha = nullptr;  // quadrature coefficients (adjoint.cu)
+  double* d_adj_omg = nullptr;
+  double* d_adj_cw = nullptr;
+  float* d_adj_M = nullptr;
   double* d_gauss = nullptr;      // Gauss-Legendre nodes and weights on [0, 1]
   int adj_nq_max = 0;
   void* d_zre;              // stationary parts, max_freqs x n (real)
@@ -339,8 +339,6 @@ kx_status launch_substep_control(kx_ctx* c, int slot0, int ns);
 kx_status launch_expm_project(kx_ctx* c, const double* dH, int ldh, int m, double beta,
                               double tau, const double* d_om, int nfreq, double* d_u);
 kx_status launch_shifted_solve(kx_ctx* c, int slot, int nfreq, int m);
-
-size_t expm_smem_bytes(int msz);
 
 // Persistent grid for a kernel: resident blocks (occupancy) x SMs, capped
 // by the work and by the partial-sum stride.

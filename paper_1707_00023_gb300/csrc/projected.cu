@@ -10,8 +10,6 @@
 
 namespace kx {
 
-size_t expm_smem_bytes(int msz) { return (size_t)6 * msz * msz * sizeof(double); }
-
 // ---------------------------------------------------------------------------
 // Time sub-step control (restart in time, Sect. 3.3): with the Arnoldi
 // decomposition of the current restart, u(t) = exp(-t H_m) beta e_1 is
