@@ -277,7 +277,7 @@ kx_status launch_pass_a_tr(kx_ctx* c, int slot0, int ns, int j);
 // pass A reading the per-cell permittivity directly (no 1/eps table)
 kx_status launch_pass_a_cells(kx_ctx* c, int slot, int j, const double* d_eps_cell);
 // pass B of step j; finalize = 1 launches its finalisation kernel, otherwise
-// the next step's pass A finalises it (non-augmented processes only)
+// the next step's pass A finalises it
 kx_status launch_pass_b(kx_ctx* c, int slot0, int ns, int j, int finalize);
 int pass_b_grid(kx_ctx* c);
 

@@ -63,43 +63,103 @@ __device__ __forceinline__ void block_partial(double x, double* part, int ps, in
   __syncthreads();
 }
 
-// Finalisation of step j-1's pass B at the start of step j's pass A
-// (non-augmented processes): every block sums the same nbb partials in the
-// same order, so all reach the same h_{j,j-1} and the same breakdown
-// decision; block 0 records them.  Returns false where the process stops
-// (lucky breakdown or a non-finite norm); *sj receives scale_j = 1/h.
+// Warp sums of eight values: lane l ends with the sum of value
+// column_of_lane8(l) (four lanes hold each).  Nine additions instead of forty
+// for eight separate sums: the lanes exchange halves of the values they keep.
 template <typename T>
-__device__ __forceinline__ bool fin_prev_b(const Slot<T>& s, int j, int ldh, int nbb, double btol, double* sj) {
-  double x = 0.0;
-  for (int b = threadIdx.x; b < nbb; b += blockDim.x) x += __ldcg(s.part + (int64_t)FINB_COL * s.ps + b);
-  __shared__ double red[NWARPS];
-  __shared__ double res;
+__device__ __forceinline__ T warp_sum8(T* p, int lane) {
+  const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    const T keep = b4 ? p[t + 4] : p[t], send = b4 ? p[t] : p[t + 4];
+    p[t] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
+  }
+#pragma unroll
+  for (int t = 0; t < 2; ++t) {
+    const T keep = b3 ? p[t + 2] : p[t], send = b3 ? p[t] : p[t + 2];
+    p[t] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
+  }
+  const T keep = b2 ? p[1] : p[0], send = b2 ? p[0] : p[1];
+  T x = keep + __shfl_xor_sync(0xffffffffu, send, 4);
+  x += __shfl_xor_sync(0xffffffffu, x, 2);
+  x += __shfl_xor_sync(0xffffffffu, x, 1);
+  return x;
+}
+__device__ __forceinline__ int column_of_lane8(int lane) { return lane >> 2; }
+
+// Finalisation of step j-1's pass B at the start of step j's pass A: every
+// block sums the same nbb partials in the same order, so all reach the same
+// h_{j,j-1} and the same breakdown decision; block 0 (rec) records them.
+// Returns false where the process stops (lucky breakdown or a non-finite
+// norm); *sj receives scale_j = 1/h.  An augmented process (AUG, the slot's
+// aug set) also gives the two phase entries of column j their Gram-Schmidt
+// update, from the raw entries that follow from column j-1's; *aj receives
+// the first (the others may not read what block 0 records).
+template <int AUG, typename T>
+__device__ __forceinline__ bool fin_prev_b(const Slot<T>& s, int j, int ldh, int nbb, double btol, bool rec,
+                                           double* sj, double* aj) {
+  double x = 0.0, pa = 0.0, pb = 0.0;
+  const int tid = threadIdx.x, nw = blockDim.x >> 5;
+  for (int b = tid; b < nbb; b += blockDim.x) x += __ldcg(s.part + (int64_t)FINB_COL * s.ps + b);
+  const bool augm = AUG && s.st->aug;
+  if (AUG && augm)
+    for (int col = tid; col < j; col += blockDim.x) {
+      const double cc = s.H[col + (int64_t)(j - 1) * ldh] * s.scale[col];
+      pa += cc * s.aug[2 * col];
+      pb += cc * s.aug[2 * col + 1];
+    }
+  __shared__ double red[3][NWARPS];
+  __shared__ double res, resa;
   __shared__ int stop;
   x = warp_sum(x);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = x;
+  if (AUG) {
+    pa = warp_sum(pa);
+    pb = warp_sum(pb);
+  }
+  if ((tid & 31) == 0) {
+    red[0][tid >> 5] = x;
+    red[1][tid >> 5] = pa;
+    red[2][tid >> 5] = pb;
+  }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double tot = 0.0;
-#pragma unroll
-    for (int w = 0; w < NWARPS; ++w) tot += red[w];
+  if (tid == 0) {
+    double tot = 0.0, a = 0.0, b = 0.0;
+    for (int w = 0; w < nw; ++w) tot += red[0][w];
+    if (AUG && augm) {
+      double sa = 0.0, sb = 0.0;
+      for (int w = 0; w < nw; ++w) {
+        sa += red[1][w];
+        sb += red[2][w];
+      }
+      const double W = s.st->omega, sp = s.scale[j - 1];
+      a = -W * sp * s.aug[2 * (j - 1) + 1] - sa;
+      b = W * sp * s.aug[2 * (j - 1)] - sb;
+      tot += a * a + b * b;
+    }
     const double h = sqrt(tot);
     int stp = 0;
     double scl = 0.0;
     if (!isfinite(h)) stp = 2;
     else if (h <= btol * s.st->wmax) stp = 1;   // invariant subspace: the projection is exact
     else scl = 1.0 / h;
-    if (blockIdx.x == 0) {
+    if (rec) {
       s.H[j + (int64_t)(j - 1) * ldh] = h;
       s.st->m_done = j;
       s.scale[j] = scl;
+      if (AUG) {
+        s.aug[2 * j] = a;
+        s.aug[2 * j + 1] = b;
+      }
       if (stp == 2) s.st->status = KX_ENONFINITE;
       if (stp || abort_requested(s.st)) s.st->done = 1;
     }
     res = scl;
+    resa = a;
     stop = stp;
   }
   __syncthreads();
   *sj = res;
+  *aj = resa;
   return stop == 0;
 }
 

@@ -153,7 +153,20 @@ kx_status launch_apply(kx_ctx* c, const void* v, void* w, int transpose) {
 // Arnoldi pass A (step j -> column j+1, Sect. 3.2 eq. (Arn)):
 //   w = A v_j  (v_j = scale[j] * V_j)       [augmented: w = [A y - (a/eta) g; -W b; W a]]
 //   d_i = V_i^T w for i <= j, and ||w||^2, fused in one sweep over the cells.
-// The last block forms H[i, j] = scale[i] * d_i.
+// k_fin_a forms H[i, j] = scale[i] * d_i.
+//
+// The launch's blockIdx.z is a group of basis columns: on small grids the
+// cells alone leave most SMs idle while each thread walks up to 64 columns
+// (36^3: 46 blocks of quads, 0.69 us a column), so the columns are split
+// between blocks that each form the same A v_j (about three columns' worth of
+// loads, from L2); group 0 writes it.  The dots of eight columns are summed
+// over a warp together (warp_sum8): in double precision, whose additions cost
+// as much as the products, eight separate sums (40 additions) took nearly as
+// long as a chunk's products (48 in 3D).
+__host__ __device__ __forceinline__ int col_group(int ncol, int groups) {
+  return ((ncol + groups - 1) / groups + 7) / 8 * 8;   // whole chunks of eight
+}
+
 template <typename T, int DIM, int AUG, typename Mat, int TR = 0>
 __global__ void __launch_bounds__(NTHREADS) k_pass_a(Geo g, SlotSet<T> ss, int j, int64_t ld, Mat mat,
                                                     const T* __restrict__ gsrc, int ldh, int nbb, double btol) {
@@ -166,18 +179,22 @@ __global__ void __launch_bounds__(NTHREADS) k_pass_a(Geo g, SlotSet<T> ss, int j
   for (int q = threadIdx.x; q < NWARPS * (MMAX + 2); q += blockDim.x) (&acc[0][0])[q] = 0.0;
   __syncthreads();
   // step j-1's pass B is finalised here when nbb > 0 (no separate kernel)
-  double sj;
+  const int grp = blockIdx.z;
+  double sj, aj = 0.0;
   if (nbb > 0) {
-    if (!fin_prev_b(s, j, ldh, nbb, btol, &sj)) return;
+    if (!fin_prev_b<AUG>(s, j, ldh, nbb, btol, blockIdx.x == 0 && grp == 0, &sj, &aj)) return;
   } else {
     sj = s.scale[j];
+    if (AUG) aj = s.aug[2 * j];
   }
   const T tsj = (T)sj;
   const T* __restrict__ vin = s.V + (int64_t)j * ld;
   T* __restrict__ wout = s.V + (int64_t)(j + 1) * ld;
   T gco = T(0);
-  if (AUG) gco = (T)(-(sj * s.aug[2 * j]) / s.st->eta);
+  if (AUG) gco = (T)(-(sj * aj) / s.st->eta);
   const int ncol = j + 1;
+  // this block's columns: group grp of gridDim.z (group 0 also writes w)
+  const int per = col_group(ncol, gridDim.z), cbeg = grp * per, cend = min(ncol, cbeg + per);
   const int64_t nc = g.ncell;
   for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < nc;
        base += (int64_t)gridDim.x * blockDim.x) {
@@ -193,7 +210,7 @@ __global__ void __launch_bounds__(NTHREADS) k_pass_a(Geo g, SlotSet<T> ss, int j
         if (AUG) {
           if (!is_wall(g, c, q.i, q.j, q.k)) o[c] += gco * gsrc[(int64_t)c * nc + cell];
         }
-        wout[(int64_t)c * nc + cell] = o[c];
+        if (grp == 0) wout[(int64_t)c * nc + cell] = o[c];
       }
     } else {
 #pragma unroll
@@ -202,32 +219,30 @@ __global__ void __launch_bounds__(NTHREADS) k_pass_a(Geo g, SlotSet<T> ss, int j
     T nrm = T(0);
 #pragma unroll
     for (int c = 0; c < NC; ++c) nrm += o[c] * o[c];
-    for (int c0 = 0; c0 < ncol; c0 += 8) {
+    for (int c0 = cbeg; c0 < cend; c0 += 8) {
       T p[8];
 #pragma unroll
       for (int t = 0; t < 8; ++t) {
         p[t] = T(0);
         const int col = c0 + t;
-        if (act && col < ncol) {
+        if (act && col < cend) {
           const T* __restrict__ vc = s.V + (int64_t)col * ld + cell;
 #pragma unroll
           for (int c = 0; c < NC; ++c) p[t] += vc[(int64_t)c * nc] * o[c];
         }
       }
-#pragma unroll
-      for (int t = 0; t < 8; ++t) p[t] = warp_sum(p[t]);
-      if (lane == 0) {
-#pragma unroll
-        for (int t = 0; t < 8; ++t)
-          if (c0 + t < ncol) acc[warp][c0 + t] += (double)p[t];
-      }
+      const T x = warp_sum8(p, lane);
+      const int col = c0 + column_of_lane8(lane);
+      if ((lane & 3) == 0 && col < cend) acc[warp][col] += (double)x;
     }
     nrm = warp_sum(nrm);
     if (lane == 0) acc[warp][MMAX + 1] += (double)nrm;
   }
   __syncthreads();
   // block partials: columns 0..j are the dots, column j+1 is ||w||^2
-  for (int col = threadIdx.x; col <= ncol; col += blockDim.x) {
+  const int nown = cend - cbeg + (grp == 0 ? 1 : 0);
+  for (int q = threadIdx.x; q < nown; q += blockDim.x) {
+    const int col = q < cend - cbeg ? cbeg + q : ncol;
     const int src = col < ncol ? col : MMAX + 1;
     double t = 0.0;
 #pragma unroll
@@ -258,18 +273,21 @@ __device__ __forceinline__ void pass_a4_body(Geo g, SlotSet<float> ss, int j, in
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int q = threadIdx.x; q < NWARPS * (MMAX + 2); q += blockDim.x) (&acc[0][0])[q] = 0.0;
   __syncthreads();
-  double sj;
+  const int grp = blockIdx.z;
+  double sj, aj = 0.0;
   if (nbb > 0) {
-    if (!fin_prev_b(s, j, ldh, nbb, btol, &sj)) return;
+    if (!fin_prev_b<AUG>(s, j, ldh, nbb, btol, blockIdx.x == 0 && grp == 0, &sj, &aj)) return;
   } else {
     sj = s.scale[j];
+    if (AUG) aj = s.aug[2 * j];
   }
   const float tsj = (float)sj;
   const float* __restrict__ v = s.V + (int64_t)j * ld;
   float* __restrict__ wout = s.V + (int64_t)(j + 1) * ld;
   float gco = 0.f;
-  if (AUG) gco = (float)(-(sj * s.aug[2 * j]) / s.st->eta);
+  if (AUG) gco = (float)(-(sj * aj) / s.st->eta);
   const int ncol = j + 1;
+  const int per = col_group(ncol, gridDim.z), cbeg = grp * per, cend = min(ncol, cbeg + per);
   const int64_t nc = g.ncell;
   const int64_t nq = nc >> 2;
   for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < nq; base += (int64_t)gridDim.x * blockDim.x) {
@@ -347,8 +365,10 @@ __device__ __forceinline__ void pass_a4_body(Geo g, SlotSet<float> ss, int j, in
           set4(o[c], e, x);
         }
       }
+      if (grp == 0) {
 #pragma unroll
-      for (int c = 0; c < 6; ++c) *reinterpret_cast<float4*>(wout + c * nc + c0) = o[c];
+        for (int c = 0; c < 6; ++c) *reinterpret_cast<float4*>(wout + c * nc + c0) = o[c];
+      }
     } else {
 #pragma unroll
       for (int c = 0; c < 6; ++c) o[c] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -357,32 +377,29 @@ __device__ __forceinline__ void pass_a4_body(Geo g, SlotSet<float> ss, int j, in
 #pragma unroll
     for (int c = 0; c < 6; ++c) nrm += dot4(o[c], o[c]);
     const int64_t cq = act ? (q4 << 2) : 0;
-    for (int cb = 0; cb < ncol; cb += 8) {
+    for (int cb = cbeg; cb < cend; cb += 8) {
       float p[8];
 #pragma unroll
       for (int t = 0; t < 8; ++t) {
         p[t] = 0.f;
         const int col = cb + t;
-        if (act && col < ncol) {
+        if (act && col < cend) {
           const float* __restrict__ vc = s.V + (int64_t)col * ld + cq;
 #pragma unroll
           for (int c = 0; c < 6; ++c) p[t] += dot4(ld4(vc + c * nc), o[c]);
         }
       }
-#pragma unroll
-      for (int t = 0; t < 8; ++t) p[t] = warp_sum(p[t]);
-      if (lane < 8 && cb + lane < ncol) {
-        float mine = p[0];
-#pragma unroll
-        for (int t = 1; t < 8; ++t) if (lane == t) mine = p[t];
-        acc[warp][cb + lane] += (double)mine;
-      }
+      const float x = warp_sum8(p, lane);
+      const int col = cb + column_of_lane8(lane);
+      if ((lane & 3) == 0 && col < cend) acc[warp][col] += (double)x;
     }
     nrm = warp_sum(nrm);
     if (lane == 0) acc[warp][MMAX + 1] += (double)nrm;
   }
   __syncthreads();
-  for (int col = threadIdx.x; col <= ncol; col += blockDim.x) {
+  const int nown = cend - cbeg + (grp == 0 ? 1 : 0);
+  for (int q = threadIdx.x; q < nown; q += blockDim.x) {
+    const int col = q < cend - cbeg ? cbeg + q : ncol;
     const int src = col < ncol ? col : MMAX + 1;
     double t = 0.0;
 #pragma unroll
@@ -467,6 +484,15 @@ __global__ void __launch_bounds__(NTHREADS) k_fin_a(SlotSet<float> ss, int j, in
 template <typename T>
 constexpr double btol_of() { return sizeof(T) == 8 ? 1e-12 : 1e-6; }
 
+// Column groups of a pass A launch: as many as fill the SMs' resident blocks
+// (cap) with the launch's cell blocks, each with a chunk of eight columns at
+// least.
+static int col_groups(int ncol, int64_t blocks, int cap) {
+  const int want = (int)std::max<int64_t>(1, std::min<int64_t>(cap / std::max<int64_t>(blocks, 1), (ncol + 7) / 8));
+  const int per = col_group(ncol, want);
+  return (ncol + per - 1) / per;   // no empty group
+}
+
 template <typename T>
 static kx_status pass_a_t(kx_ctx* c, int slot, int ns, int j, const void* gaug) {
   const Geo& g = c->geo;
@@ -497,9 +523,9 @@ static kx_status pass_a_t(kx_ctx* c, int slot, int ns, int j, const void* gaug) 
     gr = persistent_grid(c, fn, 1 << 30, 0);
   }
   const int nb = reserve_grid(c, (int)std::min<int64_t>(std::min<int64_t>(rounds, gr.load()), c->ps), gr.load());
-  const dim3 grd(nb, ns);
-  // a non-augmented process finalises step j-1's pass B here
-  const int nbb = (j >= 1 && !gaug) ? pass_b_grid(c) : 0;
+  const dim3 grd(nb, ns, col_groups(j + 1, (int64_t)nb * ns, gr.load()));
+  // step j-1's pass B is finalised here
+  const int nbb = j >= 1 ? pass_b_grid(c) : 0;
   const double bt = btol_of<T>();
   if (vec4) {
     SlotSet<float> sf = make_slotset<float>(c, slot);
@@ -545,11 +571,12 @@ static kx_status pass_a_cells_t(kx_ctx* c, int slot, int j, const double* eps) {
                                        : (const void*)k_pass_a<T, 3, 0, CellMat<T>>, 1 << 30, 0);
   const int nb = (int)std::min<int64_t>(std::min<int64_t>(rounds, gr.load()), c->ps);
   const int nbb = j >= 1 ? pass_b_grid(c) : 0;
+  const dim3 grd(nb, 1, col_groups(j + 1, nb, gr.load()));
   if (g.dim == 2)
-    k_pass_a<T, 2, 0, CellMat<T>><<<nb, NTHREADS, 0, c->stream>>>(g, s, j, c->ld, mat, nullptr, c->m + 1, nbb,
+    k_pass_a<T, 2, 0, CellMat<T>><<<grd, NTHREADS, 0, c->stream>>>(g, s, j, c->ld, mat, nullptr, c->m + 1, nbb,
                                                                   btol_of<T>());
   else
-    k_pass_a<T, 3, 0, CellMat<T>><<<nb, NTHREADS, 0, c->stream>>>(g, s, j, c->ld, mat, nullptr, c->m + 1, nbb,
+    k_pass_a<T, 3, 0, CellMat<T>><<<grd, NTHREADS, 0, c->stream>>>(g, s, j, c->ld, mat, nullptr, c->m + 1, nbb,
                                                                   btol_of<T>());
   KX_CHECK_LAUNCH(c);
   k_fin_a<<<j + 2, NTHREADS, 0, c->stream>>>(make_slotset<float>(c, slot), j, c->m + 1, nb, 0);
@@ -571,7 +598,7 @@ static kx_status pass_a_tr_t(kx_ctx* c, int slot, int ns, int j) {
     gr = persistent_grid(c, g.dim == 2 ? (const void*)k_pass_a<T, 2, 0, TableMat<T>, 1>
                                        : (const void*)k_pass_a<T, 3, 0, TableMat<T>, 1>, 1 << 30, 0);
   const int nb = (int)std::min<int64_t>(std::min<int64_t>(rounds, gr.load()), c->ps);
-  const dim3 grd(nb, ns);
+  const dim3 grd(nb, ns, col_groups(j + 1, (int64_t)nb * ns, gr.load()));
   const int nbb = j >= 1 ? pass_b_grid(c) : 0;
   if (g.dim == 2)
     k_pass_a<T, 2, 0, TableMat<T>, 1><<<grd, NTHREADS, 0, c->stream>>>(g, s, j, c->ld, mat, nullptr, c->m + 1, nbb,

@@ -564,7 +564,7 @@ __device__ __forceinline__ float warp_sum2(float v0, float v1, int lane) {
 // Sweep S_j, 3D FP32, with the basis staged through shared memory: a block
 // owns tiles of SW_TILE cells (one quad a thread) and, for each tile,
 // streams the columns V_0..V_{j-1} through a ring of SW_STAGES buffers that
-// one thread fills with one-dimensional bulk copies (cp.async.bulk, their
+// six threads fill with one-dimensional bulk copies (cp.async.bulk, their
 // completion counted on an mbarrier per buffer).  The bytes in flight per SM
 // then no longer depend on registers: a register-fed form, with the 128
 // registers two blocks per SM allow, kept one column per warp in flight
@@ -630,19 +630,23 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, unsigned b
 // (16-byte aligned: tiles start at multiples of 1024 cells, columns at
 // multiples of 64 scalars, components at multiples of ncell with
 // ncell % 4 == 0; each copy is a multiple of 16 bytes).
+// The six copies are issued by one thread each of the block's first six
+// warps: a copy takes its thread tens of clocks to issue, and one thread
+// issuing all of them held up its warp and, through the block's barrier,
+// every warp (arnoldi() in this form, 64 steps: 36^3 3080 -> 2860 us, 128^3
+// 20.2 -> 20.0 ms).  The thread of component 0 also announces the bytes; a
+// copy that lands first leaves the barrier's byte count negative, and the
+// phase still waits for that thread's arrival.
 __device__ __forceinline__ void sw_issue(const Slot<float>& s, int64_t ld, int64_t nc, int64_t tile, int col, int b,
-                                         float* ring, uint64_t* full) {
+                                         float* ring, uint64_t* full, int c) {
   const int64_t cell0 = tile * SW_TILE;
   const int64_t cells = nc - cell0 < SW_TILE ? nc - cell0 : SW_TILE;
   const unsigned bytes = (unsigned)(cells * (int64_t)sizeof(float));
-  float* dst = ring + b * SW_STAGE_FLOATS;
-  const float* src = s.V + (int64_t)col * ld + cell0;
-  mbar_expect_tx(&full[b], 6u * bytes);
-#pragma unroll
-  for (int c = 0; c < 6; ++c) bulk_load(dst + c * SW_TILE, src + c * nc, bytes, &full[b]);
+  if (c == 0) mbar_expect_tx(&full[b], 6u * bytes);
+  bulk_load(ring + b * SW_STAGE_FLOATS + c * SW_TILE, s.V + (int64_t)col * ld + cell0 + c * nc, bytes, &full[b]);
 }
 
-// The issue cursor of a block's stream (thread 0 only): advancing it by one
+// The issue cursor of a block's stream (the issuing threads): advancing it by one
 // element moves to the next column, or to the first column of the block's
 // next tile (no division in the loop).
 struct SwCursor {
@@ -685,10 +689,11 @@ __device__ __forceinline__ void sw_pass4s_body(const Geo& g, const Slot<float>& 
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
-  SwCursor cur{(int64_t)bid, 0, nblk};   // the next element to issue (thread 0)
-  if (threadIdx.x == 0)
+  const bool issuer = lane == 0 && warp < 6;   // of component `warp`
+  SwCursor cur{(int64_t)bid, 0, nblk};         // the next element to issue
+  if (issuer)
     for (int64_t e = 0; e < E && e < SW_STAGES; ++e) {
-      sw_issue(s, ld, nc, cur.tile, cur.col, (int)e, ring, full);
+      sw_issue(s, ld, nc, cur.tile, cur.col, (int)e, ring, full, warp);
       cur.next(j);
     }
   const float* __restrict__ t = (const float*)w.t;
@@ -804,11 +809,11 @@ __device__ __forceinline__ void sw_pass4s_body(const Geo& g, const Slot<float>& 
       }
       return;
     }
-    if (threadIdx.x == 0) {
+    if (issuer) {
       for (int q = 0; q < cnt; ++q) {
         if (e + q + SW_STAGES >= E) break;
         if (q == 0) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        sw_issue(s, ld, nc, cur.tile, cur.col, (int)((e + q) & (SW_STAGES - 1)), ring, full);
+        sw_issue(s, ld, nc, cur.tile, cur.col, (int)((e + q) & (SW_STAGES - 1)), ring, full, warp);
         cur.next(j);
       }
     }
