@@ -86,11 +86,15 @@ SlotState fresh_state() {
   return s;
 }
 
-// m Arnoldi steps on slots [slot0, slot0 + ns) from their (normalised)
-// column 0, all slots in the same launches.
-kx_status arnoldi_steps(kx_ctx* c, int slot0, int ns, int m, const void* g_aug) {
-  for (int j = 0; j < m; ++j) {
-    KX_TRY(launch_pass_a(c, slot0, ns, j, g_aug));
+// m Arnoldi steps (two-pass form, of A^T when transpose) on slots
+// [slot0, slot0 + ns) from their (normalised) column 0: one cooperative launch
+// where the grid fits the resident threads, else all slots in the same
+// launches, three a step.
+kx_status arnoldi_steps(kx_ctx* c, int slot0, int ns, int m, const void* g_aug, int transpose = 0) {
+  bool ran = false;
+  KX_TRY(coop_arnoldi(c, slot0, ns, m, g_aug, transpose, &ran));
+  for (int j = 0; j < m && !ran; ++j) {
+    KX_TRY(transpose ? launch_pass_a_tr(c, slot0, ns, j) : launch_pass_a(c, slot0, ns, j, g_aug));
     // the next pass A finalises it; the last step needs the kernel
     KX_TRY(launch_pass_b(c, slot0, ns, j, j == m - 1));
   }
@@ -965,10 +969,12 @@ kx_status response_at_freqs(kx_ctx* c, const void* d_g, const double* omegas, in
 
 // The Arnoldi process of one restart in Krylov dimension (basis slot
 // `slot`, non-augmented).  By default the single-sweep form runs from
-// SWEEP_MIN_UNKNOWNS unknowns up: its serial per-step finalisation (a few
-// microseconds) hides behind the apply pass only on large grids (measured on
-// GB300: at 64^3 the two-pass form is faster, from 96^3 up the single sweep).
-constexpr int64_t SWEEP_MIN_UNKNOWNS = 3000000;
+// SWEEP_MIN_UNKNOWNS unknowns up.  Below, the two-pass process in one
+// cooperative launch is faster: a restart of 64 steps takes 1.7 against 2.8 ms
+// at 48^3 and 3.0 against 3.5 ms at 56^3 (1.05e6 unknowns); at 60^3 (1.3e6)
+// 4.3 against 3.6 ms, since two of its blocks then fill every SM and the
+// projected work beside it has to wait for the process to end.
+constexpr int64_t SWEEP_MIN_UNKNOWNS = 1200000;
 
 bool rst_uses_sweep(const kx_ctx* c) {
   if (c->d.arnoldi_form == KX_ARN_SWEEP) return true;
@@ -1265,16 +1271,8 @@ kx_status adjoint_response_grad(kx_ctx* c, const void* d_g, const double* omegas
                                  c->stream), "state upload");
       KX_TRY(sync(c));
       KX_TRY(launch_norm_init(c, 0, 2));
-      for (int j = 0; j < c->m; ++j) {
-        KX_TRY(launch_pass_a(c, 0, 1, j, d_g));
-        KX_TRY(launch_pass_b(c, 0, 1, j, j == c->m - 1));
-      }
-      for (int j = 0; j < c->m; ++j) {
-        KX_TRY(launch_pass_a_tr(c, 1, 1, j));
-        KX_TRY(launch_pass_b(c, 1, 1, j, j == c->m - 1));
-      }
-      c->stats.arnoldi_steps += 2 * (int64_t)c->m;
-      c->stats.matvecs += 2 * (int64_t)c->m;
+      KX_TRY(arnoldi_steps(c, 0, 1, c->m, d_g));
+      KX_TRY(arnoldi_steps(c, 1, 1, c->m, nullptr, 1));
       KX_TRY(read_states(c, 0, 2));
       if (c->h_state[0].status || c->h_state[1].status)
         return fail(c, KX_ENONFINITE, "adjoint backward: Krylov process failed");

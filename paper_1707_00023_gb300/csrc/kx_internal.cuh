@@ -73,7 +73,7 @@ struct Slot {
   double* scale;     // m+2 column scales: v_i = scale[i] * V_i
   double* part;      // PCOLS x ps partial sums, column-major by block
   int ps;            // partial-sum column stride (>= any grid size)
-  unsigned* counter; // block-completion counter (8 slots)
+  unsigned* counter; // block-completion counter, grid barrier, stop flag (8 slots)
   double* u;         // projected coefficients (m)
   SlotState* st;
 };
@@ -280,6 +280,12 @@ kx_status launch_pass_a_cells(kx_ctx* c, int slot, int j, const double* d_eps_ce
 // the next step's pass A finalises it
 kx_status launch_pass_b(kx_ctx* c, int slot0, int ns, int j, int finalize);
 int pass_b_grid(kx_ctx* c);
+
+// coop.cu: m steps of the two-pass process on slots [slot0, slot0 + ns), from
+// their column 0 as set by the launch that normalised it, in one cooperative
+// launch (for as many slots as fit at a time); *ran = false where the grid is
+// too large for one item a resident thread
+kx_status coop_arnoldi(kx_ctx* c, int slot0, int ns, int m, const void* g_aug, int transpose, bool* ran);
 
 // adjoint.cu
 kx_status launch_adj_seed(kx_ctx* c, const void* y, void* lam, int axis, int idx);

@@ -43,10 +43,13 @@ __device__ __forceinline__ Cell make_cell(const Geo& g, int64_t cell) {
   return q;
 }
 
-template <typename T>
-__device__ __forceinline__ T ldv(const Geo& g, const T* __restrict__ v, int c, int64_t idx, int i,
-                                 int j, int k) {
-  return is_wall(g, c, i, j, k) ? T(0) : v[(int64_t)c * g.ncell + idx];
+// CG: the load goes past L1 (a vector that other blocks of the same launch write).
+template <bool CG, typename T>
+__device__ __forceinline__ T ldv(const Geo& g, const T* v, int c, int64_t idx, int i, int j, int k) {
+  if (is_wall(g, c, i, j, k)) return T(0);
+  const T* p = v + (int64_t)c * g.ncell + idx;
+  if constexpr (CG) return __ldcg(p);
+  else return *p;
 }
 
 // Material accessors.  TableMat reads the 1/eps arrays and the sigma table
@@ -116,17 +119,16 @@ __host__ __device__ constexpr int ncomp_of(int DIM) { return DIM == 3 ? 6 : (DIM
 // and A^T follows the blocks (with u = (w_Ez + sigma w_P) / eps on the Ez
 // nodes): Hx: -du/dy, Hy: sigma w_Hy + d(w_Ez/eps)/dx, Ez: sigma w_Ez + curl
 // w_H, P: -w_Ez.  sigma depends on x only.
-template <typename T, int DIM, int TR, typename Mat>
-__device__ __forceinline__ void stencil(const Geo& g, const T* __restrict__ v, const Mat& mat,
-                                        const Cell& q, T* out) {
+template <typename T, int DIM, int TR, typename Mat, bool CG = false>
+__device__ __forceinline__ void stencil(const Geo& g, const T* v, const Mat& mat, const Cell& q, T* out) {
   const int64_t nc = g.ncell;
   const int i = q.i, j = q.j, k = q.k;
   if (DIM == 4) {
     (void)nc;
-    const T Hx = ldv(g, v, 0, q.c0, i, j, k), Hy = ldv(g, v, 1, q.c0, i, j, k);
-    const T Hy_im = ldv(g, v, 1, q.cim, q.im, j, k), Hx_jm = ldv(g, v, 0, q.cjm, i, q.jm, k);
-    const T Ez = ldv(g, v, 2, q.c0, i, j, k), P = ldv(g, v, 3, q.c0, i, j, k);
-    const T Ez_jp = ldv(g, v, 2, q.cjp, i, q.jp, k), Ez_ip = ldv(g, v, 2, q.cip, q.ip, j, k);
+    const T Hx = ldv<CG>(g, v, 0, q.c0, i, j, k), Hy = ldv<CG>(g, v, 1, q.c0, i, j, k);
+    const T Hy_im = ldv<CG>(g, v, 1, q.cim, q.im, j, k), Hx_jm = ldv<CG>(g, v, 0, q.cjm, i, q.jm, k);
+    const T Ez = ldv<CG>(g, v, 2, q.c0, i, j, k), P = ldv<CG>(g, v, 3, q.c0, i, j, k);
+    const T Ez_jp = ldv<CG>(g, v, 2, q.cjp, i, q.jp, k), Ez_ip = ldv<CG>(g, v, 2, q.cip, q.ip, j, k);
     const T sH = mat.sigma(g, q, 1), sE = mat.sigma(g, q, 2);
     const T ie0 = mat.inv_eps(g, 0, q.c0);
     const T curlH = (Hy - Hy_im) - (Hx - Hx_jm);
@@ -136,7 +138,7 @@ __device__ __forceinline__ void stencil(const Geo& g, const T* __restrict__ v, c
       out[2] = sE * Ez - ie0 * curlH - P;
       out[3] = sE * ie0 * (Hx - Hx_jm);
     } else {
-      const T P_jp = ldv(g, v, 3, q.cjp, i, q.jp, k);
+      const T P_jp = ldv<CG>(g, v, 3, q.cjp, i, q.jp, k);
       const T u = (Ez + sE * P) * ie0;
       const T u_jp = (Ez_jp + sE * P_jp) * mat.inv_eps(g, 0, q.cjp);
       out[0] = -(u_jp - u);
@@ -146,10 +148,10 @@ __device__ __forceinline__ void stencil(const Geo& g, const T* __restrict__ v, c
     }
   } else if (DIM == 2) {
     // components 0 Hx (0,1/2), 1 Hy (1/2,0), 2 Ez (0,0)
-    const T Hx = ldv(g, v, 0, q.c0, i, j, k), Hy = ldv(g, v, 1, q.c0, i, j, k);
-    const T Hy_im = ldv(g, v, 1, q.cim, q.im, j, k), Hx_jm = ldv(g, v, 0, q.cjm, i, q.jm, k);
-    T Ez = ldv(g, v, 2, q.c0, i, j, k);
-    T Ez_jp = ldv(g, v, 2, q.cjp, i, q.jp, k), Ez_ip = ldv(g, v, 2, q.cip, q.ip, j, k);
+    const T Hx = ldv<CG>(g, v, 0, q.c0, i, j, k), Hy = ldv<CG>(g, v, 1, q.c0, i, j, k);
+    const T Hy_im = ldv<CG>(g, v, 1, q.cim, q.im, j, k), Hx_jm = ldv<CG>(g, v, 0, q.cjm, i, q.jm, k);
+    T Ez = ldv<CG>(g, v, 2, q.c0, i, j, k);
+    T Ez_jp = ldv<CG>(g, v, 2, q.cjp, i, q.jp, k), Ez_ip = ldv<CG>(g, v, 2, q.cip, q.ip, j, k);
     const T s0 = mat.sigma(g, q, 0), s1 = mat.sigma(g, q, 1), s2 = mat.sigma(g, q, 2);
     const T curlH = (Hy - Hy_im) - (Hx - Hx_jm);
     if (!TR) {
@@ -166,16 +168,16 @@ __device__ __forceinline__ void stencil(const Geo& g, const T* __restrict__ v, c
     }
   } else {
     const int ip = q.ip, im = q.im, jp = q.jp, jm = q.jm, kp = q.kp, km = q.km;
-    const T Hx = ldv(g, v, 0, q.c0, i, j, k), Hy = ldv(g, v, 1, q.c0, i, j, k);
-    const T Hz = ldv(g, v, 2, q.c0, i, j, k);
-    T Ex = ldv(g, v, 3, q.c0, i, j, k), Ey = ldv(g, v, 4, q.c0, i, j, k);
-    T Ez = ldv(g, v, 5, q.c0, i, j, k);
-    T Ez_jp = ldv(g, v, 5, q.cjp, i, jp, k), Ey_kp = ldv(g, v, 4, q.ckp, i, j, kp);
-    T Ex_kp = ldv(g, v, 3, q.ckp, i, j, kp), Ez_ip = ldv(g, v, 5, q.cip, ip, j, k);
-    T Ey_ip = ldv(g, v, 4, q.cip, ip, j, k), Ex_jp = ldv(g, v, 3, q.cjp, i, jp, k);
-    const T Hz_jm = ldv(g, v, 2, q.cjm, i, jm, k), Hy_km = ldv(g, v, 1, q.ckm, i, j, km);
-    const T Hx_km = ldv(g, v, 0, q.ckm, i, j, km), Hz_im = ldv(g, v, 2, q.cim, im, j, k);
-    const T Hy_im = ldv(g, v, 1, q.cim, im, j, k), Hx_jm = ldv(g, v, 0, q.cjm, i, jm, k);
+    const T Hx = ldv<CG>(g, v, 0, q.c0, i, j, k), Hy = ldv<CG>(g, v, 1, q.c0, i, j, k);
+    const T Hz = ldv<CG>(g, v, 2, q.c0, i, j, k);
+    T Ex = ldv<CG>(g, v, 3, q.c0, i, j, k), Ey = ldv<CG>(g, v, 4, q.c0, i, j, k);
+    T Ez = ldv<CG>(g, v, 5, q.c0, i, j, k);
+    T Ez_jp = ldv<CG>(g, v, 5, q.cjp, i, jp, k), Ey_kp = ldv<CG>(g, v, 4, q.ckp, i, j, kp);
+    T Ex_kp = ldv<CG>(g, v, 3, q.ckp, i, j, kp), Ez_ip = ldv<CG>(g, v, 5, q.cip, ip, j, k);
+    T Ey_ip = ldv<CG>(g, v, 4, q.cip, ip, j, k), Ex_jp = ldv<CG>(g, v, 3, q.cjp, i, jp, k);
+    const T Hz_jm = ldv<CG>(g, v, 2, q.cjm, i, jm, k), Hy_km = ldv<CG>(g, v, 1, q.ckm, i, j, km);
+    const T Hx_km = ldv<CG>(g, v, 0, q.ckm, i, j, km), Hz_im = ldv<CG>(g, v, 2, q.cim, im, j, k);
+    const T Hy_im = ldv<CG>(g, v, 1, q.cim, im, j, k), Hx_jm = ldv<CG>(g, v, 0, q.cjm, i, jm, k);
     T s[6];
 #pragma unroll
     for (int c = 0; c < 6; ++c) s[c] = mat.sigma(g, q, c);

@@ -344,7 +344,8 @@ __global__ void __launch_bounds__(NTHREADS) k_restart(SlotSet<T> ss, int64_t n, 
   if ((threadIdx.x & 31) == 0) red2[threadIdx.x >> 5] = xs;
   __syncthreads();
   if (threadIdx.x == 0) {
-    *s.counter = 0u;
+    s.counter[0] = 0u;
+    s.counter[1] = 0u;   // the grid barrier of the process that starts here (coop.cu)
     double tot = 0.0;
 #pragma unroll
     for (int w = 0; w < NWARPS; ++w) tot += red2[w];
