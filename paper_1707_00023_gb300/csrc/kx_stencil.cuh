@@ -330,16 +330,21 @@ __device__ __forceinline__ float ldw(const float* __restrict__ p, int idx, unsig
   return (w >> c) & 1u ? 0.f : p[idx];
 }
 
-// t = A v, 3D FP32 lossy-layer model, for the cells of grid column col =
-// i + nx j on planes k0 .. k1-1 (0 <= k0 < k1 <= nz): the rows of
-// stencil_quad with the same operations in the same order (the same bits
-// on every cell), the index and wall work done once per column and, marching
-// up in z, E_x, E_y of plane k+1 and H_x, H_y of plane k kept in registers,
-// where the next plane reads them as its own and its k-1 values (14 field
-// loads a cell instead of 18).  32-bit cell offsets: ncell < 2^31.
-__device__ __forceinline__ void stencil_column32(const Geo& g, const float* __restrict__ v,
-                                                 const float* __restrict__ ie, const float* __restrict__ sig2,
-                                                 float* __restrict__ t, int col, int k0, int k1) {
+// t = A v (TR = 0) or A^T v (TR = 1), 3D lossy-layer model, for the cells of
+// grid column col = i + nx j on planes k0 .. k1-1 (0 <= k0 < k1 <= nz): the rows
+// of stencil<T, 3, TR, TableMat<T>> with the same operations in the same order
+// (the same bits on every cell), the index and wall work done once per column
+// and, marching up in z, E_x, E_y of plane k+1 and H_x, H_y of plane k kept in
+// registers, where the next plane reads them as its own and its k-1 values (14
+// field loads a cell instead of 18).  32-bit cell offsets: ncell < 2^31.
+template <typename T>
+__device__ __forceinline__ T ldwt(const T* __restrict__ p, int idx, unsigned w, int c) {
+  return (w >> c) & 1u ? T(0) : p[idx];
+}
+template <typename T, int TR>
+__device__ __forceinline__ void stencil_column(const Geo& g, const T* __restrict__ v, const T* __restrict__ ie,
+                                               const T* __restrict__ sig2, T* __restrict__ t, int col, int k0,
+                                               int k1) {
   const int nx = g.nx, ny = g.ny, nz = g.nz, nxy = nx * ny;
   const int nc = (int)g.ncell;
   const int i = col % nx, j = col / nx;
@@ -353,47 +358,64 @@ __device__ __forceinline__ void stencil_column32(const Geo& g, const float* __re
   const unsigned wim = (im == 0 ? xm : 0u) | (j == 0 ? ym : 0u);
   const unsigned wjp = (i == 0 ? xm : 0u) | (jp == 0 ? ym : 0u);
   const unsigned wjm = (i == 0 ? xm : 0u) | (jm == 0 ? ym : 0u);
-  const float* __restrict__ vHx = v;
-  const float* __restrict__ vHy = v + nc;
-  const float* __restrict__ vHz = v + 2 * (int64_t)nc;
-  const float* __restrict__ vEx = v + 3 * (int64_t)nc;
-  const float* __restrict__ vEy = v + 4 * (int64_t)nc;
-  const float* __restrict__ vEz = v + 5 * (int64_t)nc;
+  const T* __restrict__ vHx = v;
+  const T* __restrict__ vHy = v + nc;
+  const T* __restrict__ vHz = v + 2 * (int64_t)nc;
+  const T* __restrict__ vEx = v + 3 * (int64_t)nc;
+  const T* __restrict__ vEy = v + 4 * (int64_t)nc;
+  const T* __restrict__ vEz = v + 5 * (int64_t)nc;
+  const T* __restrict__ ie1 = ie + nc;
+  const T* __restrict__ ie2 = ie + 2 * (int64_t)nc;
   const int km0 = k0 == 0 ? nz - 1 : k0 - 1;
   unsigned zk = k0 == 0 ? zm : 0u;
   int cell = col + k0 * nxy;
   const int ckm0 = col + km0 * nxy;
   const unsigned wkm0 = wc | (km0 == 0 ? zm : 0u);
-  float hx_km = ldw(vHx, ckm0, wkm0, 0), hy_km = ldw(vHy, ckm0, wkm0, 1);
-  float ex = ldw(vEx, cell, wc | zk, 3), ey = ldw(vEy, cell, wc | zk, 4);
+  T hx_km = ldwt(vHx, ckm0, wkm0, 0), hy_km = ldwt(vHy, ckm0, wkm0, 1);
+  T ex = ldwt(vEx, cell, wc | zk, 3), ey = ldwt(vEy, cell, wc | zk, 4);
+  if (TR) {   // the curl of E / eps
+    ex *= ie[cell];
+    ey *= ie1[cell];
+  }
   for (int k = k0; k < k1; ++k, cell += nxy) {
     const int kp = k + 1 == nz ? 0 : k + 1;
     const unsigned zkp = kp == 0 ? zm : 0u;
     const int ckp = col + kp * nxy;
     const unsigned mk = wc | zk, mkp = wc | zkp;
-    const float hx = ldw(vHx, cell, mk, 0), hy = ldw(vHy, cell, mk, 1);
-    const float hz = ldw(vHz, cell, mk, 2), ez = ldw(vEz, cell, mk, 5);
-    const float ex_kp = ldw(vEx, ckp, mkp, 3), ey_kp = ldw(vEy, ckp, mkp, 4);
-    const float ez_jp = ldw(vEz, cell + djp, wjp | zk, 5), ex_jp = ldw(vEx, cell + djp, wjp | zk, 3);
-    const float hz_jm = ldw(vHz, cell + djm, wjm | zk, 2), hx_jm = ldw(vHx, cell + djm, wjm | zk, 0);
-    const float ez_ip = ldw(vEz, cell + dip, wip | zk, 5), ey_ip = ldw(vEy, cell + dip, wip | zk, 4);
-    const float hz_im = ldw(vHz, cell + dim, wim | zk, 2), hy_im = ldw(vHy, cell + dim, wim | zk, 1);
+    const T hx = ldwt(vHx, cell, mk, 0), hy = ldwt(vHy, cell, mk, 1);
+    const T hz = ldwt(vHz, cell, mk, 2);
+    T ez = ldwt(vEz, cell, mk, 5);
+    T ex_kp = ldwt(vEx, ckp, mkp, 3), ey_kp = ldwt(vEy, ckp, mkp, 4);
+    T ez_jp = ldwt(vEz, cell + djp, wjp | zk, 5), ex_jp = ldwt(vEx, cell + djp, wjp | zk, 3);
+    const T hz_jm = ldwt(vHz, cell + djm, wjm | zk, 2), hx_jm = ldwt(vHx, cell + djm, wjm | zk, 0);
+    T ez_ip = ldwt(vEz, cell + dip, wip | zk, 5), ey_ip = ldwt(vEy, cell + dip, wip | zk, 4);
+    const T hz_im = ldwt(vHz, cell + dim, wim | zk, 2), hy_im = ldwt(vHy, cell + dim, wim | zk, 1);
+    if (TR) {
+      ez *= ie2[cell];
+      ex_kp *= ie[ckp];
+      ey_kp *= ie1[ckp];
+      ez_jp *= ie2[cell + djp];
+      ex_jp *= ie[cell + djp];
+      ez_ip *= ie2[cell + dip];
+      ey_ip *= ie1[cell + dip];
+    }
     const int li = g.la == 0 ? i : (g.la == 1 ? j : k);
-    float sg[6];
+    T sg[6];
 #pragma unroll
     for (int c = 0; c < 6; ++c) sg[c] = sig2[2 * li + g.sighalf[c]];
-    const float cHx = (hz - hz_jm) - (hy - hy_km);
-    const float cHy = (hx - hx_km) - (hz - hz_im);
-    const float cHz = (hy - hy_im) - (hx - hx_jm);
-    float o[6];
-    o[0] = sg[0] * hx + ((ez_jp - ez) - (ey_kp - ey));
-    o[1] = sg[1] * hy + ((ex_kp - ex) - (ez_ip - ez));
-    o[2] = sg[2] * hz + ((ey_ip - ey) - (ex_jp - ex));
-    o[3] = ie[cell] * (sg[3] * ex - cHx);
-    o[4] = ie[(int64_t)nc + cell] * (sg[4] * ey - cHy);
-    o[5] = ie[2 * (int64_t)nc + cell] * (sg[5] * ez - cHz);
+    const T cHx = (hz - hz_jm) - (hy - hy_km);
+    const T cHy = (hx - hx_km) - (hz - hz_im);
+    const T cHz = (hy - hy_im) - (hx - hx_jm);
+    const T uEx = (ez_jp - ez) - (ey_kp - ey), uEy = (ex_kp - ex) - (ez_ip - ez), uEz = (ey_ip - ey) - (ex_jp - ex);
+    T o[6];
+    o[0] = TR ? sg[0] * hx - uEx : sg[0] * hx + uEx;
+    o[1] = TR ? sg[1] * hy - uEy : sg[1] * hy + uEy;
+    o[2] = TR ? sg[2] * hz - uEz : sg[2] * hz + uEz;
+    o[3] = TR ? sg[3] * ex + cHx : ie[cell] * (sg[3] * ex - cHx);
+    o[4] = TR ? sg[4] * ey + cHy : ie1[cell] * (sg[4] * ey - cHy);
+    o[5] = TR ? sg[5] * ez + cHz : ie2[cell] * (sg[5] * ez - cHz);
 #pragma unroll
-    for (int c = 0; c < 6; ++c) t[c * (int64_t)nc + cell] = (mk >> c) & 1u ? 0.f : o[c];
+    for (int c = 0; c < 6; ++c) t[c * (int64_t)nc + cell] = (mk >> c) & 1u ? T(0) : o[c];
     hx_km = hx;
     hy_km = hy;
     ex = ex_kp;
@@ -416,7 +438,7 @@ __device__ __forceinline__ float4 ldw4(const float* __restrict__ p, int idx, uns
   return r;
 }
 
-// The column march of stencil_column32 on a quad of x-cells (nx % 4 == 0):
+// The column march of stencil_column on a quad of x-cells (nx % 4 == 0):
 // quad column q = i0/4 + (nx/4) j, planes k0 .. k1-1; sixteen-byte loads
 // and stores, the x neighbours outside the quad by one scalar load each
 // side, the arithmetic of stencil_quad on every cell (the same bits).

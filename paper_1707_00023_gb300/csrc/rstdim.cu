@@ -532,70 +532,111 @@ kx_status launch_rst_plane(kx_ctx* c, cudaStream_t st, int slot, int nfreq, int 
 // combination is summed error-free (two-product by FMA, Knuth's two-sum) and
 // added to the float-pair accumulator (Y_j, lo_j) by a two-sum, so the
 // accumulated response keeps about twice float precision over the restarts.
-__device__ __forceinline__ void rst_acc(float& s, float& c, float hi, float lo, float v) {
-  const float p = hi * v;
-  const float e = fmaf(hi, v, -p) + lo * v;
-  const float t = s + p;
-  const float z = t - s;
-  c += ((s - (t - z)) + (p - z)) + e;
+// One thread a field value, its basis row in registers; the coefficients'
+// float pairs are formed once a block (formed at every use, in double
+// precision on this GPU's slow pipe, they were most of this kernel's time:
+// 36^3, 4 frequencies 855 us).  FP32 takes two values a thread: the packed
+// operations serve both and each pair of coefficients is loaded once for them.
+__device__ __forceinline__ void rst_acc2(float2& s, float2& c, float2 hi, float2 lo, float2 v) {
+  const float2 m1 = make_float2(-1.f, -1.f);
+  const float2 p = __fmul2_rn(hi, v);
+  const float2 np = __fmul2_rn(p, m1);
+  const float2 e = __ffma2_rn(lo, v, __ffma2_rn(hi, v, np));
+  const float2 t = __fadd2_rn(s, p);
+  const float2 z = __ffma2_rn(s, m1, t);                       // t - s
+  const float2 d = __ffma2_rn(z, m1, t);                       // t - z
+  c = __fadd2_rn(c, __fadd2_rn(__fadd2_rn(__ffma2_rn(d, m1, s), __ffma2_rn(z, m1, p)), e));
   s = t;
 }
 
-template <typename T>
-__global__ void __launch_bounds__(NTHREADS) k_rst_full(Slot<T> s, int64_t ld, int64_t n, int nfreq,
-                                                      const int* __restrict__ fstate,
-                                                      const double* __restrict__ u, T* __restrict__ Y,
-                                                      float* __restrict__ lo_acc) {
-  __shared__ double cf[MAXF][MMAX];
+__global__ void __launch_bounds__(128) k_rst_full32(Slot<float> s, int64_t ld, int64_t n, int nfreq,
+                                                   const int* __restrict__ fstate, const double* __restrict__ u,
+                                                   float* __restrict__ Y, float* __restrict__ lo_acc) {
+  extern __shared__ __align__(16) float4 cf4[];   // per frequency and column: hi, hi, lo, lo
   __shared__ int act[MAXF];
   const int md = s.st->m_done;
   for (int q = threadIdx.x; q < nfreq * MMAX; q += blockDim.x) {
-    const int f = q / MMAX, j = q - f * MMAX;
-    cf[f][j] = j < md ? u[(int64_t)f * MMAX + j] * s.scale[j] : 0.0;
+    const int j = q % MMAX;
+    const double c = j < md ? u[q] * s.scale[j] : 0.0;
+    const float hi = (float)c, lo = (float)(c - (double)hi);
+    cf4[q] = make_float4(hi, hi, lo, lo);
+  }
+  for (int f = threadIdx.x; f < nfreq; f += blockDim.x) act[f] = !(fstate[f] == 2 || fstate[f] == 3);
+  __syncthreads();
+  const int64_t half = (n + 1) >> 1;
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < half; e += (int64_t)gridDim.x * blockDim.x) {
+    // values e and e + half (the last may not exist)
+    const int64_t e2 = e + half < n ? e + half : e;
+    float2 v[MMAX];
+#pragma unroll
+    for (int j = 0; j < MMAX; ++j)
+      v[j] = j < md ? make_float2(s.V[(int64_t)j * ld + e], s.V[(int64_t)j * ld + e2]) : make_float2(0.f, 0.f);
+    for (int f = 0; f < nfreq; ++f) {
+      if (!act[f]) continue;
+      float2 sx = make_float2(0.f, 0.f), cx = sx;
+      const float4* cf = cf4 + f * MMAX;
+#pragma unroll
+      for (int j = 0; j < MMAX; ++j) {
+        const float4 c = cf[j];
+        rst_acc2(sx, cx, make_float2(c.x, c.y), make_float2(c.z, c.w), v[j]);
+      }
+      // (Y, lo) += sx + cx
+      auto fold = [&](int64_t i, float sv, float cv) {
+        float& yh = Y[(int64_t)f * n + i];
+        float& yl = lo_acc[(int64_t)f * n + i];
+        const float t = yh + sv;
+        const float z = t - yh;
+        const float err = (yh - (t - z)) + (sv - z);
+        yh = t;
+        yl += err + cv;
+      };
+      fold(e, sx.x, cx.x);
+      if (e2 != e) fold(e2, sx.y, cx.y);
+    }
+  }
+}
+
+__global__ void __launch_bounds__(NTHREADS) k_rst_full64(Slot<double> s, int64_t ld, int64_t n, int nfreq,
+                                                        const int* __restrict__ fstate,
+                                                        const double* __restrict__ u, double* __restrict__ Y) {
+  extern __shared__ __align__(16) double cf[];    // nfreq x MMAX
+  __shared__ int act[MAXF];
+  const int md = s.st->m_done;
+  for (int q = threadIdx.x; q < nfreq * MMAX; q += blockDim.x) {
+    const int j = q % MMAX;
+    cf[q] = j < md ? u[q] * s.scale[j] : 0.0;
   }
   for (int f = threadIdx.x; f < nfreq; f += blockDim.x) act[f] = !(fstate[f] == 2 || fstate[f] == 3);
   __syncthreads();
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-    T v[MMAX];
+    double v[MMAX];
 #pragma unroll
-    for (int j = 0; j < MMAX; ++j) v[j] = j < md ? s.V[(int64_t)j * ld + e] : T(0);
+    for (int j = 0; j < MMAX; ++j) v[j] = j < md ? s.V[(int64_t)j * ld + e] : 0.0;
     for (int f = 0; f < nfreq; ++f) {
       if (!act[f]) continue;
-      if constexpr (sizeof(T) == 8) {
-        double acc = 0.0;
+      double acc = 0.0;
 #pragma unroll
-        for (int j = 0; j < MMAX; ++j) acc = fma(cf[f][j], (double)v[j], acc);
-        Y[(int64_t)f * n + e] += (T)acc;
-      } else {
-        float sx = 0.f, cx = 0.f;
-#pragma unroll
-        for (int j = 0; j < MMAX; ++j) {
-          const float hi = (float)cf[f][j];
-          const float lo = (float)(cf[f][j] - (double)hi);
-          rst_acc(sx, cx, hi, lo, (float)v[j]);
-        }
-        // (Y, lo) += sx + cx
-        float& yh = reinterpret_cast<float*>(Y)[(int64_t)f * n + e];
-        float& yl = lo_acc[(int64_t)f * n + e];
-        const float t = yh + sx;
-        const float z = t - yh;
-        const float err = (yh - (t - z)) + (sx - z);
-        yh = t;
-        yl += err + cx;
-      }
+      for (int j = 0; j < MMAX; ++j) acc = fma(cf[f * MMAX + j], v[j], acc);
+      Y[(int64_t)f * n + e] += acc;
     }
   }
 }
 
 kx_status launch_rst_full(kx_ctx* c, cudaStream_t st, int slot, int nfreq, void* Y) {
+  static SmemOptIn attr{};
+  const kx_status so = smem_opt_in(c, attr, (const void*)k_rst_full32, MAXF * MMAX * sizeof(float4));
+  if (so != KX_OK) return so;
   time_begin(c);
-  if (c->d.precision == KX_FP64)
-    k_rst_full<double><<<c->nblk, NTHREADS, 0, st>>>(make_slot<double>(c, slot), c->ld, c->n, nfreq,
-                                                            c->d_rst_state, c->d_rst_u, (double*)Y, nullptr);
-  else
-    k_rst_full<float><<<c->nblk, NTHREADS, 0, st>>>(make_slot<float>(c, slot), c->ld, c->n, nfreq,
-                                                           c->d_rst_state, c->d_rst_u, (float*)Y,
-                                                           (float*)c->d_zre);
+  if (c->d.precision == KX_FP64) {
+    k_rst_full64<<<c->nblk, NTHREADS, nfreq * MMAX * sizeof(double), st>>>(make_slot<double>(c, slot), c->ld, c->n,
+                                                                           nfreq, c->d_rst_state, c->d_rst_u,
+                                                                           (double*)Y);
+  } else {
+    const int64_t blocks = std::min<int64_t>(((c->n + 1) / 2 + 127) / 128, (int64_t)c->nsm * 8);
+    k_rst_full32<<<(int)blocks, 128, nfreq * MMAX * sizeof(float4), st>>>(make_slot<float>(c, slot), c->ld, c->n,
+                                                                          nfreq, c->d_rst_state, c->d_rst_u,
+                                                                          (float*)Y, (float*)c->d_zre);
+  }
   time_end(c, KX_K_RESTART, (c->m + 3.0 * nfreq) * c->n * c->esize);
   KX_CHECK_LAUNCH(c);
   return KX_OK;

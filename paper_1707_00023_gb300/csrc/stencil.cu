@@ -119,9 +119,53 @@ __global__ void __launch_bounds__(NTHREADS) k_apply(Geo g, const T* __restrict__
   }
 }
 
+// 3D: a thread marches one grid column (QUAD: four neighbouring ones, 16-byte
+// loads) up kz planes.  One cell a thread spent its time on index divisions and
+// wall tests: 128^3 in single precision 45.2 us for 126 MB.  Block b: columns
+// (b % ncb) NTHREADS .., planes kz (b / ncb) ..
+template <typename T, bool QUAD, int TR>
+__global__ void __launch_bounds__(NTHREADS, QUAD ? 2 : 3)
+    k_apply_col(Geo g, const T* __restrict__ v, T* __restrict__ w, const T* __restrict__ ie,
+                const T* __restrict__ sig2, int ncb, int kz) {
+  const int zc = (int)blockIdx.x / ncb;
+  const int q = ((int)blockIdx.x - zc * ncb) * NTHREADS + (int)threadIdx.x;
+  const int ncol = QUAD ? (g.nx >> 2) * g.ny : g.nx * g.ny;
+  const int k0 = zc * kz, k1 = min(g.nz, k0 + kz);
+  if (q >= ncol || k0 >= k1) return;
+  if constexpr (QUAD) stencil_column_quad(g, v, ie, sig2, w, q, k0, k1);
+  else stencil_column<T, TR>(g, v, ie, sig2, w, q, k0, k1);
+}
+
+// Planes a thread: enough blocks for every resident slot, no more than
+// APPLY_KZ planes (a longer march leaves too few loads in flight).
+constexpr int APPLY_KZ = 8;
+
+template <typename T, bool QUAD, int TR>
+static void apply_col(kx_ctx* c, const T* v, T* w, const T* ie, const T* sg) {
+  const Geo& g = c->geo;
+  const int64_t ncol = QUAD ? (int64_t)(g.nx / 4) * g.ny : (int64_t)g.nx * g.ny;
+  const int ncb = (int)((ncol + NTHREADS - 1) / NTHREADS);
+  const int slots = c->nsm * (QUAD ? 2 : 3);
+  const int64_t kz = std::min<int64_t>(APPLY_KZ, std::max<int64_t>(1, ((int64_t)g.nz * ncb + slots - 1) / slots));
+  k_apply_col<T, QUAD, TR><<<ncb * (int)((g.nz + kz - 1) / kz), NTHREADS, 0, c->stream>>>(g, v, w, ie, sg, ncb,
+                                                                                          (int)kz);
+}
+
 template <typename T>
 static kx_status apply_t(kx_ctx* c, const void* v, void* w, int tr) {
   const Geo& g = c->geo;
+  if (g.dim == 3 && g.ncell < ((int64_t)1 << 31)) {
+    const T *vt = (const T*)v, *iet = (const T*)c->d_inv_eps, *sgt = (const T*)c->d_sig2;
+    bool quad = false;
+    if constexpr (sizeof(T) == 4) {
+      quad = !tr && g.nx % 4 == 0 && ((uintptr_t)v % 16) == 0 && ((uintptr_t)w % 16) == 0;
+      if (quad) apply_col<T, true, 0>(c, vt, (T*)w, iet, sgt);
+    }
+    if (!quad && tr) apply_col<T, false, 1>(c, vt, (T*)w, iet, sgt);
+    else if (!quad) apply_col<T, false, 0>(c, vt, (T*)w, iet, sgt);
+    KX_CHECK_LAUNCH(c);
+    return KX_OK;
+  }
   const int blocks = (int)std::min<int64_t>((g.ncell + NTHREADS - 1) / NTHREADS, (int64_t)c->nblk * 4);
   const T* ie = (const T*)c->d_inv_eps;
   const T* sg = (const T*)c->d_sig2;

@@ -362,7 +362,7 @@ __device__ __forceinline__ void sw_apply4_body(const Geo& g, const Slot<float>& 
 // Apply pass K_j for j >= 1, 3D FP32: SW_RED reducer blocks in front, then
 // blocks of NTHREADS grid columns (quads of x-cells when QUAD, nx % 4 == 0),
 // block b covering planes kz (b / ncb) .. kz (b / ncb + 1) - 1 of its
-// columns, marching up in z (stencil_column_quad / stencil_column32: the
+// columns, marching up in z (stencil_column_quad / stencil_column: the
 // index work once per column, four of the eighteen neighbour values a cell
 // carried from the plane below).  Against one cell a thread with its
 // per-cell index and wall arithmetic (ALU pipe at 70 % of peak), 128^3
@@ -388,7 +388,7 @@ __global__ void __launch_bounds__(NTHREADS, QUAD ? 2 : 3)
     if constexpr (QUAD)
       stencil_column_quad(g, v, ie, sig2, t, q, k0, k1);
     else
-      stencil_column32(g, v, ie, sig2, t, q, k0, k1);
+      stencil_column<float, 0>(g, v, ie, sig2, t, q, k0, k1);
   }
   pdl_trigger();
 }
