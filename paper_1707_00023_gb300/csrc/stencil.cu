@@ -121,7 +121,8 @@ __global__ void __launch_bounds__(NTHREADS) k_apply(Geo g, const T* __restrict__
 
 // 3D: a thread marches one grid column (QUAD: four neighbouring ones, 16-byte
 // loads) up kz planes.  One cell a thread spent its time on index divisions and
-// wall tests: 128^3 in single precision 45.2 us for 126 MB.  Block b: columns
+// wall tests: 128^3 in single precision 45.2 us for 126 MB, now 26.7 (61^3
+// 8.3 -> 6.2, A^T at 128^3 53.4 -> 34.3).  Block b: columns
 // (b % ncb) NTHREADS .., planes kz (b / ncb) ..
 template <typename T, bool QUAD, int TR>
 __global__ void __launch_bounds__(NTHREADS, QUAD ? 2 : 3)
@@ -137,7 +138,11 @@ __global__ void __launch_bounds__(NTHREADS, QUAD ? 2 : 3)
 }
 
 // Planes a thread: enough blocks for every resident slot, no more than
-// APPLY_KZ planes (a longer march leaves too few loads in flight).
+// APPLY_KZ planes (a longer march leaves too few loads in flight: quads at
+// 128^3 26.7 us with 7 planes, 30.5 with 1, 37.1 with 16).  In double precision
+// one: the stencil's additions fill that pipe (128^3 110 us for 252 MB with 1
+// to 3 planes), and the carried values only lengthen the march (64^3 18.5 us
+// with 1, 22.6 with 8); A^T gains the index work (139 -> 116 us).
 constexpr int APPLY_KZ = 8;
 
 template <typename T, bool QUAD, int TR>
@@ -146,7 +151,7 @@ static void apply_col(kx_ctx* c, const T* v, T* w, const T* ie, const T* sg) {
   const int64_t ncol = QUAD ? (int64_t)(g.nx / 4) * g.ny : (int64_t)g.nx * g.ny;
   const int ncb = (int)((ncol + NTHREADS - 1) / NTHREADS);
   const int slots = c->nsm * (QUAD ? 2 : 3);
-  const int64_t kz = std::min<int64_t>(APPLY_KZ, std::max<int64_t>(1, ((int64_t)g.nz * ncb + slots - 1) / slots));
+  const int64_t kz = sizeof(T) == 8 ? 1 : std::min<int64_t>(APPLY_KZ, std::max<int64_t>(1, ((int64_t)g.nz * ncb + slots - 1) / slots));
   k_apply_col<T, QUAD, TR><<<ncb * (int)((g.nz + kz - 1) / kz), NTHREADS, 0, c->stream>>>(g, v, w, ie, sg, ncb,
                                                                                           (int)kz);
 }
