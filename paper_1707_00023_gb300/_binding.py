@@ -211,14 +211,15 @@ class Context:
             raise KxError(st, self.lib.kx_last_error(self.h).decode())
 
     def _vec(self, t, name, ncols=1):
-        torch = self._torch
-        if not isinstance(t, torch.Tensor) or not t.is_cuda:
+        """The device address (an int, which the argument types take) of a
+        checked field vector."""
+        if not isinstance(t, self._torch.Tensor) or not t.is_cuda:
             raise TypeError(f"{name} must be a CUDA tensor")
         if t.dtype != self.dtype:
             raise TypeError(f"{name} must be {self.dtype}")
         if not t.is_contiguous() or t.numel() != self.n * ncols:
             raise ValueError(f"{name} must be contiguous with {self.n * ncols} elements")
-        return ctypes.c_void_p(t.data_ptr())
+        return t.data_ptr()
 
     def empty(self, *cols):
         return self._torch.empty((*cols, self.n), dtype=self.dtype, device="cuda")
@@ -259,9 +260,15 @@ class Context:
 
     # -- ABI calls -----------------------------------------------------------
     def apply_A(self, v, w=None, transpose=False):
+        pv = self._vec(v, "v")
         if w is None:
-            w = self._torch.empty_like(v)
-        self._check(self.lib.apply_A(self.h, self._vec(v, "v"), self._vec(w, "w"), int(bool(transpose))))
+            w = self._torch.empty_like(v)   # v's shape, type and layout: nothing left to check
+            pw = w.data_ptr()
+        else:
+            pw = self._vec(w, "w")
+        st = self.lib.apply_A(self.h, pv, pw, 1 if transpose else 0)
+        if st != KX_OK:
+            self._check(st)
         return w
 
     def arnoldi(self, v0, m, want_V=True):
@@ -417,7 +424,7 @@ def response_multi(ctxs, gs, omegas, T, rtol=1e-8, method="plain", planes=None, 
     nf = om.shape[1]
     pl = np.ascontiguousarray(np.asarray(planes, np.int32).reshape(n, 2))
     hs = (ctypes.c_void_p * n)(*[c.h for c in ctxs])
-    gp = (ctypes.c_void_p * n)(*[c._vec(g, "g").value for c, g in zip(ctxs, gs)])
+    gp = (ctypes.c_void_p * n)(*[c._vec(g, "g") for c, g in zip(ctxs, gs)])
     inten = np.zeros((n, nf))
     err = np.zeros((n, nf))
     st = lib.response_at_freqs_multi(hs, n, gp, _dptr(om), nf, float(T), float(rtol),
@@ -464,7 +471,7 @@ class Batch:
         om = np.ascontiguousarray(np.asarray(omegas, np.float64).reshape(n, -1))
         nf = om.shape[1]
         pl = np.ascontiguousarray(np.asarray(planes, np.int32).reshape(n, 2))
-        gp = (ctypes.c_void_p * n)(*[c._vec(g, "g").value for c, g in zip(self.ctxs, gs)])
+        gp = (ctypes.c_void_p * n)(*[c._vec(g, "g") for c, g in zip(self.ctxs, gs)])
         inten = np.zeros((n, nf))
         res = np.zeros((n, nf))
         rst = np.zeros((n, nf), np.int32)

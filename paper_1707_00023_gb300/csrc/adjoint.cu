@@ -246,17 +246,21 @@ __global__ void __launch_bounds__(256) k_adj_moments(const double* __restrict__ 
 // thread a node, W's column of the node in registers, M in shared memory.
 // With M formed first a node costs 66 x 64 products whatever the number of
 // quadrature nodes; evaluating both factors at every node took 129 FMAs a
-// node and quadrature point (240 of them at tau = 12: 667 us at 48^3).  The
-// entries of M cancel where the factors at a node did not, so the sums carry
-// their rounding errors (hi + lo, kx_eft.cuh) and M is a float pair: five
-// packed operations for two products.
+// node and quadrature point (240 of them at tau = 12: 667 us at 48^3).
+// In double-precision contexts the sums carry their rounding errors (hi + lo,
+// kx_eft.cuh) and M is a float pair, five packed operations for two products:
+// the entries of M cancel where the factors at a node did not, and plain sums
+// missed that path's accuracy (1.07e-7 on a gradient held to 1e-7).  In
+// single-precision contexts, whose bases are off by as much, plain packed sums
+// do (48^3: 320 -> 115 us).
 template <typename T>
 __global__ void __launch_bounds__(128) k_adj_accum(Geo g, const T* __restrict__ V, const T* __restrict__ W,
                                                   int64_t ld, int mV, int mW, const T* __restrict__ gsrc,
                                                   const T* __restrict__ ie, const float* __restrict__ M,
                                                   double* __restrict__ Q) {
-  __shared__ __align__(16) float sM[2 * ADJ_A * MMAX];
-  for (int o = threadIdx.x; o < 2 * ADJ_A * MMAX; o += blockDim.x) sM[o] = M[o];
+  constexpr bool COMP = sizeof(T) == 8;
+  __shared__ __align__(16) float sM[(COMP ? 2 : 1) * ADJ_A * MMAX];
+  for (int o = threadIdx.x; o < (COMP ? 2 : 1) * ADJ_A * MMAX; o += blockDim.x) sM[o] = M[o];
   __syncthreads();
   const int64_t nE = (int64_t)g.ne * g.ncell;
   const int64_t off = (int64_t)g.nh * g.ncell;
@@ -268,29 +272,42 @@ __global__ void __launch_bounds__(128) k_adj_accum(Geo g, const T* __restrict__ 
       w[k].y = 2 * k + 1 < mW ? (float)W[(int64_t)(2 * k + 1) * ld + off + e] : 0.f;
     }
     float qh = 0.f, ql = 0.f;
-#pragma unroll 1
+#pragma unroll(COMP ? 1 : 2)
     for (int i = 0; i <= mV + 1; ++i) {
       const int row = i <= mV ? i : MMAX + 1;
       const float v = i <= mV ? (float)V[(int64_t)i * ld + off + e] : (float)gsrc[off + e];
       const float4* mh = reinterpret_cast<const float4*>(sM + row * MMAX);
-      const float4* ml = reinterpret_cast<const float4*>(sM + (ADJ_A + row) * MMAX);
       float2 h0 = make_float2(0.f, 0.f), h1 = h0, l0 = h0, l1 = h0;
+      if constexpr (COMP) {
+        const float4* ml = reinterpret_cast<const float4*>(sM + (ADJ_A + row) * MMAX);
 #pragma unroll
-      for (int k = 0; k < MMAX / 4; ++k) {
-        const float4 x = mh[k], y = ml[k];
-        l0 = __ffma2_rn(make_float2(y.x, y.y), w[2 * k], l0);
-        l1 = __ffma2_rn(make_float2(y.z, y.w), w[2 * k + 1], l1);
-        sub_fma2(h0, l0, make_float2(x.x, x.y), w[2 * k]);
-        sub_fma2(h1, l1, make_float2(x.z, x.w), w[2 * k + 1]);
+        for (int k = 0; k < MMAX / 4; ++k) {
+          const float4 x = mh[k], y = ml[k];
+          l0 = __ffma2_rn(make_float2(y.x, y.y), w[2 * k], l0);
+          l1 = __ffma2_rn(make_float2(y.z, y.w), w[2 * k + 1], l1);
+          sub_fma2(h0, l0, make_float2(x.x, x.y), w[2 * k]);
+          sub_fma2(h1, l1, make_float2(x.z, x.w), w[2 * k + 1]);
+        }
+        // t = h + l: the four partial sums added with their errors
+        float th = 0.f, tl = (l0.x + l0.y) + (l1.x + l1.y);
+        sub_fma(th, tl, 1.f, h0.x);
+        add_two(th, tl, h0.y);
+        add_two(th, tl, h1.x);
+        add_two(th, tl, h1.y);
+        ql = fmaf(v, tl, ql);
+        sub_fma(qh, ql, v, th);
+      } else {
+#pragma unroll
+        for (int k = 0; k < MMAX / 4; k += 2) {
+          const float4 x = mh[k], y = mh[k + 1];
+          h0 = __ffma2_rn(make_float2(x.x, x.y), w[2 * k], h0);
+          h1 = __ffma2_rn(make_float2(x.z, x.w), w[2 * k + 1], h1);
+          l0 = __ffma2_rn(make_float2(y.x, y.y), w[2 * k + 2], l0);
+          l1 = __ffma2_rn(make_float2(y.z, y.w), w[2 * k + 3], l1);
+        }
+        h0 = __fadd2_rn(__fadd2_rn(h0, h1), __fadd2_rn(l0, l1));
+        sub_fma(qh, ql, v, h0.x + h0.y);
       }
-      // t = h + l: the four partial sums added with their errors
-      float th = 0.f, tl = (l0.x + l0.y) + (l1.x + l1.y);
-      sub_fma(th, tl, 1.f, h0.x);
-      add_two(th, tl, h0.y);
-      add_two(th, tl, h1.x);
-      add_two(th, tl, h1.y);
-      ql = fmaf(v, tl, ql);
-      sub_fma(qh, ql, v, th);
     }
     Q[e] += ((double)qh + (double)ql) * (double)ie[e];
   }

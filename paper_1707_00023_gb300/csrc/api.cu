@@ -1019,14 +1019,13 @@ kx_status response_restart_dim(kx_ctx* c, const void* d_g, const double* omegas,
     }
   } side{c};
   c->side_ctas = nfreq + 1;
-  // the projected work of a restart (set-up, cascade, ...) runs beside the
-  // first steps of the next process; in the later steps the single-sweep
-  // launches take every SM slot (half the steps covers it at 96^3 and
-  // 128^3, where this runs 3-6 % faster than keeping the reservation
-  // throughout).  The two-pass form, used on smaller grids whose processes
-  // are shorter than the projected work, keeps it for every step.  A fixed
-  // rule, so every mode has the same grids and bits.
-  c->side_steps = (c->m + 1) / 2;
+  // the projected work of a restart (set-up, march, samples: under half a
+  // millisecond of kernels) runs beside the first steps of the next process;
+  // in the later steps the single-sweep launches take every SM slot (128^3
+  // with the reservation for 32, 16, 8, 4 steps: 516, 513.5, 513, 515 ms).  The
+  // two-pass form keeps it for every step.  A fixed rule, so every mode has
+  // the same grids and bits.
+  c->side_steps = (c->m + 7) / 8;
   // the Arnoldi chain of this method runs with programmatic dependent launch
   c->pdl = 1;
   const size_t vbytes = (size_t)c->n * c->esize;

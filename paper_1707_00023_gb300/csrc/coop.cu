@@ -40,13 +40,14 @@ constexpr unsigned CO_WAIT_LIMIT = 1u << 21;   // polls of one barrier wait (abo
 
 // Barrier over the `blocks` blocks of a slot: the counter reaches `target`
 // (blocks times the barriers so far; zeroed by the kernel that normalises
-// column 0).  False when the wait runs out.
+// column 0).  False when the wait runs out.  The release on the arrival covers
+// the writes of the whole block (ordered before it by the block barrier), and
+// the acquire on the poll the reads after it.
 __device__ __forceinline__ bool grid_barrier(unsigned* cnt, unsigned target) {
   __shared__ int ok;
   __syncthreads();
   if (threadIdx.x == 0) {
-    __threadfence();
-    atomicAdd(cnt, 1u);
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(cnt) : "memory");
     int good = 0;
     for (unsigned k = 0; k < CO_WAIT_LIMIT; ++k) {
       unsigned v;
@@ -56,7 +57,6 @@ __device__ __forceinline__ bool grid_barrier(unsigned* cnt, unsigned target) {
         break;
       }
     }
-    __threadfence();
     ok = good;
   }
   __syncthreads();
@@ -314,8 +314,8 @@ __global__ void __launch_bounds__(CO_MAXT, MINB) k_coop(Geo g, SlotSet<typename 
   __shared__ S red[CO_MAXT / 32];
   __shared__ double tot[MMAX + 8], scl[MMAX + 1], augs[2 * (MMAX + 1)];
   __shared__ T coef[MMAX + 8];
-  __shared__ double bc[2];
-  __shared__ int halt;
+  __shared__ T sh_sj, sh_gco;                         // scale of v_j, factor of g
+  __shared__ int halt, sh_bad;
   const Slot<T> s = slot_at(ss, blockIdx.y);
   SlotState* st = s.st;
   if (st->done || st->retired) return;
@@ -330,12 +330,15 @@ __global__ void __launch_bounds__(CO_MAXT, MINB) k_coop(Geo g, SlotSet<typename 
   const int64_t nc = g.ncell;
   T* Vc = s.V + (act ? P::first(item) : 0);           // this thread's part of column 0
   const bool augm = AUG && st->aug;
+  // warp 0's own: double-precision work on few values, kept off the others
   const double omega = augm ? st->omega : 0.0, reta = augm ? 1.0 / st->eta : 0.0;
-  double wmax2 = st->wmax * st->wmax, sj = s.scale[0];
+  double wmax2 = st->wmax * st->wmax, sj = s.scale[0], na = 0.0, nb = 0.0;
   if (tid == 0) {
     scl[0] = sj;
     augs[0] = s.aug[0];
     augs[1] = s.aug[1];
+    sh_sj = (T)sj;
+    sh_gco = augm ? (T)(-(sj * s.aug[0]) * reta) : T(0);
   }
   auto timeout = [&]() {
     if (tid == 0) {
@@ -349,10 +352,9 @@ __global__ void __launch_bounds__(CO_MAXT, MINB) k_coop(Geo g, SlotSet<typename 
     // phase A
     V o[NC];
     if (act) {
-      const T gco = augm ? (T)(-(sj * augs[2 * j]) * reta) : T(0);
       int64_t im = item;
       asm volatile("" : "+l"(im));   // the index work is redone each step: held over the loop it would spill
-      P::apply(g, s.V + (int64_t)j * ld, ie, sig2, gsrc, (T)sj, gco, im, o);
+      P::apply(g, s.V + (int64_t)j * ld, ie, sig2, gsrc, sh_sj, sh_gco, im, o);
     } else {
 #pragma unroll
       for (int c = 0; c < NC; ++c) o[c] = P::zero();
@@ -423,10 +425,10 @@ __global__ void __launch_bounds__(CO_MAXT, MINB) k_coop(Geo g, SlotSet<typename 
     }
     __syncthreads();
     // h_ij and the phase entries' update (a lane a column)
-    const double wa = augm ? -omega * sj * augs[2 * j + 1] : 0.0, wb = augm ? omega * sj * augs[2 * j] : 0.0;
-    int bad = 0;
     if (warp == 0) {
+      const double wa = augm ? -omega * sj * augs[2 * j + 1] : 0.0, wb = augm ? omega * sj * augs[2 * j] : 0.0;
       double pa = 0.0, pb = 0.0;
+      int bad = 0;
       for (int q = lane; q < ((ncol + 7) & ~7); q += 32) {
         double cc = 0.0;
         if (q < ncol) {
@@ -444,18 +446,17 @@ __global__ void __launch_bounds__(CO_MAXT, MINB) k_coop(Geo g, SlotSet<typename 
         coef[q] = (T)cc;   // zero past the last column of the last chunk
       }
       if (AUG && augm) {
-        pa = warp_sum(pa);
-        pb = warp_sum(pb);
-        if (lane == 0) {
-          bc[0] = wa - pa;
-          bc[1] = wb - pb;
-        }
+        na = wa - warp_sum(pa);
+        nb = wb - warp_sum(pb);
       }
+      const double wn2 = tot[ncol] + (wa * wa + wb * wb);
+      bad |= !isfinite(wn2);
+      if (wn2 > wmax2) wmax2 = wn2;
+      bad = __any_sync(0xffffffffu, bad);
+      if (lane == 0) sh_bad = bad;
     }
-    const double wn2 = tot[ncol] + (wa * wa + wb * wb);
-    bad |= !isfinite(wn2);
-    if (wn2 > wmax2) wmax2 = wn2;
-    if (__syncthreads_or(bad)) {
+    __syncthreads();
+    if (sh_bad) {
       if (rec && tid == 0) {
         st->status = KX_ENONFINITE;
         st->done = 1;
@@ -534,23 +535,25 @@ __global__ void __launch_bounds__(CO_MAXT, MINB) k_coop(Geo g, SlotSet<typename 
       S xs = SO::of(T(0));
       for (int q = lane; q < G; q += 32) xs = add(xs, SO::get(s.part + (int64_t)FINB_COL * s.ps + q));
       const int abrt = __ldcg(s.counter + 2) != 0u;
-      const double a = augm ? bc[0] : 0.0, bb = augm ? bc[1] : 0.0;
-      const double x = value(warp_total(xs)) + (a * a + bb * bb);   // h_{j+1,j}^2
+      const double x = value(warp_total(xs)) + (na * na + nb * nb);   // h_{j+1,j}^2
       int stop = 0;
       double sc = 0.0;
       if (!isfinite(x)) stop = 2;
       else if (x <= btol * btol * wmax2) stop = 1;   // invariant subspace: the projection is exact
       else sc = rsqrt(x);
+      sj = sc;
       if (lane == 0) {
         scl[j + 1] = sc;
-        augs[2 * (j + 1)] = a;
-        augs[2 * (j + 1) + 1] = bb;
+        augs[2 * (j + 1)] = na;
+        augs[2 * (j + 1) + 1] = nb;
+        sh_sj = (T)sc;
+        if (AUG) sh_gco = (T)(-(sc * na) * reta);
         halt = stop || abrt;
         if (rec) {
           s.scale[j + 1] = sc;
           if (AUG) {
-            s.aug[2 * (j + 1)] = a;
-            s.aug[2 * (j + 1) + 1] = bb;
+            s.aug[2 * (j + 1)] = na;
+            s.aug[2 * (j + 1) + 1] = nb;
           }
           st->m_done = j + 1;
           if (stop == 2) st->status = KX_ENONFINITE;
@@ -560,7 +563,6 @@ __global__ void __launch_bounds__(CO_MAXT, MINB) k_coop(Geo g, SlotSet<typename 
       if (rec && lane == 0) s.H[(j + 1) + (int64_t)j * ldh] = sqrt(x);
     }
     __syncthreads();
-    sj = scl[j + 1];
     if (halt) return;
   }
 }
