@@ -6,7 +6,8 @@
 // and an exponential 0.9 ms; the matrices themselves are 33 KB.  Each block
 // therefore owns R = ceil(n / CD_CTAS) rows of every matrix, held in its
 // shared memory, and multiplies them with a right operand staged whole in
-// shared memory (8 us for n = 64, FP64-bound).  Rows of X Y need all of Y but
+// shared memory (4.3 us for n = 64 at the pipe's rate).  Sixteen blocks against
+// the portable eight: an exponential of norm 2 at m = 64 61 against 94 us.  Rows of X Y need all of Y but
 // only the same rows of X, so a chain of products with one fixed right
 // operand (the powers of A, the Horner steps in A^4) runs without any
 // exchange between the blocks; only a new right operand is published through
@@ -21,16 +22,16 @@
 // SIAM J. Sci. Comput. 33(2), eq. (3.9)'s bound, evaluated in 60-digit
 // arithmetic).
 //
-// Measured at m = 64: an exponential of norm 2 (eight products) 94 us, the
-// step control of one sub-step 969 -> 105 us, the set-up of a restart 1060 ->
-// 235 us, the projected solutions of 32 frequencies 1337 -> 235 us.
+// Measured at m = 64: the step control of one sub-step 969 -> 88 us, the
+// set-up of a restart 1060 -> 179 us, the projected solutions of 32
+// frequencies 1337 -> 155 us.
 #pragma once
 
 #include "kx_internal.cuh"
 
 namespace kx {
 
-constexpr int CD_CTAS = 8;                 // thread blocks a cluster (the portable size)
+constexpr int CD_CTAS = 16;                // thread blocks a cluster (beyond the portable eight: opted in per kernel)
 constexpr int CD_THREADS = 256;
 constexpr int CD_NMAX = MMAX + RST_P;      // largest matrix
 constexpr int CD_RMAX = (CD_NMAX + CD_CTAS - 1) / CD_CTAS;
@@ -266,6 +267,7 @@ inline cudaError_t launch_cluster(void (*kern)(KArgs...), int clusters, size_t s
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute at[1];
+  cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = CD_CTAS;
   at[0].val.clusterDim.y = 1;

@@ -185,7 +185,7 @@ kx_status launch_substep_control(kx_ctx* c, int slot, int ns) {
 //              four extra columns P A^i e_1, whatever nfreq;
 //   squaring : X <- X^2, Y <- X Y + Y exp(J).
 // Against one exponential of order m + 2 a frequency, each on one block (32
-// frequencies, m = 64, tau ||H|| = 40: 1337 us) now 235 us.
+// frequencies, m = 64, tau ||H|| = 40: 1337 us) now 155 us.
 constexpr int PHI_YLD = 2 * MAXF;                       // row stride of the Y block
 constexpr int PHI_SMEM = CD_SMEM + (2 * CD_RMAX + MMAX) * PHI_YLD * (int)sizeof(double);
 static_assert(CD_WS_MATS * CD_MAT + 2 * MMAX * PHI_YLD <= 2 * CD_WS, "the workspace of two clusters holds it");
