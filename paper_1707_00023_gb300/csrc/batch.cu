@@ -170,7 +170,7 @@ kx_status set_grids(kx_batch* b, int tpb, int rpt) {
     I.ncb = (int)((ncol + NTHREADS - 1) / NTHREADS);
     I.kz = std::min(c->geo.nz, 2 * rpt);
     I.c0 = b->coff[i];
-    I.nc = SW_RED + I.ncb * ((c->geo.nz + I.kz - 1) / I.kz);
+    I.nc = I.ncb * ((c->geo.nz + I.kz - 1) / I.kz);
     b->coff[i + 1] = b->coff[i] + I.nc;
   }
   b->na = b->aoff[n];
@@ -340,7 +340,7 @@ kx_status autotune(kx_batch* b) {
   const int saved_m = b->ctx[0]->m;
   const int steps = std::min(TUNE_STEPS, saved_m);   // never past the slot's m + 1 columns
   static const int TPB[] = {1, 2, 4, 8, 16};
-  static const int RPT[] = {1, 2, 4};
+  static const int RPT[] = {1, 2, 4, 8};
   cudaEvent_t e0, e1;
   KB_CUDA(b, cudaEventCreate(&e0), "event");
   if (cudaEventCreate(&e1) != cudaSuccess) {
@@ -485,7 +485,7 @@ kx_status kx_batch_get_info(const kx_batch* b, kx_batch_info* out) {
   out->sweep_tiles_per_block = b->tpb;
   out->apply_rounds_per_thread = b->rpt;
   out->sweep_blocks = b->ns;
-  out->apply_blocks = b->nc;
+  out->apply_blocks = (int)b->ctx.size() * SW_RED + b->nc;
   out->from_cache = b->from_cache;
   out->tune_ms = b->tune_ms;
   out->batched_launches = b->launches;

@@ -172,8 +172,8 @@ struct SwInst {
   int64_t ld;
   int ldh;
   int a0, na, s0, ns;
-  // the column-march apply launch of steps j >= 1: blocks [c0, c0 + nc),
-  // SW_RED reducers then ncb column blocks on each range of kz planes
+  // the column-march apply launch of steps j >= 1, past the reducers of all
+  // problems: blocks [c0, c0 + nc), ncb column blocks on each range of kz planes
   int c0, nc, ncb, kz;
 };
 

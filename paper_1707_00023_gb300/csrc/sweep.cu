@@ -901,23 +901,26 @@ __global__ void __launch_bounds__(NTHREADS, 2) k_sw_pass4s_batch(const SwInst* _
 }
 
 // Apply pass K_j (j >= 1) of every problem still running, the column march
-// of k_sw_apply_col: the problem's SW_RED reducer blocks, then its column
-// blocks, each over kz planes of NTHREADS quad columns.
+// of k_sw_apply_col: first the SW_RED reducer blocks of every problem, whose
+// finalisation is the launch's longest chain (behind the stencil blocks of
+// earlier problems it started a wave late), then each problem's column blocks,
+// each over kz planes of NTHREADS quad columns.
 __global__ void __launch_bounds__(NTHREADS, 2) k_sw_apply_col_batch(const SwInst* __restrict__ tab,
                                                                 const int* __restrict__ off, int n, int slot,
                                                                 int j, double btol) {
   __shared__ SwInst I;
-  const int i = inst_of(off, n, blockIdx.x);
+  const bool red = (int)blockIdx.x < n * SW_RED;
+  const int bid = red ? (int)blockIdx.x % SW_RED : (int)blockIdx.x - n * SW_RED;
+  const int i = red ? (int)blockIdx.x / SW_RED : inst_of(off, n, bid);
   load_inst(I, tab, i);
   pdl_wait();
   const Slot<float> s = I.s[slot];
   if (s.st->done || s.st->retired) return;
-  const int bid = (int)blockIdx.x - I.c0;
-  if (bid < SW_RED) {
+  if (red) {
     sw_reduce_fin<float>(s, I.w[slot], j, I.ldh, I.ns, btol, bid);
     return;
   }
-  const int b = bid - SW_RED;
+  const int b = bid - I.c0;
   const int zc = b / I.ncb;
   const int q = (b - zc * I.ncb) * NTHREADS + (int)threadIdx.x;
   const int k0 = zc * I.kz, k1 = min(I.g.nz, k0 + I.kz);
@@ -999,7 +1002,7 @@ kx_status sweep_arnoldi_batch(kx_ctx* c0, cudaStream_t st, const SwInst* tab, co
       // step 0's apply also takes the dots of its finalisation: the quad form
       e = j == m   ? launch_pdl(k_sw_last_batch, n, 0, st, tab, slot, m, bt)
           : j == 0 ? launch_pdl(k_sw_apply4_batch, na, 0, st, tab, aoff, n, slot, j, bt)
-                   : launch_pdl(k_sw_apply_col_batch, nc, 0, st, tab, coff, n, slot, j, bt);
+                   : launch_pdl(k_sw_apply_col_batch, n * SW_RED + nc, 0, st, tab, coff, n, slot, j, bt);
       if (e == cudaSuccess) ++*launches;
     }
     if (e != cudaSuccess) {
