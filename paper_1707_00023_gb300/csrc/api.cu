@@ -508,7 +508,10 @@ kx_status create_impl(const kx_desc* desc, const double* eps_cell, const uint8_t
   const int B = d.batch, m = c->m;
   const int nla = d.n[d.layer_axis];
   size_t bytes_V = (size_t)B * (m + 1) * c->ld * c->esize;
-  struct Alloc { void** p; size_t bytes; } allocs[] = {
+  // one device allocation for the whole workspace (thirty separate ones took
+  // longer than everything else in a small context's creation)
+  struct Alloc { void** p; size_t bytes; };
+  Alloc allocs[48] = {
       {(void**)&c->d_inv_eps, (size_t)g.ne * ncell * c->esize},
       {(void**)&c->d_sig2, (size_t)2 * nla * c->esize},
       {(void**)&c->d_eps_cell, (size_t)ncell * sizeof(double)},
@@ -536,19 +539,13 @@ kx_status create_impl(const kx_desc* desc, const double* eps_cell, const uint8_t
       {(void**)&c->d_swG, (size_t)B * (MMAX + 1) * (MMAX + 1) * sizeof(double)},
       {(void**)&c->d_swco, (size_t)B * sizeof(SwCoef)},
   };
-  for (auto& a : allocs) {
-    e = cudaMalloc(a.p, a.bytes);
-    if (e != cudaSuccess) {
-      cudaGetLastError();
-      krylov_expm_destroy(c);
-      return fail(nullptr, KX_ENOMEM, std::string("device allocation failed: ") + cudaGetErrorString(e));
-    }
-  }
+  int nalloc = 0;
+  while (allocs[nalloc].p) ++nalloc;
   if (d.max_checkpoints > 0) {
     const int P = gauss_points();
     c->adj_nq_max = 64 * P;
     const int64_t nE = (int64_t)g.ne * ncell;
-    Alloc adj[] = {
+    const Alloc adj[] = {
         {(void**)&c->d_ckpt, (size_t)d.max_checkpoints * c->ld * c->esize},
         {(void**)&c->d_adj_Q, (size_t)nE * sizeof(double)},
         {(void**)&c->d_adj_alpha, (size_t)c->adj_nq_max * (MMAX + 2) * sizeof(double)},
@@ -557,21 +554,7 @@ kx_status create_impl(const kx_desc* desc, const double* eps_cell, const uint8_t
         {(void**)&c->d_adj_M, (size_t)2 * (MMAX + 2) * MMAX * sizeof(float)},
         {(void**)&c->d_gauss, (size_t)2 * P * sizeof(double)},
     };
-    for (auto& a : adj) {
-      e = cudaMalloc(a.p, a.bytes);
-      if (e != cudaSuccess) {
-        cudaGetLastError();
-        krylov_expm_destroy(c);
-        return fail(nullptr, KX_ENOMEM, std::string("adjoint allocation failed: ") + cudaGetErrorString(e));
-      }
-    }
-    std::vector<double> gw(2 * P);
-    gauss_legendre01(P, gw.data(), gw.data() + P);
-    e = cudaMemcpy(c->d_gauss, gw.data(), sizeof(double) * 2 * P, cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) {
-      krylov_expm_destroy(c);
-      return fail(nullptr, KX_ECUDA, std::string("Gauss nodes upload failed: ") + cudaGetErrorString(e));
-    }
+    for (const Alloc& a : adj) allocs[nalloc++] = a;
   }
   if (d.rst_samples > 0) {
     int na = 0, nb = 0;
@@ -581,7 +564,7 @@ kx_status create_impl(const kx_desc* desc, const double* eps_cell, const uint8_t
       pmax = std::max<int64_t>(pmax, (int64_t)na * nb);
     }
     c->rst_plane_max = (int64_t)g.ne * pmax;
-    Alloc rst[] = {
+    const Alloc rst[] = {
         {(void**)&c->d_rst_b, (size_t)d.max_freqs * d.rst_samples * RST_P * sizeof(double)},
         {(void**)&c->d_rst_smp, (size_t)d.max_freqs * (d.rst_samples + 1) * 3 * sizeof(double)},
         {(void**)&c->d_rst_mats, (size_t)RST_MATS * sizeof(double)},
@@ -593,14 +576,32 @@ kx_status create_impl(const kx_desc* desc, const double* eps_cell, const uint8_t
         {(void**)&c->d_rst_state, (size_t)MAXF * sizeof(int)},
         {(void**)&c->d_rst_yp, (size_t)d.max_freqs * c->rst_plane_max * sizeof(double)},
     };
-    for (auto& a : rst) {
-      e = cudaMalloc(a.p, a.bytes);
-      if (e != cudaSuccess) {
-        cudaGetLastError();
-        krylov_expm_destroy(c);
-        return fail(nullptr, KX_ENOMEM, std::string("restart workspace allocation failed: ") + cudaGetErrorString(e));
-      }
+    for (const Alloc& a : rst) allocs[nalloc++] = a;
+  }
+  size_t total = 0;
+  for (int i = 0; i < nalloc; ++i) total += (allocs[i].bytes + 255) / 256 * 256;
+  e = cudaMalloc(&c->arena, total);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    krylov_expm_destroy(c);
+    return fail(nullptr, KX_ENOMEM, std::string("device allocation failed: ") + cudaGetErrorString(e));
+  }
+  size_t used = 0;
+  for (int i = 0; i < nalloc; ++i) {
+    *allocs[i].p = (char*)c->arena + used;
+    used += (allocs[i].bytes + 255) / 256 * 256;
+  }
+  if (d.max_checkpoints > 0) {
+    const int P = gauss_points();
+    std::vector<double> gw(2 * P);
+    gauss_legendre01(P, gw.data(), gw.data() + P);
+    e = cudaMemcpy(c->d_gauss, gw.data(), sizeof(double) * 2 * P, cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) {
+      krylov_expm_destroy(c);
+      return fail(nullptr, KX_ECUDA, std::string("Gauss nodes upload failed: ") + cudaGetErrorString(e));
     }
+  }
+  if (d.rst_samples > 0) {
     e = cudaStreamCreateWithFlags(&c->aux_stream, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_arnoldi, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_proj[0], cudaEventDisableTiming);
@@ -611,8 +612,8 @@ kx_status create_impl(const kx_desc* desc, const double* eps_cell, const uint8_t
       return fail(nullptr, KX_ECUDA, std::string("auxiliary stream creation failed: ") + cudaGetErrorString(e));
     }
   }
-  e = cudaMallocHost((void**)&c->h_state, (size_t)B * sizeof(SlotState));
-  if (e == cudaSuccess) e = cudaMallocHost((void**)&c->h_small, 256 * sizeof(double));
+  e = cudaMallocHost((void**)&c->h_small, 256 * sizeof(double) + (size_t)B * sizeof(SlotState));
+  if (e == cudaSuccess) c->h_state = reinterpret_cast<SlotState*>(c->h_small + 256);
   if (e != cudaSuccess) {
     cudaGetLastError();
     krylov_expm_destroy(c);
@@ -681,15 +682,7 @@ kx_status krylov_expm_create_mat(const kx_desc* desc, const uint8_t* d_mat_id, c
 kx_status krylov_expm_destroy(kx_ctx* c) {
   if (!c) return KX_OK;
   cudaStreamSynchronize(c->stream);
-  void* ptrs[] = {c->d_inv_eps, c->d_sig2, c->d_eps_cell, c->d_V, c->d_aug, c->d_H, c->d_scale,
-                  c->d_part, c->d_counter, c->d_u, c->d_state, c->d_rho, c->d_coef, c->d_coefd,
-                  c->d_omegas, c->d_small, c->d_tmp, c->d_tmp2, c->d_expm_ws, c->d_cd_ws, c->d_zre, c->d_zim,
-                  c->d_ckpt, c->d_adj_Q, c->d_adj_alpha, c->d_adj_omg, c->d_adj_cw, c->d_adj_M,
-                  c->d_gauss, c->d_rst_b, c->d_rst_smp, c->d_rst_mats, c->d_rst_fu, c->d_rst_cnt, c->d_rst_u, c->d_rst_res,
-                  c->d_rst_state, c->d_rst_yp, c->d_swT, c->d_swpart, c->d_swG, c->d_swco};
-  for (void* p : ptrs)
-    if (p) cudaFree(p);
-  if (c->h_state) cudaFreeHost(c->h_state);
+  if (c->arena) cudaFree(c->arena);
   if (c->h_small) cudaFreeHost(c->h_small);
   if (c->aux_stream) {
     cudaStreamSynchronize(c->aux_stream);
@@ -971,10 +964,10 @@ kx_status response_at_freqs(kx_ctx* c, const void* d_g, const double* omegas, in
 // `slot`, non-augmented).  By default the single-sweep form runs from
 // SWEEP_MIN_UNKNOWNS unknowns up.  Below, the two-pass process in one
 // cooperative launch is faster: a restart of 64 steps takes 1.7 against 2.8 ms
-// at 48^3 and 3.0 against 3.5 ms at 56^3 (1.05e6 unknowns); at 60^3 (1.3e6)
-// 4.3 against 3.6 ms, since two of its blocks then fill every SM and the
+// at 48^3 and 3.3 against 3.5 ms at 60^3 (1.3e6 unknowns); at 64^3 (1.57e6) 4.5
+// against 3.7 ms, since its blocks then fill every SM's registers and the
 // projected work beside it has to wait for the process to end.
-constexpr int64_t SWEEP_MIN_UNKNOWNS = 1200000;
+constexpr int64_t SWEEP_MIN_UNKNOWNS = 1400000;
 
 bool rst_uses_sweep(const kx_ctx* c) {
   if (c->d.arnoldi_form == KX_ARN_SWEEP) return true;

@@ -35,7 +35,7 @@ namespace kx {
 
 namespace {
 
-constexpr int CO_MAXT = 256;               // threads a block at most
+constexpr int CO_GROUPT = 256;             // threads a block may have by splitting the columns
 constexpr unsigned CO_WAIT_LIMIT = 1u << 21;   // polls of one barrier wait (about a second)
 
 // Barrier over the `blocks` blocks of a slot: the counter reaches `target`
@@ -145,7 +145,9 @@ struct QuadItem {
   using T = float;
   using V = float4;
   static constexpr int NC = 6;
-  static constexpr int DOTS = B, BATCH = B;   // columns in flight in the dots and the update (registers)
+  // columns in flight in the dots and the update, and threads a block: four
+  // with up to 255 registers, two with 128
+  static constexpr int DOTS = B, BATCH = B, MAXT = B == 4 ? 256 : 512;
   static __device__ __forceinline__ int64_t count(const Geo& g) { return g.ncell >> 2; }
   static __device__ __forceinline__ int64_t first(int64_t item) { return item << 2; }
   static __device__ __forceinline__ V zero() { return make_float4(0.f, 0.f, 0.f, 0.f); }
@@ -258,7 +260,7 @@ struct CellItem {
   using T = TT;
   using V = TT;
   static constexpr int NC = ncomp_of(DIM);
-  static constexpr int DOTS = sizeof(T) == 4 || NC < 6 ? 8 : 4, BATCH = DOTS;
+  static constexpr int DOTS = sizeof(T) == 4 || NC < 6 ? 8 : 4, BATCH = DOTS, MAXT = DIM == 3 ? 768 : 512;
   static __device__ __forceinline__ int64_t count(const Geo& g) { return g.ncell; }
   static __device__ __forceinline__ int64_t first(int64_t item) { return item; }
   static __device__ __forceinline__ V zero() { return T(0); }
@@ -297,12 +299,12 @@ struct CellItem {
 // columns in chunks of eight.  Loads of a chunk carry no conditions (a column
 // past the last reads the last again and is not used, an idle thread reads
 // item 0), so that they are all in flight together.
-template <typename P, int AUG, int MINB>
-__global__ void __launch_bounds__(CO_MAXT, MINB) k_coop(Geo g, SlotSet<typename P::T> ss, int m, int64_t ld,
-                                                       const typename P::T* __restrict__ ie,
-                                                       const typename P::T* __restrict__ sig2,
-                                                       const typename P::T* __restrict__ gsrc, int ldh, double btol,
-                                                       int nti) {
+template <typename P, int AUG>
+__global__ void __launch_bounds__(P::MAXT, 1) k_coop(Geo g, SlotSet<typename P::T> ss, int m, int64_t ld,
+                                                    const typename P::T* __restrict__ ie,
+                                                    const typename P::T* __restrict__ sig2,
+                                                    const typename P::T* __restrict__ gsrc, int ldh, double btol,
+                                                    int nti) {
   using T = typename P::T;
   using V = typename P::V;
   using SO = SumOf<T>;
@@ -310,8 +312,8 @@ __global__ void __launch_bounds__(CO_MAXT, MINB) k_coop(Geo g, SlotSet<typename 
   constexpr int NC = P::NC;
   extern __shared__ __align__(16) unsigned char co_dyn[];
   V* share = reinterpret_cast<V*>(co_dyn);            // groups x 2 NC x nti (more than one group)
-  __shared__ T acc[CO_MAXT / 32][MMAX + 2];           // a warp's dots; column MMAX + 1: ||w||^2
-  __shared__ S red[CO_MAXT / 32];
+  __shared__ T acc[P::MAXT / 32][MMAX + 2];           // a warp's dots; column MMAX + 1: ||w||^2
+  __shared__ S red[P::MAXT / 32];
   __shared__ double tot[MMAX + 8], scl[MMAX + 1], augs[2 * (MMAX + 1)];
   __shared__ T coef[MMAX + 8];
   __shared__ T sh_sj, sh_gco;                         // scale of v_j, factor of g
@@ -572,16 +574,17 @@ struct CoopPlan {
   size_t smem;
 };
 
-// Blocks for one slot's items: one a SM where 256 threads hold an SM's share,
-// else as few a SM as do; groups of warps that split the columns where the
-// items leave a block half empty or more.  slots = 0: they do not fit.
-CoopPlan coop_plan(const kx_ctx* c, const void* kernel, int64_t items, size_t vbytes, int ncomp) {
+// One block a SM, its threads an SM's share of the items (fewer, larger
+// blocks: half the partials and arrivals of two blocks a SM, 64^3 4.1 -> 3.8
+// ms); groups of warps that split the columns where that leaves CO_GROUPT
+// threads half used or less.  slots: how many slots' blocks are resident at
+// once (0: the items do not fit).
+CoopPlan coop_plan(const kx_ctx* c, const void* kernel, int64_t items, int maxt, size_t vbytes, int ncomp) {
   CoopPlan p{0, 0, 0, 0, 0};
   const int64_t per = (items + c->nsm - 1) / c->nsm;
-  const int64_t k = (per + CO_MAXT - 1) / CO_MAXT;
-  if (k > 8) return p;
-  p.nti = (int)(((per + k - 1) / k + 31) / 32 * 32);
-  p.groups = std::max(1, std::min(8, CO_MAXT / p.nti));
+  if (per > maxt) return p;
+  p.nti = (int)((per + 31) / 32 * 32);
+  p.groups = std::max(1, CO_GROUPT / p.nti);
   p.blocks = (int)((items + p.nti - 1) / p.nti);
   p.smem = p.groups > 1 ? (size_t)p.groups * 2 * ncomp * p.nti * vbytes : 0;
   int occ = 0;
@@ -589,20 +592,19 @@ CoopPlan coop_plan(const kx_ctx* c, const void* kernel, int64_t items, size_t vb
     cudaGetLastError();
     return p;
   }
-  if (p.blocks > c->ps) return p;
   p.slots = (int)((int64_t)occ * c->nsm / p.blocks);
   return p;
 }
 
-template <typename P, int AUG, int MINB>
+template <typename P, int AUG>
 kx_status coop_run(kx_ctx* c, int slot0, int ns, int m, const void* g_aug, int64_t items, bool* ran) {
   using T = typename P::T;
-  const void* fn = (const void*)k_coop<P, AUG, MINB>;
+  const void* fn = (const void*)k_coop<P, AUG>;
   static SmemOptIn attr{};
-  constexpr size_t SMEM_MOST = (size_t)2 * P::NC * CO_MAXT * sizeof(typename P::V);   // groups nti <= CO_MAXT
+  constexpr size_t SMEM_MOST = (size_t)2 * P::NC * CO_GROUPT * sizeof(typename P::V);   // groups nti <= CO_GROUPT
   const kx_status so = smem_opt_in(c, attr, fn, SMEM_MOST);
   if (so != KX_OK) return so;
-  const CoopPlan p = coop_plan(c, fn, items, sizeof(typename P::V), P::NC);
+  const CoopPlan p = coop_plan(c, fn, items, P::MAXT, sizeof(typename P::V), P::NC);
   *ran = p.slots > 0;
   if (!*ran) return KX_OK;
   for (int q = 0; q < ns; q += p.slots) {
@@ -619,7 +621,7 @@ kx_status coop_run(kx_ctx* c, int slot0, int ns, int m, const void* g_aug, int64
     cfg.numAttrs = 1;
     const double vb = (double)c->n * c->esize;
     time_begin(c);
-    cudaLaunchKernelEx(&cfg, k_coop<P, AUG, MINB>, c->geo, make_slotset<T>(c, slot0 + q), m, c->ld,
+    cudaLaunchKernelEx(&cfg, k_coop<P, AUG>, c->geo, make_slotset<T>(c, slot0 + q), m, c->ld,
                        (const T*)c->d_inv_eps, (const T*)c->d_sig2, (const T*)g_aug, c->m + 1,
                        sizeof(T) == 8 ? 1e-12 : 1e-6, p.nti);
     // algorithmic bytes: per step v_j, V_0 .. V_{j-1} twice, v_{j+1}, 1/eps (and g)
@@ -635,20 +637,18 @@ kx_status coop_model(kx_ctx* c, int slot0, int ns, int m, const void* g_aug, boo
   const Geo& g = c->geo;
   if (g.dim == 2 && g.pml) {
     if constexpr (TR) return KX_OK;   // the adjoint does not cover the PML model
-    else return coop_run<CellItem<T, 4, AUG, 0>, AUG, 2>(c, slot0, ns, m, g_aug, g.ncell, ran);
+    else return coop_run<CellItem<T, 4, AUG, 0>, AUG>(c, slot0, ns, m, g_aug, g.ncell, ran);
   }
-  if (g.dim == 2) return coop_run<CellItem<T, 2, AUG, TR>, AUG, 2>(c, slot0, ns, m, g_aug, g.ncell, ran);
+  if (g.dim == 2) return coop_run<CellItem<T, 2, AUG, TR>, AUG>(c, slot0, ns, m, g_aug, g.ncell, ran);
   if constexpr (sizeof(T) == 4) {
     // the quads need 16-byte aligned rows of every array they read
     if (g.nx % 4 == 0 && (uintptr_t)g_aug % 16 == 0 && g.ncell < ((int64_t)1 << 31)) {
-      // four columns in flight where one block a SM holds the grid and a
-      // thread may have 255 registers, two where it takes two blocks
-      if (g.ncell / 4 <= (int64_t)c->nsm * CO_MAXT)
-        return coop_run<QuadItem<AUG, TR, 4>, AUG, 1>(c, slot0, ns, m, g_aug, g.ncell / 4, ran);
-      return coop_run<QuadItem<AUG, TR, 2>, AUG, 2>(c, slot0, ns, m, g_aug, g.ncell / 4, ran);
+      if (g.ncell / 4 <= (int64_t)c->nsm * QuadItem<AUG, TR, 4>::MAXT)
+        return coop_run<QuadItem<AUG, TR, 4>, AUG>(c, slot0, ns, m, g_aug, g.ncell / 4, ran);
+      return coop_run<QuadItem<AUG, TR, 2>, AUG>(c, slot0, ns, m, g_aug, g.ncell / 4, ran);
     }
   }
-  return coop_run<CellItem<T, 3, AUG, TR>, AUG, 3>(c, slot0, ns, m, g_aug, g.ncell, ran);
+  return coop_run<CellItem<T, 3, AUG, TR>, AUG>(c, slot0, ns, m, g_aug, g.ncell, ran);
 }
 
 }  // namespace

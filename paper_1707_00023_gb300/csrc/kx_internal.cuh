@@ -196,6 +196,7 @@ struct kx_ctx {
   int nblk;         // blocks of the light bulk kernels
   int nsm;          // streaming multiprocessors
   int ps;           // partial-sum column stride = nsm * 8
+  void* arena = nullptr;    // the device workspace; every device pointer below lies in it
   void* d_inv_eps;
   void* d_sig2;
   double* d_eps_cell;
@@ -208,7 +209,7 @@ struct kx_ctx {
   unsigned* d_counter;
   double* d_u;
   kx::SlotState* d_state;
-  kx::SlotState* h_state;   // pinned host mirror
+  kx::SlotState* h_state;   // pinned host mirror (behind h_small)
   // stationary-solve workspace
   double* d_rho;            // 2 x MAXF complex residual coefficients
   float* d_coef;            // 2 x MAXF x MMAX update coefficients (FP32 path)
