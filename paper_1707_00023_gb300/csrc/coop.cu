@@ -13,9 +13,13 @@
 // so all reach the same coefficients and decisions; block 0 records them.
 //   phase A: w = A v_j, partial dots V_i . w (i <= j) and ||w||^2
 //   phase B: v_{j+1} = w - sum_i h_ij v_i (compensated in FP32), partial norm
-// A thread always reads the same part of every column, so the columns stay in
-// its SM's L1 and its die's L2; phase A takes them upwards and phase B
-// downwards, each starting on those the other ended on.
+// A thread always reads the same part of every column.  The first columns,
+// those read most often, are held in its SM's shared memory (the barrier's
+// acquire drops L1; m = 64, us with and without: 64^3 3758 and 3951 (4
+// columns), 48^3 1551 and 1725 (8), 36^3 1118 and 1184 (16), 2D 64^2 in double
+// precision 908 and 946 (all)); the others stay in its die's L2, phase A
+// taking them upwards and phase B downwards, each starting on those the other
+// ended on.
 // Where a block's items fill less than half of it, its warps split the
 // columns as well (CS groups; the groups' shares of the update are added
 // through shared memory).
@@ -36,6 +40,10 @@ namespace kx {
 namespace {
 
 constexpr int CO_GROUPT = 256;             // threads a block may have by splitting the columns
+// Shared memory a block may take: past 196 KB the next carve-out leaves 28 KB
+// of L1, too few for the loads in flight (64^3 with 4 columns held 3758 us,
+// with 5 4430; 45^3 cells with 8 1585, with 16 1737).
+constexpr size_t CO_SMEM = 195 * 1024;
 constexpr unsigned CO_WAIT_LIMIT = 1u << 21;   // polls of one barrier wait (about a second)
 
 // Barrier over the `blocks` blocks of a slot: the counter reaches `target`
@@ -147,7 +155,7 @@ struct QuadItem {
   static constexpr int NC = 6;
   // columns in flight in the dots and the update, and threads a block: four
   // with up to 255 registers, two with 128
-  static constexpr int DOTS = B, BATCH = B, MAXT = B == 4 ? 256 : 512;
+  static constexpr int BATCH = B, MAXT = B == 4 ? 256 : 512;
   static __device__ __forceinline__ int64_t count(const Geo& g) { return g.ncell >> 2; }
   static __device__ __forceinline__ int64_t first(int64_t item) { return item << 2; }
   static __device__ __forceinline__ V zero() { return make_float4(0.f, 0.f, 0.f, 0.f); }
@@ -260,7 +268,7 @@ struct CellItem {
   using T = TT;
   using V = TT;
   static constexpr int NC = ncomp_of(DIM);
-  static constexpr int DOTS = sizeof(T) == 4 || NC < 6 ? 8 : 4, BATCH = DOTS, MAXT = DIM == 3 ? 768 : 512;
+  static constexpr int BATCH = sizeof(T) == 4 || NC < 6 ? 8 : 4, MAXT = DIM == 3 ? 768 : 512;
   static __device__ __forceinline__ int64_t count(const Geo& g) { return g.ncell; }
   static __device__ __forceinline__ int64_t first(int64_t item) { return item; }
   static __device__ __forceinline__ V zero() { return T(0); }
@@ -304,7 +312,7 @@ __global__ void __launch_bounds__(P::MAXT, 1) k_coop(Geo g, SlotSet<typename P::
                                                     const typename P::T* __restrict__ ie,
                                                     const typename P::T* __restrict__ sig2,
                                                     const typename P::T* __restrict__ gsrc, int ldh, double btol,
-                                                    int nti) {
+                                                    int nti, int kc) {
   using T = typename P::T;
   using V = typename P::V;
   using SO = SumOf<T>;
@@ -312,6 +320,7 @@ __global__ void __launch_bounds__(P::MAXT, 1) k_coop(Geo g, SlotSet<typename P::
   constexpr int NC = P::NC;
   extern __shared__ __align__(16) unsigned char co_dyn[];
   V* share = reinterpret_cast<V*>(co_dyn);            // groups x 2 NC x nti (more than one group)
+  V* keep = share + ((int)blockDim.x > nti ? 2 * NC * blockDim.x : 0);   // columns 0 .. kc-1: kc x NC x nti
   __shared__ T acc[P::MAXT / 32][MMAX + 2];           // a warp's dots; column MMAX + 1: ||w||^2
   __shared__ S red[P::MAXT / 32];
   __shared__ double tot[MMAX + 8], scl[MMAX + 1], augs[2 * (MMAX + 1)];
@@ -348,6 +357,29 @@ __global__ void __launch_bounds__(P::MAXT, 1) k_coop(Geo g, SlotSet<typename P::
       st->done = 1;
     }
   };
+  if (grp == 0 && kc > 0) {
+#pragma unroll
+    for (int c = 0; c < NC; ++c) keep[c * nti + it] = act ? P::load(Vc + c * nc) : P::zero();
+  }
+  // this thread's part of columns col .. col + N - 1 (past j: column j)
+  auto batch = [&](auto& v, int col, int j) {
+    constexpr int N = sizeof(v) / sizeof(v[0]);
+    if (min(col + N - 1, j) < kc) {
+#pragma unroll
+      for (int t = 0; t < N; ++t) {
+        const V* vc = keep + min(col + t, j) * NC * nti + it;
+#pragma unroll
+        for (int c = 0; c < NC; ++c) v[t][c] = vc[c * nti];
+      }
+    } else {
+#pragma unroll
+      for (int t = 0; t < N; ++t) {
+        const T* vc = Vc + (int64_t)min(col + t, j) * ld;
+#pragma unroll
+        for (int c = 0; c < NC; ++c) v[t][c] = P::load(vc + c * nc);
+      }
+    }
+  };
   __syncthreads();
   for (int j = 0; j < m; ++j) {
     const int ncol = j + 1;
@@ -364,16 +396,11 @@ __global__ void __launch_bounds__(P::MAXT, 1) k_coop(Geo g, SlotSet<typename P::
     for (int c0 = 8 * grp; c0 < ncol; c0 += 8 * ngrp) {
       T p[8];
 #pragma unroll
-      for (int h = 0; h < 8; h += P::DOTS) {
-        V v[P::DOTS][NC];
+      for (int h = 0; h < 8; h += P::BATCH) {
+        V v[P::BATCH][NC];
+        batch(v, c0 + h, j);
 #pragma unroll
-        for (int t = 0; t < P::DOTS; ++t) {
-          const T* vc = Vc + (int64_t)min(c0 + h + t, j) * ld;
-#pragma unroll
-          for (int c = 0; c < NC; ++c) v[t][c] = P::load(vc + c * nc);
-        }
-#pragma unroll
-        for (int t = 0; t < P::DOTS; ++t) {
+        for (int t = 0; t < P::BATCH; ++t) {
           p[h + t] = T(0);
 #pragma unroll
           for (int c = 0; c < NC; ++c) p[h + t] += P::dot(v[t][c], o[c]);
@@ -479,12 +506,7 @@ __global__ void __launch_bounds__(P::MAXT, 1) k_coop(Geo g, SlotSet<typename P::
 #pragma unroll
         for (int h = 8 - P::BATCH; h >= 0; h -= P::BATCH) {
           V v[P::BATCH][NC];
-#pragma unroll
-          for (int t = 0; t < P::BATCH; ++t) {
-            const T* vc = Vc + (int64_t)min(c0 + h + t, j) * ld;
-#pragma unroll
-            for (int c = 0; c < NC; ++c) v[t][c] = P::load(vc + c * nc);
-          }
+          batch(v, c0 + h, j);
 #pragma unroll
           for (int t = P::BATCH - 1; t >= 0; --t)
 #pragma unroll
@@ -493,6 +515,8 @@ __global__ void __launch_bounds__(P::MAXT, 1) k_coop(Geo g, SlotSet<typename P::
       }
     }
     T* out = Vc + (int64_t)(j + 1) * ld;
+    V* kout = keep + (j + 1) * NC * nti + it;
+    const bool held = j + 1 < kc;
     T t2 = T(0);
     if (ngrp == 1) {
       if (act) {
@@ -503,6 +527,10 @@ __global__ void __launch_bounds__(P::MAXT, 1) k_coop(Geo g, SlotSet<typename P::
           t2 += P::dot(o[c], o[c]);
         }
       }
+      if (held) {
+#pragma unroll
+        for (int c = 0; c < NC; ++c) kout[c * nti] = act ? o[c] : P::zero();
+      }
     } else {
       // the groups' shares added, a component a group
 #pragma unroll
@@ -511,6 +539,8 @@ __global__ void __launch_bounds__(P::MAXT, 1) k_coop(Geo g, SlotSet<typename P::
         share[((size_t)grp * 2 * NC + NC + c) * nti + it] = lo[c];
       }
       __syncthreads();
+      if (held && !act)
+        for (int c = grp; c < NC; c += ngrp) kout[c * nti] = P::zero();
       if (act)
         for (int c = grp; c < NC; c += ngrp) {
           V h = share[(size_t)c * nti + it], l = share[(size_t)(NC + c) * nti + it];
@@ -518,6 +548,7 @@ __global__ void __launch_bounds__(P::MAXT, 1) k_coop(Geo g, SlotSet<typename P::
             P::join(h, l, share[((size_t)q * 2 * NC + c) * nti + it], share[((size_t)q * 2 * NC + NC + c) * nti + it]);
           h = P::fold(h, l);
           P::store(out + c * nc, h);
+          if (held) kout[c * nti] = h;
           t2 += P::dot(h, h);
         }
     }
@@ -571,6 +602,7 @@ __global__ void __launch_bounds__(P::MAXT, 1) k_coop(Geo g, SlotSet<typename P::
 
 struct CoopPlan {
   int nti, groups, blocks, slots;   // slots: how many fit one launch
+  int keep;                         // columns held in shared memory
   size_t smem;
 };
 
@@ -578,21 +610,38 @@ struct CoopPlan {
 // blocks: half the partials and arrivals of two blocks a SM, 64^3 4.1 -> 3.8
 // ms); groups of warps that split the columns where that leaves CO_GROUPT
 // threads half used or less.  slots: how many slots' blocks are resident at
-// once (0: the items do not fit).
-CoopPlan coop_plan(const kx_ctx* c, const void* kernel, int64_t items, int maxt, size_t vbytes, int ncomp) {
-  CoopPlan p{0, 0, 0, 0, 0};
+// once (0: the items do not fit).  The first columns are held in whole
+// batches in `room` bytes a block, as far as no slot is put off for them.
+CoopPlan coop_plan(const kx_ctx* c, const void* kernel, int64_t items, int ns, int m, int maxt, size_t vbytes, int ncomp,
+                   int batch, size_t room) {
+  CoopPlan p{0, 0, 0, 0, 0, 0};
   const int64_t per = (items + c->nsm - 1) / c->nsm;
   if (per > maxt) return p;
   p.nti = (int)((per + 31) / 32 * 32);
   p.groups = std::max(1, CO_GROUPT / p.nti);
   p.blocks = (int)((items + p.nti - 1) / p.nti);
-  p.smem = p.groups > 1 ? (size_t)p.groups * 2 * ncomp * p.nti * vbytes : 0;
-  int occ = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, p.nti * p.groups, p.smem) != cudaSuccess) {
-    cudaGetLastError();
-    return p;
+  const size_t part = (size_t)ncomp * p.nti * vbytes;   // a block's part of a column
+  p.smem = p.groups > 1 ? p.groups * 2 * part : 0;
+  auto slots = [&](size_t smem) {
+    int occ = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, p.nti * p.groups, smem) != cudaSuccess) {
+      cudaGetLastError();
+      return 0;
+    }
+    return (int)((int64_t)occ * c->nsm / p.blocks);
+  };
+  p.slots = slots(p.smem);
+  const int need = std::min(ns, p.slots);
+  int k = room > p.smem ? (int)std::min<size_t>(m, (room - p.smem) / part) : 0;
+  if (k < m) k -= k % batch;
+  for (; p.slots > 0 && k > 0; k = (k - 1) / batch * batch) {
+    const int fit = slots(p.smem + k * part);
+    if (fit < need) continue;
+    p.keep = k;
+    p.smem += k * part;
+    p.slots = fit;
+    break;
   }
-  p.slots = (int)((int64_t)occ * c->nsm / p.blocks);
   return p;
 }
 
@@ -601,10 +650,12 @@ kx_status coop_run(kx_ctx* c, int slot0, int ns, int m, const void* g_aug, int64
   using T = typename P::T;
   const void* fn = (const void*)k_coop<P, AUG>;
   static SmemOptIn attr{};
-  constexpr size_t SMEM_MOST = (size_t)2 * P::NC * CO_GROUPT * sizeof(typename P::V);   // groups nti <= CO_GROUPT
-  const kx_status so = smem_opt_in(c, attr, fn, SMEM_MOST);
+  // CO_SMEM less the kernel's own arrays (the largest: the warps' dots)
+  constexpr size_t ROOM = CO_SMEM - (P::MAXT / 32 * (MMAX + 2) + MMAX) * sizeof(T) - 5 * 1024;
+  static_assert(ROOM >= (size_t)2 * P::NC * CO_GROUPT * sizeof(typename P::V), "the groups' shares");
+  const kx_status so = smem_opt_in(c, attr, fn, ROOM);
   if (so != KX_OK) return so;
-  const CoopPlan p = coop_plan(c, fn, items, P::MAXT, sizeof(typename P::V), P::NC);
+  const CoopPlan p = coop_plan(c, fn, items, ns, m, P::MAXT, sizeof(typename P::V), P::NC, P::BATCH, ROOM);
   *ran = p.slots > 0;
   if (!*ran) return KX_OK;
   for (int q = 0; q < ns; q += p.slots) {
@@ -623,7 +674,7 @@ kx_status coop_run(kx_ctx* c, int slot0, int ns, int m, const void* g_aug, int64
     time_begin(c);
     cudaLaunchKernelEx(&cfg, k_coop<P, AUG>, c->geo, make_slotset<T>(c, slot0 + q), m, c->ld,
                        (const T*)c->d_inv_eps, (const T*)c->d_sig2, (const T*)g_aug, c->m + 1,
-                       sizeof(T) == 8 ? 1e-12 : 1e-6, p.nti);
+                       sizeof(T) == 8 ? 1e-12 : 1e-6, p.nti, p.keep);
     // algorithmic bytes: per step v_j, V_0 .. V_{j-1} twice, v_{j+1}, 1/eps (and g)
     time_end(c, KX_K_PASS_A,
              nq * m * ((m + 2.0) * vb + (double)c->geo.ne * c->geo.ncell * c->esize + (g_aug ? vb : 0.0)));
