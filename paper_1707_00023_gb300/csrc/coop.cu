@@ -148,14 +148,13 @@ __device__ __forceinline__ float4 mul4(const float4& a, const float4& b) {
 
 // Items of four x-cells, 3D FP32 lossy layer (nx % 4 == 0): stencil_quad32's
 // operations, field loads past L1.
-template <int AUG, int TR, int B>
+template <int AUG, int TR, int MT>
 struct QuadItem {
   using T = float;
   using V = float4;
   static constexpr int NC = 6;
-  // columns in flight in the dots and the update, and threads a block: four
-  // with up to 255 registers, two with 128
-  static constexpr int BATCH = B, MAXT = B == 4 ? 256 : 512;
+  // columns in flight in the dots and the update (what the registers hold)
+  static constexpr int BATCH = MT <= 384 ? 4 : 2, MAXT = MT;
   static __device__ __forceinline__ int64_t count(const Geo& g) { return g.ncell >> 2; }
   static __device__ __forceinline__ int64_t first(int64_t item) { return item << 2; }
   static __device__ __forceinline__ V zero() { return make_float4(0.f, 0.f, 0.f, 0.f); }
@@ -694,9 +693,16 @@ kx_status coop_model(kx_ctx* c, int slot0, int ns, int m, const void* g_aug, boo
   if constexpr (sizeof(T) == 4) {
     // the quads need 16-byte aligned rows of every array they read
     if (g.nx % 4 == 0 && (uintptr_t)g_aug % 16 == 0 && g.ncell < ((int64_t)1 << 31)) {
-      if (g.ncell / 4 <= (int64_t)c->nsm * QuadItem<AUG, TR, 4>::MAXT)
-        return coop_run<QuadItem<AUG, TR, 4>, AUG>(c, slot0, ns, m, g_aug, g.ncell / 4, ran);
-      return coop_run<QuadItem<AUG, TR, 2>, AUG>(c, slot0, ns, m, g_aug, g.ncell / 4, ran);
+      // By the threads a block needs: up to 256 have 232 registers and four
+      // columns in flight, up to 384 168 registers and still four (56^3, 64
+      // steps: 2380 us, with two columns 2655; 60^3 2980 and 3132), above that
+      // 128 registers and two (64^3: compiled for 448 threads 3655 us, for 512
+      // 3748).
+      const int64_t quads = g.ncell / 4, sm = c->nsm;
+      if (quads <= sm * 256) return coop_run<QuadItem<AUG, TR, 256>, AUG>(c, slot0, ns, m, g_aug, quads, ran);
+      if (quads <= sm * 384) return coop_run<QuadItem<AUG, TR, 384>, AUG>(c, slot0, ns, m, g_aug, quads, ran);
+      if (quads <= sm * 448) return coop_run<QuadItem<AUG, TR, 448>, AUG>(c, slot0, ns, m, g_aug, quads, ran);
+      return coop_run<QuadItem<AUG, TR, 512>, AUG>(c, slot0, ns, m, g_aug, quads, ran);
     }
   }
   return coop_run<CellItem<T, 3, AUG, TR>, AUG>(c, slot0, ns, m, g_aug, g.ncell, ran);

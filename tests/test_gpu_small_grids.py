@@ -41,6 +41,9 @@ GRIDS = {
     "quads_two_groups": S.Grid(3, (36, 35, 37), (P, P, C), 2, 4, 1.0),
     "quads_one_group": S.Grid(3, (52, 49, 50), (P, P, C), 2, 4, 1.0),
     "quads_past_256_a_block": S.Grid(3, (56, 55, 54), (P, P, C), 2, 4, 1.0),
+    "quads_past_384_a_block": S.Grid(3, (64, 61, 62), (P, P, C), 2, 4, 1.0),
+    "quads_past_448_a_block": S.Grid(3, (68, 63, 64), (P, P, C), 2, 4, 1.0),
+    "quads_too_many": S.Grid(3, (68, 70, 66), (P, P, C), 2, 4, 1.0),
     "cells_few": S.Grid(3, (5, 3, 4), (C, P, C), 2, 1, 1.0),
     "cells_layer_x": S.Grid(3, (21, 18, 23), (C, P, P), 0, 3, 1.0),
     "cells_most": S.Grid(3, (47, 49, 50), (P, P, C), 2, 4, 1.0),
