@@ -964,7 +964,7 @@ kx_status response_at_freqs(kx_ctx* c, const void* d_g, const double* omegas, in
 // `slot`, non-augmented).  By default the single-sweep form runs from
 // SWEEP_MIN_UNKNOWNS unknowns up.  Below, the two-pass process in one
 // cooperative launch is faster: a restart of 64 steps takes 1.7 against 2.8 ms
-// at 48^3 and 3.3 against 3.5 ms at 60^3 (1.3e6 unknowns); at 64^3 (1.57e6) 4.5
+// at 48^3 and 3.2 against 3.5 ms at 60^3 (1.3e6 unknowns); at 64^3 (1.57e6) 4.1
 // against 3.7 ms, since its blocks then fill every SM's registers and the
 // projected work beside it has to wait for the process to end.
 constexpr int64_t SWEEP_MIN_UNKNOWNS = 1400000;
