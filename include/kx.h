@@ -348,7 +348,7 @@ kx_status response_at_freqs_multi(kx_ctx* const* ctxs, int nctx, const void* con
  * Creation allocates a small table and chooses how each launch is split
  * (an autotuner times an Arnoldi process of min(12, krylov_dim) steps of the whole batch for each
  * candidate granularity -- sweep tiles per block 1..16, apply work per thread
- * r = 1, 2, 4 (step 0: r quad rounds; later steps: 2 r planes a thread in the
+ * r = 1, 2, 4, 8 (step 0: r quad rounds; later steps: 2 r planes a thread in the
  * column march) -- and keeps the fastest; the choice is cached per size
  * class, the multiset of the problems' grids, for the rest of the process).
  * The timing runs overwrite basis slot 0 of every context.  The batched
