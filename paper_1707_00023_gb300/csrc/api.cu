@@ -578,8 +578,16 @@ kx_status create_impl(const kx_desc* desc, const double* eps_cell, const uint8_t
     };
     for (const Alloc& a : rst) allocs[nalloc++] = a;
   }
+  // arrays of a mebibyte or more start on 2 MB boundaries, as allocations of
+  // their own would: with the basis at a 256-byte offset the two passes of a
+  // 96^3 process read it 2 % slower (pass B 7.40 against 7.24 ms, pass A 8.16
+  // against 8.06; 72^3 3.32 against 3.27 and 4.12 against 4.09)
+  auto place = [](size_t at, size_t bytes) {
+    const size_t a = bytes >= ((size_t)1 << 20) ? (size_t)1 << 21 : 256;
+    return (at + a - 1) / a * a;
+  };
   size_t total = 0;
-  for (int i = 0; i < nalloc; ++i) total += (allocs[i].bytes + 255) / 256 * 256;
+  for (int i = 0; i < nalloc; ++i) total = place(total, allocs[i].bytes) + allocs[i].bytes;
   e = cudaMalloc(&c->arena, total);
   if (e != cudaSuccess) {
     cudaGetLastError();
@@ -588,8 +596,9 @@ kx_status create_impl(const kx_desc* desc, const double* eps_cell, const uint8_t
   }
   size_t used = 0;
   for (int i = 0; i < nalloc; ++i) {
+    used = place(used, allocs[i].bytes);
     *allocs[i].p = (char*)c->arena + used;
-    used += (allocs[i].bytes + 255) / 256 * 256;
+    used += allocs[i].bytes;
   }
   if (d.max_checkpoints > 0) {
     const int P = gauss_points();
