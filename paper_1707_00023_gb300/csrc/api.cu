@@ -93,10 +93,11 @@ SlotState fresh_state() {
 kx_status arnoldi_steps(kx_ctx* c, int slot0, int ns, int m, const void* g_aug, int transpose = 0) {
   bool ran = false;
   KX_TRY(coop_arnoldi(c, slot0, ns, m, g_aug, transpose, &ran));
+  const bool fold = transpose || ran || pass_a_finalises(c, ns, g_aug);
   for (int j = 0; j < m && !ran; ++j) {
     KX_TRY(transpose ? launch_pass_a_tr(c, slot0, ns, j) : launch_pass_a(c, slot0, ns, j, g_aug));
-    // the next pass A finalises it; the last step needs the kernel
-    KX_TRY(launch_pass_b(c, slot0, ns, j, j == m - 1));
+    // the next pass A finalises it, or the kernel (always the last step)
+    KX_TRY(launch_pass_b(c, slot0, ns, j, !fold || j == m - 1));
   }
   c->stats.arnoldi_steps += (int64_t)m * ns;
   c->stats.matvecs += (int64_t)m * ns;

@@ -273,12 +273,14 @@ kx_status launch_setup_material(kx_ctx* c);
 kx_status launch_expand_materials(kx_ctx* c, const uint8_t* d_id, const double* d_table, int n_mat, int* d_bad);
 kx_status launch_apply(kx_ctx* c, const void* v, void* w, int transpose);
 kx_status launch_pass_a(kx_ctx* c, int slot0, int ns, int j, const void* g_aug);
+// whether that launch of step j finalises step j - 1's pass B
+bool pass_a_finalises(kx_ctx* c, int ns, const void* g_aug);
 // pass A with the transposed operator A^T
 kx_status launch_pass_a_tr(kx_ctx* c, int slot0, int ns, int j);
 // pass A reading the per-cell permittivity directly (no 1/eps table)
 kx_status launch_pass_a_cells(kx_ctx* c, int slot, int j, const double* d_eps_cell);
 // pass B of step j; finalize = 1 launches its finalisation kernel, otherwise
-// the next step's pass A finalises it
+// the next step's pass A finalises it (pass_a_finalises)
 kx_status launch_pass_b(kx_ctx* c, int slot0, int ns, int j, int finalize);
 int pass_b_grid(kx_ctx* c);
 

@@ -87,6 +87,11 @@ __device__ __forceinline__ T warp_sum8(T* p, int lane) {
 }
 __device__ __forceinline__ int column_of_lane8(int lane) { return lane >> 2; }
 
+// a^2 + b^2 of the phase entries, rounded alike in every kernel that adds it
+// (as are the entries themselves: which kernel finalises a step depends on how
+// many slots run, and the bits must not).
+__device__ __forceinline__ double phase_norm2(double a, double b) { return fma(a, a, __dmul_rn(b, b)); }
+
 // Finalisation of step j-1's pass B at the start of step j's pass A: every
 // block sums the same nbb partials in the same order, so all reach the same
 // h_{j,j-1} and the same breakdown decision; block 0 (rec) records them.
@@ -132,9 +137,9 @@ __device__ __forceinline__ bool fin_prev_b(const Slot<T>& s, int j, int ldh, int
         sb += red[2][w];
       }
       const double W = s.st->omega, sp = s.scale[j - 1];
-      a = -W * sp * s.aug[2 * (j - 1) + 1] - sa;
-      b = W * sp * s.aug[2 * (j - 1)] - sb;
-      tot += a * a + b * b;
+      a = __dmul_rn(-W * sp, s.aug[2 * (j - 1) + 1]) - sa;
+      b = __dmul_rn(W * sp, s.aug[2 * (j - 1)]) - sb;
+      tot += phase_norm2(a, b);
     }
     const double h = sqrt(tot);
     int stp = 0;

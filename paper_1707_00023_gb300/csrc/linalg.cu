@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(NTHREADS) k_fin_b(SlotSet<T> ss, int j, int ld
       const double a = s.aug[2 * (j + 1)] - sa, b = s.aug[2 * (j + 1) + 1] - sb;
       s.aug[2 * (j + 1)] = a;
       s.aug[2 * (j + 1) + 1] = b;
-      tot += a * a + b * b;
+      tot += phase_norm2(a, b);
     }
     const double h = sqrt(tot);
     s.H[(j + 1) + (int64_t)j * ldh] = h;

@@ -309,7 +309,8 @@ __global__ void __launch_bounds__(NTHREADS) k_pass_a(Geo g, SlotSet<T> ss, int j
 // registers.  Its index arithmetic is 32-bit (ncell < 2^31).
 
 // The body of pass A in its quad form; two kernels below instantiate it.
-template <int AUG>
+// SPLIT: the launch may split the columns between groups of blocks.
+template <int AUG, bool SPLIT>
 __device__ __forceinline__ void pass_a4_body(Geo g, SlotSet<float> ss, int j, int64_t ld,
                                              const float* __restrict__ ie,
                                              const float* __restrict__ sig2,
@@ -322,7 +323,7 @@ __device__ __forceinline__ void pass_a4_body(Geo g, SlotSet<float> ss, int j, in
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int q = threadIdx.x; q < NWARPS * (MMAX + 2); q += blockDim.x) (&acc[0][0])[q] = 0.0;
   __syncthreads();
-  const int grp = blockIdx.z;
+  const int grp = SPLIT ? blockIdx.z : 0;
   double sj, aj = 0.0;
   if (nbb > 0) {
     if (!fin_prev_b<AUG>(s, j, ldh, nbb, btol, blockIdx.x == 0 && grp == 0, &sj, &aj)) return;
@@ -336,7 +337,7 @@ __device__ __forceinline__ void pass_a4_body(Geo g, SlotSet<float> ss, int j, in
   float gco = 0.f;
   if (AUG) gco = (float)(-(sj * aj) / s.st->eta);
   const int ncol = j + 1;
-  const int per = col_group(ncol, gridDim.z), cbeg = grp * per, cend = min(ncol, cbeg + per);
+  const int per = SPLIT ? col_group(ncol, gridDim.z) : ncol, cbeg = grp * per, cend = min(ncol, cbeg + per);
   const int64_t nc = g.ncell;
   const int64_t nq = nc >> 2;
   for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < nq; base += (int64_t)gridDim.x * blockDim.x) {
@@ -463,19 +464,20 @@ template <int AUG>
 __global__ void __launch_bounds__(NTHREADS) k_pass_a4(Geo g, SlotSet<float> ss, int j, int64_t ld,
                                                      const float* __restrict__ ie, const float* __restrict__ sig2,
                                                      const float* __restrict__ gsrc, int ldh, int nbb, double btol) {
-  pass_a4_body<AUG>(g, ss, j, ld, ie, sig2, gsrc, ldh, nbb, btol);
+  pass_a4_body<AUG, true>(g, ss, j, ld, ie, sig2, gsrc, ldh, nbb, btol);
 }
 
 // Three resident blocks per SM (at most 85 registers a thread), for work
 // that fills the GPU: at 128^3 the pass ran at 80 % of the measured copy
-// bandwidth with two blocks and at 94 % with three.
+// bandwidth with two blocks and at 94 % with three.  Such a launch has no
+// column groups.
 template <int AUG>
 __global__ void __launch_bounds__(NTHREADS, 3) k_pass_a4_dense(Geo g, SlotSet<float> ss, int j, int64_t ld,
                                                               const float* __restrict__ ie,
                                                               const float* __restrict__ sig2,
                                                               const float* __restrict__ gsrc, int ldh, int nbb,
                                                               double btol) {
-  pass_a4_body<AUG>(g, ss, j, ld, ie, sig2, gsrc, ldh, nbb, btol);
+  pass_a4_body<AUG, false>(g, ss, j, ld, ie, sig2, gsrc, ldh, nbb, btol);
 }
 
 // ---------------------------------------------------------------------------
@@ -542,6 +544,54 @@ static int col_groups(int ncol, int64_t blocks, int cap) {
   return (ncol + per - 1) / per;   // no empty group
 }
 
+// How pass A of ns slots runs: its kernel (quad form, and that in its
+// three-block form), blocks a slot, resident blocks, and whether each launch
+// finalises the step before's pass B itself.  A non-augmented process always
+// does.  An augmented one does where one wave of blocks holds the launch: every
+// block then also forms the phase entries' update, microseconds of
+// double-precision work before its first load, hidden by no other block (72^3,
+// 64 steps in every block against the separate kernel, pass A: 4 slots 12.1
+// against 10.6 ms, 8 slots 21.6 against 19.1; one slot 13 us a step saved in
+// pass B's class and 5 lost in pass A's).
+struct PassAPlan {
+  bool vec4, dense, fold;
+  int nb, gr;
+};
+
+template <typename T>
+static PassAPlan pass_a_plan(kx_ctx* c, int ns, const void* gaug) {
+  const Geo& g = c->geo;
+  PassAPlan p;
+  // the quad kernel needs 16-byte aligned rows of every array it reads
+  p.vec4 = sizeof(T) == 4 && g.dim == 3 && (g.nx % 4) == 0 && ((uintptr_t)gaug % 16) == 0 &&
+           g.ncell < ((int64_t)1 << 31);
+  const int64_t items = p.vec4 ? g.ncell / 4 : g.ncell;
+  const int64_t rounds = (items + NTHREADS - 1) / NTHREADS;
+  // the quad kernel in its three-block form when the launch's work (all its
+  // slots) exceeds what two resident blocks per SM cover
+  p.dense = p.vec4 && rounds * ns > 2 * (int64_t)c->nsm;
+  static std::atomic<int> grid[5][2];
+  const int kind = p.vec4 ? (p.dense ? 4 : 2) : (g.pml ? 3 : (g.dim == 3));
+  std::atomic<int>& gr = grid[kind][gaug != nullptr];
+  if (!gr) {
+    const void* fn;
+    if (p.vec4 && p.dense) fn = gaug ? (const void*)k_pass_a4_dense<1> : (const void*)k_pass_a4_dense<0>;
+    else if (p.vec4) fn = gaug ? (const void*)k_pass_a4<1> : (const void*)k_pass_a4<0>;
+    else if (g.dim == 2 && g.pml) fn = gaug ? (const void*)k_pass_a<T, 4, 1, TableMat<T>> : (const void*)k_pass_a<T, 4, 0, TableMat<T>>;
+    else if (g.dim == 2) fn = gaug ? (const void*)k_pass_a<T, 2, 1, TableMat<T>> : (const void*)k_pass_a<T, 2, 0, TableMat<T>>;
+    else fn = gaug ? (const void*)k_pass_a<T, 3, 1, TableMat<T>> : (const void*)k_pass_a<T, 3, 0, TableMat<T>>;
+    gr = persistent_grid(c, fn, 1 << 30, 0);
+  }
+  p.gr = gr.load();
+  p.nb = reserve_grid(c, (int)std::min<int64_t>(std::min<int64_t>(rounds, p.gr), c->ps), p.gr);
+  p.fold = !gaug || (int64_t)p.nb * ns <= p.gr;
+  return p;
+}
+
+bool pass_a_finalises(kx_ctx* c, int ns, const void* g_aug) {
+  return c->d.precision == KX_FP64 ? pass_a_plan<double>(c, ns, g_aug).fold : pass_a_plan<float>(c, ns, g_aug).fold;
+}
+
 template <typename T>
 static kx_status pass_a_t(kx_ctx* c, int slot, int ns, int j, const void* gaug) {
   const Geo& g = c->geo;
@@ -551,30 +601,11 @@ static kx_status pass_a_t(kx_ctx* c, int slot, int ns, int j, const void* gaug) 
   const T* sg = (const T*)c->d_sig2;
   const T* gs = (const T*)gaug;
   const int ldh = m + 1;
-  // the quad kernel needs 16-byte aligned rows of every array it reads
-  const bool vec4 = sizeof(T) == 4 && g.dim == 3 && (g.nx % 4) == 0 &&
-                    ((uintptr_t)gaug % 16) == 0 && g.ncell < ((int64_t)1 << 31);
-  const int64_t items = vec4 ? g.ncell / 4 : g.ncell;
-  const int64_t rounds = (items + NTHREADS - 1) / NTHREADS;
-  // the quad kernel in its three-block form when the launch's work (all its
-  // slots) exceeds what two resident blocks per SM cover
-  const bool dense = vec4 && rounds * ns > 2 * (int64_t)c->nsm;
-  static std::atomic<int> grid[5][2];
-  const int kind = vec4 ? (dense ? 4 : 2) : (g.pml ? 3 : (g.dim == 3));
-  std::atomic<int>& gr = grid[kind][gaug != nullptr];
-  if (!gr) {
-    const void* fn;
-    if (vec4 && dense) fn = gaug ? (const void*)k_pass_a4_dense<1> : (const void*)k_pass_a4_dense<0>;
-    else if (vec4) fn = gaug ? (const void*)k_pass_a4<1> : (const void*)k_pass_a4<0>;
-    else if (g.dim == 2 && g.pml) fn = gaug ? (const void*)k_pass_a<T, 4, 1, TableMat<T>> : (const void*)k_pass_a<T, 4, 0, TableMat<T>>;
-    else if (g.dim == 2) fn = gaug ? (const void*)k_pass_a<T, 2, 1, TableMat<T>> : (const void*)k_pass_a<T, 2, 0, TableMat<T>>;
-    else fn = gaug ? (const void*)k_pass_a<T, 3, 1, TableMat<T>> : (const void*)k_pass_a<T, 3, 0, TableMat<T>>;
-    gr = persistent_grid(c, fn, 1 << 30, 0);
-  }
-  const int nb = reserve_grid(c, (int)std::min<int64_t>(std::min<int64_t>(rounds, gr.load()), c->ps), gr.load());
-  const dim3 grd(nb, ns, col_groups(j + 1, (int64_t)nb * ns, gr.load()));
-  // step j-1's pass B is finalised here
-  const int nbb = j >= 1 ? pass_b_grid(c) : 0;
+  const PassAPlan p = pass_a_plan<T>(c, ns, gaug);
+  const int nb = p.nb;
+  const bool vec4 = p.vec4, dense = p.dense;
+  const dim3 grd(nb, ns, dense ? 1 : col_groups(j + 1, (int64_t)nb * ns, p.gr));
+  const int nbb = j >= 1 && p.fold ? pass_b_grid(c) : 0;
   const double bt = btol_of<T>();
   if (vec4) {
     SlotSet<float> sf = make_slotset<float>(c, slot);
