@@ -68,19 +68,19 @@ __global__ void __launch_bounds__(NTHREADS) k_pass_b(SlotSet<T> ss, int j, int64
          q += (int64_t)gridDim.x * blockDim.x) {
       float4 x = reinterpret_cast<const float4*>(wf)[q];
       float4 lo = make_float4(0.f, 0.f, 0.f, 0.f);
+      // the columns from the last to the first: the pass starts on those that
+      // pass A ended on
+      const int last = ncol - 1;
       int col = 0;
-      // eight independent column loads in flight per thread (the columns
-      // downwards, to start on those pass A ended on, are no gain once a
-      // thread takes several quads: 72^3 3.44 against 3.27 ms a process, 80^3
-      // 4.73 against 4.35, 96^3 7.50 against 7.24)
+      // eight independent column loads in flight per thread
       for (; col + 8 <= ncol; col += 8) {
         float4 v[8];
 #pragma unroll
-        for (int t = 0; t < 8; ++t) v[t] = Vf[(int64_t)(col + t) * ldv + q];
+        for (int t = 0; t < 8; ++t) v[t] = Vf[(int64_t)(last - (col + t)) * ldv + q];
 #pragma unroll
-        for (int t = 0; t < 8; ++t) sub_fma4(x, lo, -(float)coef[col + t], v[t]);
+        for (int t = 0; t < 8; ++t) sub_fma4(x, lo, -(float)coef[last - (col + t)], v[t]);
       }
-      for (; col < ncol; ++col) sub_fma4(x, lo, -(float)coef[col], Vf[(int64_t)col * ldv + q]);
+      for (; col < ncol; ++col) sub_fma4(x, lo, -(float)coef[last - col], Vf[(int64_t)(last - col) * ldv + q]);
       x = make_float4(x.x + lo.x, x.y + lo.y, x.z + lo.z, x.w + lo.w);
       reinterpret_cast<float4*>(wf)[q] = x;
       nrm += (double)vdot(x);
@@ -189,7 +189,11 @@ __global__ void __launch_bounds__(NTHREADS) k_fin_b(SlotSet<T> ss, int j, int ld
 }
 
 // Grid of pass B: a persistent grid (shrunk for resident side CTAs); the
-// next pass A needs it to finalise pass B itself.
+// next pass A needs it to finalise pass B itself.  In single precision six
+// blocks a SM (all that are resident), or five where those leave a twentieth
+// less of their waves empty: 64 steps with five and six, 64^3 2.60 and 2.26 ms,
+// 76^3 3.85 and 3.61, 96^3 7.17 and 7.00, but 68^3 2.81 and 2.96, 80^3 4.30 and
+// 4.36.  By the grid alone: the order of the norm's sums follows it.
 int pass_b_grid(kx_ctx* c) {
   static std::atomic<int> grid[2];
   const int fp64 = c->d.precision == KX_FP64;
@@ -197,8 +201,13 @@ int pass_b_grid(kx_ctx* c) {
     grid[fp64] = persistent_grid(c, fp64 ? (const void*)k_pass_b<double> : (const void*)k_pass_b<float>,
                                  1 << 30, 0);
   const int64_t rounds = (c->n / (fp64 ? 2 : 4) + NTHREADS - 1) / NTHREADS;
-  return reserve_grid(c, (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(rounds, grid[fp64].load()), c->ps)),
-                      grid[fp64].load());
+  int64_t cap = grid[fp64].load();
+  const int64_t less = cap - c->nsm;
+  if (!fp64 && less >= 5 * (int64_t)c->nsm) {
+    const int64_t w0 = (rounds + cap - 1) / cap, w1 = (rounds + less - 1) / less;
+    if (21 * w1 * less <= 20 * w0 * cap) cap = less;
+  }
+  return reserve_grid(c, (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(rounds, cap), c->ps)), (int)cap);
 }
 
 // Algorithmic bytes of pass B at step j: read w and V_0..V_j (j+2 vectors),
