@@ -1026,8 +1026,9 @@ kx_status response_restart_dim(kx_ctx* c, const void* d_g, const double* omegas,
   // millisecond of kernels) runs beside the first steps of the next process;
   // in the later steps the single-sweep launches take every SM slot (128^3
   // with the reservation for 32, 16, 8, 4 steps: 516, 513.5, 513, 515 ms).  The
-  // two-pass form keeps it for every step.  A fixed rule, so every mode has
-  // the same grids and bits.
+  // two-pass launches keep it for every step.  The cooperative process makes
+  // none: where its blocks leave no room, the projected work waits for its end
+  // or it for theirs.  A fixed rule, so every mode has the same grids and bits.
   c->side_steps = (c->m + 7) / 8;
   // the Arnoldi chain of this method runs with programmatic dependent launch
   c->pdl = 1;
