@@ -421,7 +421,9 @@ kx_status launch_axpy(kx_ctx* c, double a, const void* x, void* y) {
 
 // ---------------------------------------------------------------------------
 // Export the orthonormal basis: dV[:, i] = scale_i V_i (i <= m_done, and the
-// column past a lucky breakdown is zero), one column a blockIdx.y.  A copy,
+// column past a lucky breakdown is zero), one column a blockIdx.y; dV may be
+// the basis itself (ld = n), each value read by the thread that then writes it.
+// A copy,
 // bound by memory: in single precision the scale is a float pair and the
 // product rounded once from hi v (exact with its FMA residual) + lo v; through
 // double precision (two conversions and a product a value) it took 588 us at
@@ -432,12 +434,12 @@ __device__ __forceinline__ float scaled(float hi, float lo, float v) {
 }
 
 template <typename T>
-__global__ void __launch_bounds__(NTHREADS) k_export(Slot<T> s, T* __restrict__ dV, int64_t n, int64_t ld, int vec) {
+__global__ void __launch_bounds__(NTHREADS) k_export(Slot<T> s, T* dV, int64_t n, int64_t ld, int vec) {
   const int col = blockIdx.y, md = s.st->m_done;
   const bool on = col < md || (col == md && !s.st->done);
   const double sc = on ? s.scale[col] : 0.0;
-  const T* __restrict__ src = s.V + (int64_t)col * ld;
-  T* __restrict__ dst = dV + (int64_t)col * n;
+  const T* src = s.V + (int64_t)col * ld;
+  T* dst = dV + (int64_t)col * n;
   const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, nt = (int64_t)gridDim.x * blockDim.x;
   if constexpr (sizeof(T) == 4) {
     const float hi = (float)sc, lo = (float)(sc - (double)hi);
