@@ -423,14 +423,24 @@ kx_status launch_axpy(kx_ctx* c, double a, const void* x, void* y) {
 // Export the orthonormal basis: dV[:, i] = scale_i V_i (i <= m_done, and the
 // column past a lucky breakdown is zero), one column a blockIdx.y; dV may be
 // the basis itself (ld = n), each value read by the thread that then writes it.
-// A copy,
-// bound by memory: in single precision the scale is a float pair and the
-// product rounded once from hi v (exact with its FMA residual) + lo v; through
-// double precision (two conversions and a product a value) it took 588 us at
-// 64^3, 65 columns, 3.4 times as long as its bytes.
-__device__ __forceinline__ float scaled(float hi, float lo, float v) {
-  const float p = hi * v;
-  return p + fmaf(lo, v, fmaf(hi, v, -p));
+// A copy, bound by memory; in single precision through double precision (two
+// conversions and a product a value) it took 588 us at 64^3, 65 columns, 3.4
+// times as long as its bytes.
+//
+// The float nearest to sc v, without those: with sc as a float pair and the
+// FMA's residual, p + c is within 2^-45 |p| of the double product, so where
+// moving it by 2^-44 |p| either way rounds to the same float that is the result;
+// the few others (one in 2^19) and products near the denormals take the double
+// product.
+// Not inlined: predicated into the loop it took the double pipe's time for
+// every value (64^3 620 us; so 174).
+__device__ __noinline__ float scaled_double(double sc, float v) { return (float)(sc * (double)v); }
+__device__ __forceinline__ float scaled(double sc, float hi, float lo, float v) {
+  const float p = hi * v, c = fmaf(lo, v, fmaf(hi, v, -p)), d = fabsf(p) * 0x1p-44f;
+  const float r = p + (c + d);
+  if (v == 0.f) return p;
+  if (r == p + (c - d) && fabsf(p) > 1e-30f) return r;
+  return scaled_double(sc, v);
 }
 
 template <typename T>
@@ -448,11 +458,11 @@ __global__ void __launch_bounds__(NTHREADS) k_export(Slot<T> s, T* dV, int64_t n
       float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
       if (on) {
         const float4 v = reinterpret_cast<const float4*>(src)[q];
-        r = make_float4(scaled(hi, lo, v.x), scaled(hi, lo, v.y), scaled(hi, lo, v.z), scaled(hi, lo, v.w));
+        r = make_float4(scaled(sc, hi, lo, v.x), scaled(sc, hi, lo, v.y), scaled(sc, hi, lo, v.z), scaled(sc, hi, lo, v.w));
       }
       reinterpret_cast<float4*>(dst)[q] = r;
     }
-    for (int64_t e = 4 * nq + t0; e < n; e += nt) dst[e] = on ? scaled(hi, lo, src[e]) : 0.f;
+    for (int64_t e = 4 * nq + t0; e < n; e += nt) dst[e] = on ? scaled(sc, hi, lo, src[e]) : 0.f;
   } else {
     (void)vec;
     for (int64_t e = t0; e < n; e += nt) dst[e] = on ? sc * src[e] : 0.0;
