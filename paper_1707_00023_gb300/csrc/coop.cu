@@ -75,6 +75,11 @@ __device__ __forceinline__ bool grid_barrier(unsigned* cnt, unsigned target) {
 // (Knuth's TwoSum at every addition, 2^-48 of the terms), because a chain of
 // double-precision additions is what these reductions would wait for on this
 // GPU (tens of clocks each; every block sums up to 65 columns of partials).
+// The terms are a warp's float sums, good to 2^-24, so the five bits fewer than
+// in double precision are not seen: fields of the plain method against a
+// double-precision context, geometric means over 48 media of 24^3 to 64^3,
+// 3.61e-7 with the per-step launches (which sum in double precision), 3.61e-7
+// with pairs, 3.63e-7 with triples (2^-72; 45^3 1585 -> 1880 us a process).
 // Double precision: double.
 struct Pair {
   float h, l;
@@ -84,6 +89,13 @@ __device__ __forceinline__ Pair add(Pair a, Pair b) {
   r.h = a.h + b.h;
   const float z = r.h - a.h;
   r.l = (a.l + b.l) + ((a.h - (r.h - z)) + (b.h - z));
+  return r;
+}
+__device__ __forceinline__ Pair add(Pair a, float b) {
+  Pair r;
+  r.h = a.h + b;
+  const float z = r.h - a.h;
+  r.l = a.l + ((a.h - (r.h - z)) + (b - z));
   return r;
 }
 __device__ __forceinline__ double add(double a, double b) { return a + b; }
@@ -420,7 +432,7 @@ __global__ void __launch_bounds__(P::MAXT, 1) k_coop(Geo g, SlotSet<typename P::
     for (int col = tid; col <= ncol; col += blockDim.x) {
       const int w0 = col < ncol ? ((col >> 3) % ngrp) * wpg : 0, src = col < ncol ? col : MMAX + 1;
       S t = SO::of(acc[w0][src]);
-      for (int w = 1; w < wpg; ++w) t = add(t, SO::of(acc[w0 + w][src]));
+      for (int w = 1; w < wpg; ++w) t = add(t, acc[w0 + w][src]);
       SO::put(s.part + (int64_t)col * s.ps + b, t);
     }
     bars += G;
@@ -516,14 +528,16 @@ __global__ void __launch_bounds__(P::MAXT, 1) k_coop(Geo g, SlotSet<typename P::
     T* out = Vc + (int64_t)(j + 1) * ld;
     V* kout = keep + (j + 1) * NC * nti + it;
     const bool held = j + 1 < kc;
-    T t2 = T(0);
+    // the squares of a quad of values (or of one) summed in the working
+    // precision, as in pass B, no more
+    S t2 = SO::of(T(0));
     if (ngrp == 1) {
       if (act) {
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
           o[c] = P::fold(o[c], lo[c]);
           P::store(out + c * nc, o[c]);
-          t2 += P::dot(o[c], o[c]);
+          t2 = add(t2, P::dot(o[c], o[c]));
         }
       }
       if (held) {
@@ -548,10 +562,10 @@ __global__ void __launch_bounds__(P::MAXT, 1) k_coop(Geo g, SlotSet<typename P::
           h = P::fold(h, l);
           P::store(out + c * nc, h);
           if (held) kout[c * nti] = h;
-          t2 += P::dot(h, h);
+          t2 = add(t2, P::dot(h, h));
         }
     }
-    const S n2 = warp_total(SO::of(t2));
+    const S n2 = warp_total(t2);
     if (lane == 0) red[warp] = n2;
     __syncthreads();
     if (tid == 0) {
