@@ -148,9 +148,9 @@ class Context:
     problems, since torch hands out streams from a small pool).
     ``rst_samples``: time samples per frequency held for the restart-in-
     dimension method (``method="rstdim"``; 0 leaves it unavailable).
-    ``arnoldi``: "default" (single sweep for restart in dimension on grids of
-    1.4e6 unknowns or more, two passes elsewhere), "twopass" or "sweep" (also
-    for ``arnoldi()``).
+    ``arnoldi``: "default" (single sweep for restart in dimension in single
+    precision on grids of 1.4e6 unknowns or more, two passes elsewhere),
+    "twopass" or "sweep" (also for ``arnoldi()``).
     ``mat_id`` / ``eps_table``: instead of ``eps_cell`` (pass None), a CUDA
     uint8 tensor of material ids per cell and the materials' permittivities
     (``krylov_expm_create_mat``).

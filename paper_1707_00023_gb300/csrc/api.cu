@@ -971,18 +971,22 @@ kx_status response_at_freqs(kx_ctx* c, const void* d_g, const double* omegas, in
 }
 
 // The Arnoldi process of one restart in Krylov dimension (basis slot
-// `slot`, non-augmented).  By default the single-sweep form runs from
-// SWEEP_MIN_UNKNOWNS unknowns up.  Below, the two-pass process in one
+// `slot`, non-augmented).  By default, in single precision, the single-sweep
+// form runs from SWEEP_MIN_UNKNOWNS unknowns up.  Below, the two-pass process in one
 // cooperative launch is faster: a restart of 64 steps takes 1.7 against 2.8 ms
 // at 48^3 and 3.2 against 3.5 ms at 60^3 (1.3e6 unknowns); at 64^3 (1.57e6) 4.1
 // against 3.7 ms, since its blocks then fill every SM's registers and the
-// projected work beside it has to wait for the process to end.
+// projected work beside it has to wait for the process to end.  In double
+// precision the two passes at every size: the sweep reads the basis once but has
+// as many products and more sums, and that pipe is what bounds it (4 frequencies,
+// T = 40 or 20, two passes against the sweep: 64^3 53 and 119 ms, 80^3 61 and
+// 155, 96^3 100 and 254; 2D 704^2 38 and 102).
 constexpr int64_t SWEEP_MIN_UNKNOWNS = 1400000;
 
 bool rst_uses_sweep(const kx_ctx* c) {
   if (c->d.arnoldi_form == KX_ARN_SWEEP) return true;
   if (c->d.arnoldi_form == KX_ARN_TWOPASS) return false;
-  return c->n >= SWEEP_MIN_UNKNOWNS;
+  return c->d.precision == KX_FP32 && c->n >= SWEEP_MIN_UNKNOWNS;
 }
 
 kx_status rst_arnoldi(kx_ctx* c, int slot) {
