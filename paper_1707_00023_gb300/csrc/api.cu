@@ -89,10 +89,11 @@ SlotState fresh_state() {
 // m Arnoldi steps (two-pass form, of A^T when transpose) on slots
 // [slot0, slot0 + ns) from their (normalised) column 0: one cooperative launch
 // where the grid fits the resident threads, else all slots in the same
-// launches, three a step.
-kx_status arnoldi_steps(kx_ctx* c, int slot0, int ns, int m, const void* g_aug, int transpose = 0) {
+// launches, three a step.  want: the slots that calls of this kind may run
+// (the route does not depend on how many of them still do).
+kx_status arnoldi_steps(kx_ctx* c, int slot0, int ns, int want, int m, const void* g_aug, int transpose = 0) {
   bool ran = false;
-  KX_TRY(coop_arnoldi(c, slot0, ns, m, g_aug, transpose, &ran));
+  KX_TRY(coop_arnoldi(c, slot0, ns, want, m, g_aug, transpose, &ran));
   const bool fold = transpose || ran || pass_a_finalises(c, ns, g_aug);
   for (int j = 0; j < m && !ran; ++j) {
     KX_TRY(transpose ? launch_pass_a_tr(c, slot0, ns, j) : launch_pass_a(c, slot0, ns, j, g_aug));
@@ -116,8 +117,8 @@ kx_status read_states(kx_ctx* c, int slot0, int ns) {
 // every later kernel skips it.
 // One sub-step's launches: m Arnoldi steps, the projected step control, the
 // combination.
-kx_status substep_launches(kx_ctx* c, int slot0, int ns, const void* g_aug) {
-  KX_TRY(arnoldi_steps(c, slot0, ns, c->m, g_aug));
+kx_status substep_launches(kx_ctx* c, int slot0, int ns, int want, const void* g_aug) {
+  KX_TRY(arnoldi_steps(c, slot0, ns, want, c->m, g_aug));
   KX_TRY(launch_substep_control(c, slot0, ns));
   return launch_combine(c, slot0, ns);
 }
@@ -132,14 +133,14 @@ struct SubstepGraph {
   }
 };
 
-kx_status capture_substep(kx_ctx* c, int slot0, int ns, const void* g_aug, SubstepGraph* out) {
+kx_status capture_substep(kx_ctx* c, int slot0, int ns, int want, const void* g_aug, SubstepGraph* out) {
   const kx_stats saved = c->stats;   // capturing executes nothing: restore the counters
   const int64_t before = c->stats.kernel_launches;
   if (cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
     cudaGetLastError();
     return KX_ECUDA;
   }
-  const kx_status st = substep_launches(c, slot0, ns, g_aug);
+  const kx_status st = substep_launches(c, slot0, ns, want, g_aug);
   cudaGraph_t graph = nullptr;
   const cudaError_t e = cudaStreamEndCapture(c->stream, &graph);
   if (st != KX_OK || e != cudaSuccess || !graph) {
@@ -168,7 +169,7 @@ kx_status capture_substep(kx_ctx* c, int slot0, int ns, const void* g_aug, Subst
 // every sub-step; queued sub-steps past the end cost only empty launches.
 constexpr int SUBSTEP_BATCH = 8;
 
-kx_status time_loop(kx_ctx* c, int slot0, int ns, const void* g_aug, double* err_est) {
+kx_status time_loop(kx_ctx* c, int slot0, int ns, int want, const void* g_aug, double* err_est) {
   KX_TRY(launch_norm_init(c, slot0, ns));
   const int max_sub = 20000;
   bool all = false;
@@ -180,14 +181,14 @@ kx_status time_loop(kx_ctx* c, int slot0, int ns, const void* g_aug, double* err
   int queued = 0, batch = 1;
   while (queued < max_sub && !all) {
     for (int b = 0; b < batch && queued < max_sub; ++b, ++queued) {
-      if (use_graph && queued >= 1 && !graph.exec && capture_substep(c, slot0, ns, g_aug, &graph) != KX_OK)
+      if (use_graph && queued >= 1 && !graph.exec && capture_substep(c, slot0, ns, want, g_aug, &graph) != KX_OK)
         use_graph = false;
       if (use_graph && graph.exec) {
         KX_CUDA(c, cudaGraphLaunch(graph.exec, c->stream), "sub-step graph launch");
         c->stats.kernel_launches += graph.launches;
       } else {
         const kx_stats before = c->stats;
-        KX_TRY(substep_launches(c, slot0, ns, g_aug));
+        KX_TRY(substep_launches(c, slot0, ns, want, g_aug));
         // Arnoldi work is counted from the accepted sub-steps below
         c->stats.arnoldi_steps = before.arnoldi_steps;
         c->stats.matvecs = before.matvecs;
@@ -280,7 +281,7 @@ kx_status stationary_core(kx_ctx* c, const void* d_g, const double* omegas, int 
   double best = INFINITY;
   int since_best = 0;
   for (int cyc = 0; matvecs < max_matvecs; ++cyc) {
-    KX_TRY(arnoldi_steps(c, slot, 1, c->m, nullptr));
+    KX_TRY(arnoldi_steps(c, slot, 1, 1, c->m, nullptr));
     KX_TRY(read_state(c, slot, &st));
     if (st.status) return fail(c, (kx_status)st.status, "non-finite value in the Arnoldi process");
     const int md = st.m_done;
@@ -340,7 +341,7 @@ kx_status slots_time_loop(kx_ctx* c, int ns, bool aug, const void* d_g, const do
           "state upload");
   KX_TRY(sync(c));
   std::vector<double> e(ns, 0.0);
-  KX_TRY(time_loop(c, 0, ns, aug ? d_g : nullptr, e.data()));
+  KX_TRY(time_loop(c, 0, ns, c->d.batch, aug ? d_g : nullptr, e.data()));
   for (int q = 0; q < ns; ++q)
     if (on[q]) err[q] += e[q];
   return KX_OK;
@@ -735,7 +736,7 @@ kx_status arnoldi(kx_ctx* c, const void* d_v0, int m, void* d_V, double* H, doub
   KX_TRY(read_state(c, slot, &st));
   if (!(st.beta > 0.0) || !std::isfinite(st.beta)) return fail(c, KX_ENONFINITE, "v0 is zero or non-finite");
   if (c->d.arnoldi_form == KX_ARN_SWEEP) KX_TRY(sweep_arnoldi(c, slot, m));
-  else KX_TRY(arnoldi_steps(c, slot, 1, m, nullptr));
+  else KX_TRY(arnoldi_steps(c, slot, 1, 1, m, nullptr));
   KX_TRY(read_state(c, slot, &st));
   if (st.status) return fail(c, (kx_status)st.status, "non-finite value in the Arnoldi process");
   *beta = st.beta;
@@ -815,7 +816,7 @@ kx_status expm_action(kx_ctx* c, const void* d_y0, double T, double rtol, void* 
   s.rtol = rtol;
   s.tol_mode = 0;
   KX_TRY(upload_state(c, slot, s));
-  KX_TRY(time_loop(c, slot, 1, nullptr, err_est));
+  KX_TRY(time_loop(c, slot, 1, 1, nullptr, err_est));
   KX_CUDA(c, cudaMemcpyAsync(d_y, slot_col(c, slot, 0), c->n * c->esize, cudaMemcpyDeviceToDevice,
                              c->stream), "copy y");
   return sync(c);
@@ -908,7 +909,7 @@ kx_status response_at_freqs(kx_ctx* c, const void* d_g, const double* omegas, in
       KX_CUDA(c, cudaMemcpyAsync(c->d_state, c->h_state, sizeof(SlotState) * ns, cudaMemcpyHostToDevice,
                                  c->stream), "state upload");
       KX_TRY(sync(c));
-      KX_TRY(time_loop(c, 0, ns, nullptr, err_est ? err_est + f0 : nullptr));
+      KX_TRY(time_loop(c, 0, ns, c->d.batch, nullptr, err_est ? err_est + f0 : nullptr));
       // yhat_f(T) = yhat_{f-1}(T) + w_f(T)  (Fig. alg:spl1 steps 5-6); the
       // previous wave's last transient waits in d_tmp
       for (int q = 0; q < ns; ++q) {
@@ -950,7 +951,7 @@ kx_status response_at_freqs(kx_ctx* c, const void* d_g, const double* omegas, in
     KX_CUDA(c, cudaMemcpyAsync(c->d_state, c->h_state, sizeof(SlotState) * ns, cudaMemcpyHostToDevice,
                                c->stream), "state upload");
     KX_TRY(sync(c));
-    KX_TRY(time_loop(c, 0, ns, method == KX_SPLIT ? nullptr : d_g, err_est ? err_est + f0 : nullptr));
+    KX_TRY(time_loop(c, 0, ns, c->d.batch, method == KX_SPLIT ? nullptr : d_g, err_est ? err_est + f0 : nullptr));
     for (int q = 0; q < ns; ++q) {
       const int f = f0 + q;
       void* Ep = d_E_plane ? (char*)d_E_plane + (int64_t)f * nE * np * c->esize : nullptr;
@@ -991,7 +992,7 @@ bool rst_uses_sweep(const kx_ctx* c) {
 
 kx_status rst_arnoldi(kx_ctx* c, int slot) {
   if (rst_uses_sweep(c)) return sweep_arnoldi(c, slot, c->m);
-  return arnoldi_steps(c, slot, 1, c->m, nullptr);
+  return arnoldi_steps(c, slot, 1, 1, c->m, nullptr);
 }
 
 kx_status response_restart_dim(kx_ctx* c, const void* d_g, const double* omegas, int nfreq, double T,
@@ -1246,7 +1247,7 @@ kx_status adjoint_response_grad(kx_ctx* c, const void* d_g, const double* omegas
       KX_CUDA(c, cudaMemcpyAsync((char*)c->d_ckpt + tk.size() * c->ld * c->esize, slot_col(c, 0, 0), vbytes,
                                  cudaMemcpyDeviceToDevice, c->stream), "checkpoint");
       tk.push_back(tnow);
-      KX_TRY(arnoldi_steps(c, 0, 1, c->m, d_g));
+      KX_TRY(arnoldi_steps(c, 0, 1, 1, c->m, d_g));
       KX_TRY(launch_substep_control(c, 0, 1));
       KX_TRY(launch_combine(c, 0, 1));
       KX_TRY(read_states(c, 0, 1));
@@ -1278,8 +1279,8 @@ kx_status adjoint_response_grad(kx_ctx* c, const void* d_g, const double* omegas
                                  c->stream), "state upload");
       KX_TRY(sync(c));
       KX_TRY(launch_norm_init(c, 0, 2));
-      KX_TRY(arnoldi_steps(c, 0, 1, c->m, d_g));
-      KX_TRY(arnoldi_steps(c, 1, 1, c->m, nullptr, 1));
+      KX_TRY(arnoldi_steps(c, 0, 1, 1, c->m, d_g));
+      KX_TRY(arnoldi_steps(c, 1, 1, 1, c->m, nullptr, 1));
       KX_TRY(read_states(c, 0, 2));
       if (c->h_state[0].status || c->h_state[1].status)
         return fail(c, KX_ENONFINITE, "adjoint backward: Krylov process failed");

@@ -619,20 +619,13 @@ struct CoopPlan {
   size_t smem;
 };
 
-// One block a SM, its threads an SM's share of the items (fewer, larger
-// blocks: half the partials and arrivals of two blocks a SM, 64^3 4.1 -> 3.8
-// ms); groups of warps that split the columns where that leaves CO_GROUPT
-// threads half used or less.  slots: how many slots' blocks are resident at
-// once (0: the items do not fit).  The first columns are held in whole
-// batches in `room` bytes a block, as far as no slot is put off for them.
-CoopPlan coop_plan(const kx_ctx* c, const void* kernel, int64_t items, int ns, int m, int maxt, size_t vbytes, int ncomp,
+// Blocks of nti items each; groups of warps that split the columns where that
+// leaves CO_GROUPT threads half used or less.  slots: how many slots' blocks
+// are resident at once.  The first columns are held in whole batches in `room`
+// bytes a block, as far as none of `want` slots is put off for them.
+CoopPlan coop_plan(const kx_ctx* c, const void* kernel, int64_t items, int nti, int want, int m, size_t vbytes, int ncomp,
                    int batch, size_t room) {
-  CoopPlan p{0, 0, 0, 0, 0, 0};
-  const int64_t per = (items + c->nsm - 1) / c->nsm;
-  if (per > maxt) return p;
-  p.nti = (int)((per + 31) / 32 * 32);
-  p.groups = std::max(1, CO_GROUPT / p.nti);
-  p.blocks = (int)((items + p.nti - 1) / p.nti);
+  CoopPlan p{nti, std::max(1, CO_GROUPT / nti), (int)((items + nti - 1) / nti), 0, 0, 0};
   const size_t part = (size_t)ncomp * p.nti * vbytes;   // a block's part of a column
   p.smem = p.groups > 1 ? p.groups * 2 * part : 0;
   auto slots = [&](size_t smem) {
@@ -644,7 +637,7 @@ CoopPlan coop_plan(const kx_ctx* c, const void* kernel, int64_t items, int ns, i
     return (int)((int64_t)occ * c->nsm / p.blocks);
   };
   p.slots = slots(p.smem);
-  const int need = std::min(ns, p.slots);
+  const int need = std::min(want, p.slots);
   int k = room > p.smem ? (int)std::min<size_t>(m, (room - p.smem) / part) : 0;
   if (k < m) k -= k % batch;
   for (; p.slots > 0 && k > 0; k = (k - 1) / batch * batch) {
@@ -658,17 +651,65 @@ CoopPlan coop_plan(const kx_ctx* c, const void* kernel, int64_t items, int ns, i
   return p;
 }
 
+// Estimated microseconds of one step of `want` slots, on GB300: fixed cost of
+// the barriers and sums, a value's products and update with m / 2 columns by
+// the threads of an SM (its items, in as many blocks as share it), and the
+// basis' two reads where that is more.  Measured (m = 64, items a block: us):
+// 24^3 32: 12.9, 128: 15.3, 256: 20.4, 512: 32; double precision 24^3 96: 27.7,
+// 256: 46.7; 2D 64^2 in double precision (m = 30) 32: 15.2, 256: 21.9.
+double coop_us(const kx_ctx* c, const CoopPlan& p, int want, int m, int values) {
+  const bool f64 = c->esize == 8;
+  const int used = std::min(want, p.slots);
+  const int share = (int)(((int64_t)used * p.blocks + c->nsm - 1) / c->nsm);
+  const double work = (f64 ? 14.0 : 10.0) + (f64 ? 7e-4 : 5.6e-5) * share * p.nti * values * (0.5 * m);
+  const double mem = (double)used * c->n * c->esize * m / 7.5e6;
+  return std::max(work, mem) * ((want + p.slots - 1) / p.slots);
+}
+// The same with the per-step launches, which serve every slot: 24^3 1 slot 26,
+// 32 slots 148; 36^3 31 and 466; 2D 128^2 in double precision 32 slots 233.
+double steps_us(const kx_ctx* c, int want, int m) {
+  return 22.0 + (c->esize == 8 ? 5.5e-6 : 1.54e-6) * want * c->n * (0.5 * m);
+}
+
 template <typename P, int AUG>
-kx_status coop_run(kx_ctx* c, int slot0, int ns, int m, const void* g_aug, int64_t items, bool* ran) {
+kx_status coop_run(kx_ctx* c, int slot0, int ns, int want, int m, const void* g_aug, int64_t items, bool* ran) {
   using T = typename P::T;
+  using V = typename P::V;
   const void* fn = (const void*)k_coop<P, AUG>;
   static SmemOptIn attr{};
   // CO_SMEM less the kernel's own arrays (the largest: the warps' dots)
   constexpr size_t ROOM = CO_SMEM - (P::MAXT / 32 * (MMAX + 2) + MMAX) * sizeof(T) - 5 * 1024;
-  static_assert(ROOM >= (size_t)2 * P::NC * CO_GROUPT * sizeof(typename P::V), "the groups' shares");
+  static_assert(ROOM >= (size_t)2 * P::NC * CO_GROUPT * sizeof(V), "the groups' shares");
+  const int64_t per = (items + c->nsm - 1) / c->nsm;
+  if (per > P::MAXT) return KX_OK;
   const kx_status so = smem_opt_in(c, attr, fn, ROOM);
   if (so != KX_OK) return so;
-  const CoopPlan p = coop_plan(c, fn, items, ns, m, P::MAXT, sizeof(typename P::V), P::NC, P::BATCH, ROOM);
+  auto plan = [&](int nti) { return coop_plan(c, fn, items, nti, want, m, sizeof(V), P::NC, P::BATCH, ROOM); };
+  // One block a SM, its threads an SM's share of the items (fewer, larger
+  // blocks: half the partials and arrivals of two blocks a SM, 64^3 4.1 -> 3.8
+  // ms): the shortest process.  A small grid's blocks then hold nearly every SM
+  // and the slots of a lockstep batch would run one after the other, so where
+  // they do not all fit at once, fuller blocks or the per-step launches, by the
+  // estimates above.  They know the slots that may run (want), not those of one
+  // call: a context's bits do not depend on how many still run.  plain, 32
+  // frequencies, T = 60, one after the other / per-step launches / this rule:
+  // 24^3 158 / 57 / 39 ms, 36^3 214 / 176 / 140, 30^3 in double precision 323 /
+  // 284 / 274, 2D 64^2 in double precision 125 / 35 / 35.
+  CoopPlan p = plan((int)((per + 31) / 32 * 32));
+  if (p.slots > 0 && want > p.slots) {
+    const int values = P::NC * (int)(sizeof(V) / sizeof(T));
+    double best = coop_us(c, p, want, m, values);
+    for (int nti = 64; nti <= std::min(CO_GROUPT, P::MAXT); nti += 64) {
+      if (nti <= p.nti) continue;
+      const CoopPlan f = plan(nti);
+      const double us = f.slots > 0 ? coop_us(c, f, want, m, values) : best;
+      if (us < best) {
+        best = us;
+        p = f;
+      }
+    }
+    if (steps_us(c, want, m) < best) return KX_OK;
+  }
   *ran = p.slots > 0;
   if (!*ran) return KX_OK;
   for (int q = 0; q < ns; q += p.slots) {
@@ -697,13 +738,13 @@ kx_status coop_run(kx_ctx* c, int slot0, int ns, int m, const void* g_aug, int64
 }
 
 template <typename T, int AUG, int TR>
-kx_status coop_model(kx_ctx* c, int slot0, int ns, int m, const void* g_aug, bool* ran) {
+kx_status coop_model(kx_ctx* c, int slot0, int ns, int want, int m, const void* g_aug, bool* ran) {
   const Geo& g = c->geo;
   if (g.dim == 2 && g.pml) {
     if constexpr (TR) return KX_OK;   // the adjoint does not cover the PML model
-    else return coop_run<CellItem<T, 4, AUG, 0>, AUG>(c, slot0, ns, m, g_aug, g.ncell, ran);
+    else return coop_run<CellItem<T, 4, AUG, 0>, AUG>(c, slot0, ns, want, m, g_aug, g.ncell, ran);
   }
-  if (g.dim == 2) return coop_run<CellItem<T, 2, AUG, TR>, AUG>(c, slot0, ns, m, g_aug, g.ncell, ran);
+  if (g.dim == 2) return coop_run<CellItem<T, 2, AUG, TR>, AUG>(c, slot0, ns, want, m, g_aug, g.ncell, ran);
   if constexpr (sizeof(T) == 4) {
     // the quads need 16-byte aligned rows of every array they read
     if (g.nx % 4 == 0 && (uintptr_t)g_aug % 16 == 0 && g.ncell < ((int64_t)1 << 31)) {
@@ -713,28 +754,28 @@ kx_status coop_model(kx_ctx* c, int slot0, int ns, int m, const void* g_aug, boo
       // 128 registers and two (64^3: compiled for 448 threads 3655 us, for 512
       // 3748).
       const int64_t quads = g.ncell / 4, sm = c->nsm;
-      if (quads <= sm * 256) return coop_run<QuadItem<AUG, TR, 256>, AUG>(c, slot0, ns, m, g_aug, quads, ran);
-      if (quads <= sm * 384) return coop_run<QuadItem<AUG, TR, 384>, AUG>(c, slot0, ns, m, g_aug, quads, ran);
-      if (quads <= sm * 448) return coop_run<QuadItem<AUG, TR, 448>, AUG>(c, slot0, ns, m, g_aug, quads, ran);
-      return coop_run<QuadItem<AUG, TR, 512>, AUG>(c, slot0, ns, m, g_aug, quads, ran);
+      if (quads <= sm * 256) return coop_run<QuadItem<AUG, TR, 256>, AUG>(c, slot0, ns, want, m, g_aug, quads, ran);
+      if (quads <= sm * 384) return coop_run<QuadItem<AUG, TR, 384>, AUG>(c, slot0, ns, want, m, g_aug, quads, ran);
+      if (quads <= sm * 448) return coop_run<QuadItem<AUG, TR, 448>, AUG>(c, slot0, ns, want, m, g_aug, quads, ran);
+      return coop_run<QuadItem<AUG, TR, 512>, AUG>(c, slot0, ns, want, m, g_aug, quads, ran);
     }
   }
-  return coop_run<CellItem<T, 3, AUG, TR>, AUG>(c, slot0, ns, m, g_aug, g.ncell, ran);
+  return coop_run<CellItem<T, 3, AUG, TR>, AUG>(c, slot0, ns, want, m, g_aug, g.ncell, ran);
 }
 
 }  // namespace
 
-kx_status coop_arnoldi(kx_ctx* c, int slot0, int ns, int m, const void* g_aug, int transpose, bool* ran) {
+kx_status coop_arnoldi(kx_ctx* c, int slot0, int ns, int want, int m, const void* g_aug, int transpose, bool* ran) {
   *ran = false;
   const bool f64 = c->d.precision == KX_FP64;
   if (transpose)
-    return f64 ? coop_model<double, 0, 1>(c, slot0, ns, m, nullptr, ran)
-               : coop_model<float, 0, 1>(c, slot0, ns, m, nullptr, ran);
+    return f64 ? coop_model<double, 0, 1>(c, slot0, ns, want, m, nullptr, ran)
+               : coop_model<float, 0, 1>(c, slot0, ns, want, m, nullptr, ran);
   if (g_aug)
-    return f64 ? coop_model<double, 1, 0>(c, slot0, ns, m, g_aug, ran)
-               : coop_model<float, 1, 0>(c, slot0, ns, m, g_aug, ran);
-  return f64 ? coop_model<double, 0, 0>(c, slot0, ns, m, nullptr, ran)
-             : coop_model<float, 0, 0>(c, slot0, ns, m, nullptr, ran);
+    return f64 ? coop_model<double, 1, 0>(c, slot0, ns, want, m, g_aug, ran)
+               : coop_model<float, 1, 0>(c, slot0, ns, want, m, g_aug, ran);
+  return f64 ? coop_model<double, 0, 0>(c, slot0, ns, want, m, nullptr, ran)
+             : coop_model<float, 0, 0>(c, slot0, ns, want, m, nullptr, ran);
 }
 
 }  // namespace kx

@@ -287,8 +287,9 @@ int pass_b_grid(kx_ctx* c);
 // coop.cu: m steps of the two-pass process on slots [slot0, slot0 + ns), from
 // their column 0 as set by the launch that normalised it, in one cooperative
 // launch (for as many slots as fit at a time); *ran = false where the grid is
-// too large for one item a resident thread
-kx_status coop_arnoldi(kx_ctx* c, int slot0, int ns, int m, const void* g_aug, int transpose, bool* ran);
+// too large for one item a resident thread, or the per-step launches serve
+// `want` slots sooner (want: the slots that calls of this kind may run at once)
+kx_status coop_arnoldi(kx_ctx* c, int slot0, int ns, int want, int m, const void* g_aug, int transpose, bool* ran);
 
 // adjoint.cu
 kx_status launch_adj_seed(kx_ctx* c, const void* y, void* lam, int axis, int idx);

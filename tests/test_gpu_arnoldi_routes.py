@@ -40,3 +40,37 @@ def test_default_form_of_restart_in_dimension_between_the_size_lines(prec):
         assert k["sweep"] == 0 and k["pass_a"] > 0
     else:
         assert k["sweep"] > 0 and k["pass_b"] == 0
+
+
+@pytest.mark.parametrize("dim,n,prec,m", [(3, 24, "fp32", 64), (3, 36, "fp32", 40), (3, 25, "fp32", 40), (2, 64, "fp64", 30),
+                                          (2, 96, "fp32", 30), (3, 16, "fp64", 30)])
+def test_lockstep_batch_on_a_small_grid_shares_its_launches(dim, n, prec, m):
+    """Sixteen frequencies in lockstep: a small grid's process holds nearly
+    every multiprocessor, and run one slot after the other they took up to
+    twice as long as by the per-step launches.  Either those run, or one
+    launch serves several slots; the fields are those of one frequency at a
+    time, each held to its own distance from the exact ones elsewhere (1e-6 in
+    single precision, 1e-10 in double)."""
+    sc = S.config_2d(n=n, ndisks=2, T=12.0) if dim == 2 else S.config_3d(n=n, fill=0.3, T=12.0)
+    dt = torch.float64 if prec == "fp64" else torch.float32
+    g = torch.tensor(sc.g, dtype=dt, device="cuda")
+    oms = S.freq_list(16)
+    rtol = 1e-11 if prec == "fp64" else 1e-7
+    many = Context(sc.grid, sc.eps_cell, precision=prec, krylov_dim=m, max_freqs=16, batch=16)
+    out = {}
+
+    def call():
+        out["Y"] = many.response_at_freqs(g, oms, sc.T, rtol=rtol, method="plain", plane=sc.plane, want_full=True)["Y"]
+
+    many.reset_stats()
+    k = launches(many, call)
+    steps = many.stats()["substeps"]
+    assert steps >= 16
+    assert k["pass_b"] > 0 or k["pass_a"] <= steps / 2
+    many.close()
+    one = Context(sc.grid, sc.eps_cell, precision=prec, krylov_dim=m, max_freqs=1, batch=1)
+    for f in (0, 7, 15):
+        y = one.response_at_freqs(g, oms[f:f + 1], sc.T, rtol=rtol, method="plain", plane=sc.plane, want_full=True)["Y"][0]
+        d = (out["Y"][f].double() - y.double()).norm() / y.double().norm()
+        assert float(d) < (2e-10 if prec == "fp64" else 2e-6)
+    one.close()
