@@ -324,7 +324,9 @@ kx_status kx_set_permittivity(kx_ctx* ctx, const double* eps_cell);
  * context's sub-steps replay a captured CUDA graph).  The streams of the
  * contexts must be distinct (KX_OWN_STREAM guarantees it).  Each context must be
  * created with max_freqs >= nfreq; its batch sets how many of its frequencies
- * advance together.  On failure the first error is returned and its text is
+ * advance together.  Results equal response_at_freqs on each problem up to
+ * rounding (small grids whose processes would hold the whole GPU leave room for
+ * the other threads').  On failure the first error is returned and its text is
  * kx_last_error(NULL). */
 kx_status response_at_freqs_multi(kx_ctx* const* ctxs, int nctx, const void* const* d_g,
                                   const double* omegas, int nfreq, double T, double rtol, int method,

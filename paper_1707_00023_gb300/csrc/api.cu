@@ -1332,15 +1332,18 @@ kx_status response_at_freqs_multi(kx_ctx* const* ctxs, int nctx, const void* con
   std::atomic<int> first_err{KX_OK};
   std::mutex mu;
   std::string err_text;
+  const int sharers = std::max(1, std::min(nthreads, nctx));
   auto worker = [&]() {
     cudaSetDevice(dev);
     for (;;) {
       const int k = next.fetch_add(1);
       if (k >= nctx || first_err.load() != KX_OK) return;
       const int i = order[k];
+      ctxs[i]->sharers = sharers;   // the routes of its processes know the others
       const kx_status st = response_at_freqs(ctxs[i], d_g[i], omegas + (size_t)i * nfreq, nfreq, T, rtol, method,
                                              planes + 2 * i, nullptr, intensity ? intensity + (size_t)i * nfreq : nullptr,
                                              err_est ? err_est + (size_t)i * nfreq : nullptr, nullptr);
+      ctxs[i]->sharers = 1;
       if (st != KX_OK) {
         int expect = KX_OK;
         if (first_err.compare_exchange_strong(expect, st)) {

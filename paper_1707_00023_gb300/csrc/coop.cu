@@ -667,8 +667,9 @@ double coop_us(const kx_ctx* c, const CoopPlan& p, int want, int m, int values) 
 }
 // The same with the per-step launches, which serve every slot: 24^3 1 slot 26,
 // 32 slots 148; 36^3 31 and 466; 2D 128^2 in double precision 32 slots 233.
+// Beside other contexts' launches the fixed cost is hidden by theirs.
 double steps_us(const kx_ctx* c, int want, int m) {
-  return 22.0 + (c->esize == 8 ? 5.5e-6 : 1.54e-6) * want * c->n * (0.5 * m);
+  return 22.0 / c->sharers + (c->esize == 8 ? 5.5e-6 : 1.54e-6) * want * c->n * (0.5 * m);
 }
 
 template <typename P, int AUG>
@@ -677,6 +678,7 @@ kx_status coop_run(kx_ctx* c, int slot0, int ns, int want, int m, const void* g_
   using V = typename P::V;
   const void* fn = (const void*)k_coop<P, AUG>;
   static SmemOptIn attr{};
+  want *= c->sharers;
   // CO_SMEM less the kernel's own arrays (the largest: the warps' dots)
   constexpr size_t ROOM = CO_SMEM - (P::MAXT / 32 * (MMAX + 2) + MMAX) * sizeof(T) - 5 * 1024;
   static_assert(ROOM >= (size_t)2 * P::NC * CO_GROUPT * sizeof(V), "the groups' shares");
@@ -690,8 +692,9 @@ kx_status coop_run(kx_ctx* c, int slot0, int ns, int want, int m, const void* g_
   // ms): the shortest process.  A small grid's blocks then hold nearly every SM
   // and the slots of a lockstep batch would run one after the other, so where
   // they do not all fit at once, fuller blocks or the per-step launches, by the
-  // estimates above.  They know the slots that may run (want), not those of one
-  // call: a context's bits do not depend on how many still run.  plain, 32
+  // estimates above.  They know the slots that may run (want, of every context
+  // that the threaded driver runs beside this one), not those of one call: a
+  // context's bits do not depend on how many still run.  plain, 32
   // frequencies, T = 60, one after the other / per-step launches / this rule:
   // 24^3 158 / 57 / 39 ms, 36^3 214 / 176 / 140, 30^3 in double precision 323 /
   // 284 / 274, 2D 64^2 in double precision 125 / 35 / 35.

@@ -246,6 +246,7 @@ struct kx_ctx {
   cudaStream_t aux_stream = nullptr;   // projected work overlapping the next Arnoldi process
   int side_ctas = 0;        // long-lived CTAs of other kernels sharing the SMs meanwhile
   int side_steps = 1 << 30; // leading steps of each Arnoldi process that the side CTAs may overlap
+  int sharers = 1;          // contexts that the threaded driver runs at once, this one among them
   int pdl = 0;              // launch the Arnoldi chain with programmatic dependent launch
   // single-sweep Arnoldi workspace (per slot, and one shared vector)
   void* d_swT = nullptr;

@@ -536,7 +536,8 @@ template <typename T>
 constexpr double btol_of() { return sizeof(T) == 8 ? 1e-12 : 1e-6; }
 
 // Column groups of a pass A launch: as many as fill the resident blocks it may
-// take (cap: without those kept free for side work) with the launch's cell
+// take (cap: without those kept free for side work, a share where the threaded
+// driver runs other contexts beside it) with the launch's cell
 // blocks, each with a chunk of eight columns at least.
 static int col_groups(int ncol, int64_t blocks, int cap) {
   const int want = (int)std::max<int64_t>(1, std::min<int64_t>(cap / std::max<int64_t>(blocks, 1), (ncol + 7) / 8));
@@ -584,7 +585,7 @@ static PassAPlan pass_a_plan(kx_ctx* c, int ns, const void* gaug) {
   }
   p.gr = gr.load();
   p.nb = reserve_grid(c, (int)std::min<int64_t>(std::min<int64_t>(rounds, p.gr), c->ps), p.gr);
-  p.fold = !gaug || (int64_t)p.nb * ns <= p.gr;
+  p.fold = !gaug || (int64_t)p.nb * ns * c->sharers <= p.gr;
   return p;
 }
 
@@ -604,7 +605,7 @@ static kx_status pass_a_t(kx_ctx* c, int slot, int ns, int j, const void* gaug) 
   const PassAPlan p = pass_a_plan<T>(c, ns, gaug);
   const int nb = p.nb;
   const bool vec4 = p.vec4, dense = p.dense;
-  const dim3 grd(nb, ns, dense ? 1 : col_groups(j + 1, (int64_t)nb * ns, reserve_grid(c, p.gr, p.gr)));
+  const dim3 grd(nb, ns, dense ? 1 : col_groups(j + 1, (int64_t)nb * ns, reserve_grid(c, p.gr, p.gr) / c->sharers));
   const int nbb = j >= 1 && p.fold ? pass_b_grid(c) : 0;
   const double bt = btol_of<T>();
   if (vec4) {
