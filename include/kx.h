@@ -440,7 +440,7 @@ const char* kx_last_error(const kx_ctx* ctx);
 
 /* Check of the device-side failure path (not a paper operation): every wait
  * in this library's kernels is bounded (the single-sweep Arnoldi waits on
- * mbarriers for its basis copies); when a wait runs out the kernel records
+ * mbarriers for its basis copies, the cooperative process at a grid barrier); when a wait runs out the kernel records
  * KX_ETIMEOUT, returns normally and the context stays usable.  This call
  * runs that wait, `rounds` try_wait rounds (1 .. KX_WAIT_SELFTEST_MAX_ROUNDS,
  * the limit of one wait in the library's own kernels), on an mbarrier that
@@ -449,6 +449,14 @@ const char* kx_last_error(const kx_ctx* ctx);
  * range) or KX_ECUDA. */
 #define KX_WAIT_SELFTEST_MAX_ROUNDS (4194304u)
 kx_status kx_wait_selftest(kx_ctx* ctx, unsigned rounds);
+
+/* Limit of one wait at the grid barrier of this context's cooperative
+ * Arnoldi processes, in polls (0 .. KX_BARRIER_MAX_POLLS, which is the default
+ * and about a second).  With 0 or a few polls the waits run out at once: the
+ * call that ran the process returns KX_ETIMEOUT, and after the limit is set
+ * back the context computes as before.  A check of the failure path. */
+#define KX_BARRIER_MAX_POLLS (2097152u)
+kx_status kx_set_wait_limit(kx_ctx* ctx, unsigned polls);
 
 /* Allocation-free Arnoldi (the paper has no counterpart: this is a
  * deployment convenience).  Some callers cannot allocate device memory at

@@ -200,9 +200,7 @@ kx_status time_loop(kx_ctx* c, int slot0, int ns, int want, const void* g_aug, d
     for (int q = 0; q < ns; ++q) {
       const SlotState& st = c->h_state[slot0 + q];
       if (st.status)
-        return fail(c, (kx_status)st.status,
-                    st.status == KX_ENOCONV ? "time sub-step control: no step length met the tolerance"
-                                            : "non-finite value in the Krylov process");
+        return fail(c, (kx_status)st.status, process_error(st.status));
       all = all && st.retired;
       if (!st.retired && st.substeps > 0 && st.t_now > 0.0)
         need = std::max(need, std::ceil((st.T - st.t_now) * st.substeps / st.t_now));
@@ -283,7 +281,7 @@ kx_status stationary_core(kx_ctx* c, const void* d_g, const double* omegas, int 
   for (int cyc = 0; matvecs < max_matvecs; ++cyc) {
     KX_TRY(arnoldi_steps(c, slot, 1, 1, c->m, nullptr));
     KX_TRY(read_state(c, slot, &st));
-    if (st.status) return fail(c, (kx_status)st.status, "non-finite value in the Arnoldi process");
+    if (st.status) return fail(c, (kx_status)st.status, process_error(st.status));
     const int md = st.m_done;
     KX_TRY(launch_shifted_solve(c, slot, nfreq, md));
     KX_TRY(launch_zupdate(c, slot, nfreq, zre, zim, md));
@@ -738,7 +736,7 @@ kx_status arnoldi(kx_ctx* c, const void* d_v0, int m, void* d_V, double* H, doub
   if (c->d.arnoldi_form == KX_ARN_SWEEP) KX_TRY(sweep_arnoldi(c, slot, m));
   else KX_TRY(arnoldi_steps(c, slot, 1, 1, m, nullptr));
   KX_TRY(read_state(c, slot, &st));
-  if (st.status) return fail(c, (kx_status)st.status, "non-finite value in the Arnoldi process");
+  if (st.status) return fail(c, (kx_status)st.status, process_error(st.status));
   *beta = st.beta;
   *m_done = st.m_done;
   // H: context stride c->m + 1 -> caller stride m + 1
@@ -782,7 +780,7 @@ kx_status expm_phi_project(kx_ctx* c, const double* H, int ldh, int m, double be
           "status read");
   KX_TRY(sync(c));
   std::memcpy(&status, c->h_small, sizeof(int));
-  if (status) return fail(c, KX_ENONFINITE, "singular Pade denominator");
+  if (status) return fail(c, KX_ENONFINITE, "non-finite projected matrix");
   return KX_OK;
 }
 
@@ -1071,7 +1069,7 @@ kx_status response_restart_dim(kx_ctx* c, const void* d_g, const double* omegas,
           "omega upload");
   KX_TRY(rst_arnoldi(c, 0));
   KX_TRY(read_state(c, 0, &st));
-  if (st.status) return fail(c, (kx_status)st.status, "non-finite value in the Arnoldi process");
+  if (st.status) return fail(c, (kx_status)st.status, process_error(st.status));
   // sample grid from ||H_m||_1 of the first restart
   const int ldh = c->m + 1;
   std::vector<double> Hh((size_t)ldh * c->m);
@@ -1137,7 +1135,7 @@ kx_status response_restart_dim(kx_ctx* c, const void* d_g, const double* omegas,
     if (*h_status) {
       sync(c);
       if (*h_status == KX_ETIMEOUT)
-        return fail(c, KX_ETIMEOUT, "Arnoldi process: a bounded wait for a basis copy ran out");
+        return fail(c, KX_ETIMEOUT, process_error(KX_ETIMEOUT));
       return fail(c, KX_ENONFINITE, "restart set-up: non-finite Arnoldi process or projected exponential");
     }
     all_stopped = true;
@@ -1252,7 +1250,7 @@ kx_status adjoint_response_grad(kx_ctx* c, const void* d_g, const double* omegas
       KX_TRY(launch_combine(c, 0, 1));
       KX_TRY(read_states(c, 0, 1));
       const SlotState& st = c->h_state[0];
-      if (st.status) return fail(c, (kx_status)st.status, "adjoint forward: Krylov process failed");
+      if (st.status) return fail(c, (kx_status)st.status, std::string("adjoint forward: ") + process_error(st.status));
       tauk.push_back(st.t_acc);
       tnow = st.t_now;
       if (st.retired) break;
@@ -1282,8 +1280,9 @@ kx_status adjoint_response_grad(kx_ctx* c, const void* d_g, const double* omegas
       KX_TRY(arnoldi_steps(c, 0, 1, 1, c->m, d_g));
       KX_TRY(arnoldi_steps(c, 1, 1, 1, c->m, nullptr, 1));
       KX_TRY(read_states(c, 0, 2));
-      if (c->h_state[0].status || c->h_state[1].status)
-        return fail(c, KX_ENONFINITE, "adjoint backward: Krylov process failed");
+      for (int q = 0; q < 2; ++q)
+        if (const int bad = c->h_state[q].status)
+          return fail(c, (kx_status)bad, std::string("adjoint backward: ") + process_error(bad));
       KX_CUDA(c, cudaMemsetAsync(c->d_small + 64, 0, sizeof(int), c->stream), "status reset");
       KX_TRY(launch_adj_substep(c, tauk[k], W, tk[k], d_g));
       KX_TRY(launch_combine(c, 1, 1));   // lambda(t_k) = W w(tau_k)
@@ -1297,7 +1296,7 @@ kx_status adjoint_response_grad(kx_ctx* c, const void* d_g, const double* omegas
   KX_TRY(sync(c));
   int status = 0;
   std::memcpy(&status, c->h_small + 128, sizeof(int));
-  if (status) return fail(c, KX_ENONFINITE, "adjoint: singular projected exponential");
+  if (status) return fail(c, KX_ENONFINITE, "adjoint: non-finite projected exponential");
   double L = 0.0;
   for (int f = 0; f < nfreq; ++f) L += c->h_small[f];
   *loss = L;
@@ -1419,6 +1418,13 @@ kx_status kx_wait_selftest(kx_ctx* c, unsigned rounds) {
   KX_TRY(sync(c));
   if (h == KX_ETIMEOUT) return fail(c, KX_ETIMEOUT, "bounded device wait ran out (self-test)");
   if (h != KX_OK) return fail(c, KX_ECUDA, "self-test kernel did not report");
+  return KX_OK;
+}
+
+kx_status kx_set_wait_limit(kx_ctx* c, unsigned polls) {
+  if (!c) return KX_EINVAL;
+  if (polls > KX_BARRIER_MAX_POLLS) return fail(c, KX_EINVAL, "polls must be 0 .. KX_BARRIER_MAX_POLLS (2097152)");
+  c->wait_polls = polls;
   return KX_OK;
 }
 

@@ -569,7 +569,7 @@ kx_status response_restart_dim_batch(kx_batch* b, const void* const* d_g, const 
     kx_ctx* c = b->ctx[i];
     const SlotState& st = c->h_state[0];
     if (st.status)
-      return bfail(b, (kx_status)st.status, "problem " + std::to_string(i) + ": Arnoldi process failed");
+      return bfail(b, (kx_status)st.status, "problem " + std::to_string(i) + ": " + process_error(st.status));
     KB_CUDA(b, cudaMemcpy(Hh.data(), make_slot<double>(c, 0).H, Hh.size() * sizeof(double), cudaMemcpyDeviceToHost),
             "H read");
     double nu = 0.0;
@@ -641,7 +641,7 @@ kx_status response_restart_dim_batch(kx_batch* b, const void* const* d_g, const 
         cudaStreamSynchronize(S);
         return bfail(b, hs[MAXF] == KX_ETIMEOUT ? KX_ETIMEOUT : KX_ENONFINITE,
                      "problem " + std::to_string(i) +
-                         (hs[MAXF] == KX_ETIMEOUT ? ": a bounded wait for a basis copy ran out"
+                         (hs[MAXF] == KX_ETIMEOUT ? std::string(": ") + process_error(KX_ETIMEOUT)
                                                   : ": non-finite Arnoldi process or projected exponential"));
       }
       bool all_stopped = true;

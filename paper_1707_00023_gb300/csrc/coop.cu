@@ -44,20 +44,21 @@ constexpr int CO_GROUPT = 256;             // threads a block may have by splitt
 // of L1, too few for the loads in flight (64^3 with 4 columns held 3758 us,
 // with 5 4430; 45^3 cells with 8 1585, with 16 1737).
 constexpr size_t CO_SMEM = 195 * 1024;
-constexpr unsigned CO_WAIT_LIMIT = 1u << 21;   // polls of one barrier wait (about a second)
 
 // Barrier over the `blocks` blocks of a slot: the counter reaches `target`
 // (blocks times the barriers so far; zeroed by the kernel that normalises
-// column 0).  False when the wait runs out.  The release on the arrival covers
+// column 0).  False when the wait runs out: after `limit` polls (a cooperative
+// grid starts all its blocks or none, so other kernels' blocks are never
+// waited for here).  The release on the arrival covers
 // the writes of the whole block (ordered before it by the block barrier), and
 // the acquire on the poll the reads after it.
-__device__ __forceinline__ bool grid_barrier(unsigned* cnt, unsigned target) {
+__device__ __forceinline__ bool grid_barrier(unsigned* cnt, unsigned target, unsigned limit) {
   __shared__ int ok;
   __syncthreads();
   if (threadIdx.x == 0) {
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(cnt) : "memory");
     int good = 0;
-    for (unsigned k = 0; k < CO_WAIT_LIMIT; ++k) {
+    for (unsigned k = 0; k < limit; ++k) {
       unsigned v;
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(cnt) : "memory");
       if ((int)(v - target) >= 0) {
@@ -323,7 +324,7 @@ __global__ void __launch_bounds__(P::MAXT, 1) k_coop(Geo g, SlotSet<typename P::
                                                     const typename P::T* __restrict__ ie,
                                                     const typename P::T* __restrict__ sig2,
                                                     const typename P::T* __restrict__ gsrc, int ldh, double btol,
-                                                    int nti, int kc) {
+                                                    int nti, int kc, unsigned wait) {
   using T = typename P::T;
   using V = typename P::V;
   using SO = SumOf<T>;
@@ -436,7 +437,7 @@ __global__ void __launch_bounds__(P::MAXT, 1) k_coop(Geo g, SlotSet<typename P::
       SO::put(s.part + (int64_t)col * s.ps + b, t);
     }
     bars += G;
-    if (!grid_barrier(cnt, bars)) return timeout();
+    if (!grid_barrier(cnt, bars, wait)) return timeout();
     if constexpr (sizeof(T) == 4) {
       // the dots' totals in every block, eight columns a warp
       for (int c0 = 8 * warp; c0 <= ncol; c0 += 8 * nw) {
@@ -460,7 +461,7 @@ __global__ void __launch_bounds__(P::MAXT, 1) k_coop(Geo g, SlotSet<typename P::
         if (lane == 0) SO::put(s.part + (int64_t)TOT_COL * s.ps + col, x);
       }
       bars += G;
-      if (!grid_barrier(cnt, bars)) return timeout();
+      if (!grid_barrier(cnt, bars, wait)) return timeout();
       for (int col = tid; col <= ncol; col += blockDim.x) tot[col] = SO::get(s.part + (int64_t)TOT_COL * s.ps + col);
     }
     __syncthreads();
@@ -576,7 +577,7 @@ __global__ void __launch_bounds__(P::MAXT, 1) k_coop(Geo g, SlotSet<typename P::
       if (rec) s.counter[2] = abort_requested(st) ? 1u : 0u;
     }
     bars += G;
-    if (!grid_barrier(cnt, bars)) return timeout();
+    if (!grid_barrier(cnt, bars, wait)) return timeout();
     if (warp == 0) {
       S xs = SO::of(T(0));
       for (int q = lane; q < G; q += 32) xs = add(xs, SO::get(s.part + (int64_t)FINB_COL * s.ps + q));
@@ -731,7 +732,7 @@ kx_status coop_run(kx_ctx* c, int slot0, int ns, int want, int m, const void* g_
     time_begin(c);
     cudaLaunchKernelEx(&cfg, k_coop<P, AUG>, c->geo, make_slotset<T>(c, slot0 + q), m, c->ld,
                        (const T*)c->d_inv_eps, (const T*)c->d_sig2, (const T*)g_aug, c->m + 1,
-                       sizeof(T) == 8 ? 1e-12 : 1e-6, p.nti, p.keep);
+                       sizeof(T) == 8 ? 1e-12 : 1e-6, p.nti, p.keep, c->wait_polls);
     // algorithmic bytes: per step v_j, V_0 .. V_{j-1} twice, v_{j+1}, 1/eps (and g)
     time_end(c, KX_K_PASS_A,
              nq * m * ((m + 2.0) * vb + (double)c->geo.ne * c->geo.ncell * c->esize + (g_aug ? vb : 0.0)));

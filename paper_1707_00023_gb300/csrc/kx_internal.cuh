@@ -246,6 +246,7 @@ struct kx_ctx {
   cudaStream_t aux_stream = nullptr;   // projected work overlapping the next Arnoldi process
   int side_ctas = 0;        // long-lived CTAs of other kernels sharing the SMs meanwhile
   int side_steps = 1 << 30; // leading steps of each Arnoldi process that the side CTAs may overlap
+  unsigned wait_polls = KX_BARRIER_MAX_POLLS;   // polls of one grid-barrier wait (coop.cu)
   int sharers = 1;          // contexts that the threaded driver runs at once, this one among them
   int pdl = 0;              // launch the Arnoldi chain with programmatic dependent launch
   // single-sweep Arnoldi workspace (per slot, and one shared vector)
@@ -416,6 +417,13 @@ inline int reserve_grid(const kx_ctx* c, int nb, int gr) {
 // expected beside the first side_steps steps of a process.
 inline int reserve_grid_at(const kx_ctx* c, int nb, int gr, int j) {
   return j < c->side_steps ? reserve_grid(c, nb, gr) : nb;
+}
+
+// The text for a slot's failure status.
+inline const char* process_error(int status) {
+  return status == KX_ETIMEOUT  ? "Arnoldi process: a bounded device wait ran out"
+         : status == KX_ENOCONV ? "time sub-step control: no step length met the tolerance"
+                                : "non-finite value in the Arnoldi process";
 }
 
 // Timing brackets around one launch (no-ops unless timing is on).
