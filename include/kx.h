@@ -458,6 +458,12 @@ kx_status kx_wait_selftest(kx_ctx* ctx, unsigned rounds);
 #define KX_BARRIER_MAX_POLLS (2097152u)
 kx_status kx_set_wait_limit(kx_ctx* ctx, unsigned polls);
 
+/* Most blocks of the thread-block clusters that do the context's projected
+ * (dense) work: 0 (the default) takes 16 where the device can place such a
+ * cluster and 8, the portable size, elsewhere; 8 or 16 asks for that size (16
+ * as far as the device allows).  The results have the same bits. */
+kx_status kx_set_cluster_blocks(kx_ctx* ctx, int blocks);
+
 /* Allocation-free Arnoldi (the paper has no counterpart: this is a
  * deployment convenience).  Some callers cannot allocate device memory at
  * all -- code running inside another runtime's memory pool, plug-ins handed

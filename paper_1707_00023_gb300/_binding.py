@@ -29,7 +29,8 @@ EXPORTS = ["krylov_expm_create", "krylov_expm_create_mat", "krylov_expm_destroy"
            "response_at_freqs", "kx_get_stats", "kx_reset_stats", "kx_set_timing",
            "kx_kernel_times", "kx_last_error", "kx_arnoldi_noalloc", "kx_noalloc_last_error",
            "adjoint_response_grad", "kx_set_permittivity", "response_at_freqs_multi", "kx_stream",
-           "response_restart_dim", "kx_wait_selftest", "kx_set_wait_limit", "kx_batch_create", "kx_batch_destroy",
+           "response_restart_dim", "kx_wait_selftest", "kx_set_wait_limit", "kx_set_cluster_blocks",
+           "kx_batch_create", "kx_batch_destroy",
            "kx_batch_get_info", "kx_batch_last_error", "response_restart_dim_batch", "kx_batch_set_timing"]
 KCLASSES = ["pass_a", "pass_b", "restart", "projected", "zupdate", "apply", "cascade", "sweep", "swapply"]
 # Arnoldi forms (kx_desc.arnoldi_form)
@@ -116,6 +117,7 @@ def load_library(path: Optional[str] = None):
     lib.kx_noalloc_last_error.argtypes = []
     lib.kx_wait_selftest.argtypes = [vp, ctypes.c_uint]
     lib.kx_set_wait_limit.argtypes = [vp, ctypes.c_uint]
+    lib.kx_set_cluster_blocks.argtypes = [vp, ctypes.c_int]
     lib.kx_noalloc_last_error.restype = ctypes.c_char_p
     lib.kx_batch_create.argtypes = [ctypes.POINTER(vp), ctypes.c_int, vp, ctypes.POINTER(vp)]
     lib.kx_batch_destroy.argtypes = [vp]
@@ -256,6 +258,11 @@ class Context:
         """Polls of one grid-barrier wait of the cooperative Arnoldi process
         (0 .. 2097152, the default); a check of the failure path."""
         self._check(self.lib.kx_set_wait_limit(self.h, polls))
+
+    def set_cluster_blocks(self, blocks: int):
+        """Blocks a cluster of the projected work: 0 (by the device), 8 or 16;
+        the same bits."""
+        self._check(self.lib.kx_set_cluster_blocks(self.h, blocks))
 
     def kernel_times(self):
         """Per-class {ms, bytes, launches} recorded since timing was switched on."""

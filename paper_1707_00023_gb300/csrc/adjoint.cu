@@ -69,7 +69,7 @@ __global__ void __launch_bounds__(CD_THREADS) k_adj_expm(SlotSet<float> ss, int 
                                                          int* status) {
   extern __shared__ __align__(16) double sm[];
   __shared__ double red[32];
-  const int which = blockIdx.x / CD_CTAS, rank = cl_rank();
+  const int which = blockIdx.x / cl_size(), rank = cl_rank();
   const Slot<float> sl = slot_at(ss, which);
   const double* H = sl.H;
   const int m = sl.st->m_done;
@@ -357,14 +357,15 @@ kx_status launch_adj_substep(kx_ctx* c, double tau, double omega, double tk, con
     return KX_EINVAL;
   }
   const int m = c->m;
-  static SmemOptIn attr{};
-  const kx_status so = smem_opt_in(c, attr, (const void*)k_adj_expm, CD_SMEM);
+  static ClusterOptIn attr{};
+  int cl = 0;
+  const kx_status so = cluster_opt_in(c, attr, (const void*)k_adj_expm, CD_SMEM, &cl);
   if (so != KX_OK) return so;
   int* status = reinterpret_cast<int*>(c->d_small + 64);
   const SlotSet<float> ss = make_slotset<float>(c, 0);
   const int nq = nsub * GAUSS_P;
   time_begin(c);
-  launch_cluster(k_adj_expm, 2, CD_SMEM, c->stream, ss, m + 1, tau / nsub, c->d_cd_ws, status);
+  launch_cluster(k_adj_expm, cl, 2, CD_SMEM, c->stream, ss, m + 1, tau / nsub, c->d_cd_ws, status);
   KX_CHECK_LAUNCH(c);
   k_adj_march<<<dim3(GAUSS_P + 1, 2), 256, 0, c->stream>>>(ss, m + 1, tau, nsub, c->d_gauss, c->d_gauss + GAUSS_P,
                                                            omega, tk, c->d_cd_ws, c->d_adj_alpha, c->d_adj_omg,

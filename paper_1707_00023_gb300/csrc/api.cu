@@ -1428,6 +1428,13 @@ kx_status kx_set_wait_limit(kx_ctx* c, unsigned polls) {
   return KX_OK;
 }
 
+kx_status kx_set_cluster_blocks(kx_ctx* c, int blocks) {
+  if (!c) return KX_EINVAL;
+  if (blocks != 0 && blocks != CD_PORTABLE && blocks != CD_WIDE) return fail(c, KX_EINVAL, "blocks must be 0, 8 or 16");
+  c->cluster_blocks = blocks;
+  return KX_OK;
+}
+
 kx_status kx_set_timing(kx_ctx* c, int on) {
   if (!c) return KX_EINVAL;
   c->timing = on ? 1 : 0;

@@ -1,15 +1,16 @@
 // Dense FP64 work on the projected (small) matrices, spread over a cluster
-// of CD_CTAS thread blocks.
+// of C = 16 thread blocks (8, the portable size, where the device cannot place
+// one of 16: the same operations on other rows, the same bits).
 //
 // What bounds it: this GPU's double-precision pipe does about two FMAs a
 // clock on one SM, so one product of 64-square matrices takes one SM 66 us
 // and an exponential 0.9 ms; the matrices themselves are 33 KB.  Each block
-// therefore owns R = ceil(n / CD_CTAS) rows of every matrix, held in its
+// therefore owns R = ceil(n / C) rows of every matrix, held in its
 // shared memory, and multiplies them with a right operand staged whole in
 // shared memory (4.3 us for n = 64 at the pipe's rate).  Sixteen blocks against
-// the portable eight: an exponential of norm 2 at m = 64 61 against 94 us.  Rows of X Y need all of Y but
-// only the same rows of X, so a chain of products with one fixed right
-// operand (the powers of A, the Horner steps in A^4) runs without any
+// eight: an exponential of norm 2 at m = 64 61 against 94 us.  Rows of X Y need
+// all of Y but only the same rows of X, so a chain of products with one fixed
+// right operand (the powers of A, the Horner steps in A^4) runs without any
 // exchange between the blocks; only a new right operand is published through
 // global memory (L2) with one cluster barrier.
 //
@@ -31,10 +32,10 @@
 
 namespace kx {
 
-constexpr int CD_CTAS = 16;                // thread blocks a cluster (beyond the portable eight: opted in per kernel)
+constexpr int CD_WIDE = 16, CD_PORTABLE = 8;   // thread blocks a cluster (the wide form is opted in per kernel)
 constexpr int CD_THREADS = 256;
 constexpr int CD_NMAX = MMAX + RST_P;      // largest matrix
-constexpr int CD_RMAX = (CD_NMAX + CD_CTAS - 1) / CD_CTAS;
+constexpr int CD_RMAX = (CD_NMAX + CD_PORTABLE - 1) / CD_PORTABLE;
 constexpr int CD_LD = 72;                  // row stride, shared and global
 constexpr int CD_MAT = CD_NMAX * CD_LD;    // doubles of one matrix
 constexpr int CD_SLICE = CD_RMAX * CD_LD;  // doubles of one block's rows
@@ -47,6 +48,11 @@ static_assert(CD_NMAX <= CD_LD && CD_LD % 2 == 0, "rows are loaded as 16-byte pa
 __device__ __forceinline__ int cl_rank() {
   unsigned r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return (int)r;
+}
+__device__ __forceinline__ int cl_size() {
+  unsigned r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
   return (int)r;
 }
 // All threads of the cluster: what any of them wrote before (shared or
@@ -67,7 +73,7 @@ struct CdRows {
   int r0, R;
 };
 __device__ __forceinline__ CdRows cd_rows(int n, int rank) {
-  const int per = (n + CD_CTAS - 1) / CD_CTAS;
+  const int C = cl_size(), per = (n + C - 1) / C;
   const int r0 = min(n, rank * per);
   return {r0, min(n, r0 + per) - r0};
 }
@@ -258,18 +264,54 @@ __device__ double* cd_expm(const CdShared& sh, double* g, int n, CdRows w, int q
   return P;
 }
 
-// Launch of a cluster kernel: `clusters` clusters of CD_CTAS blocks.
+// Blocks a cluster of this kernel (with `smem` bytes of dynamic shared memory)
+// on the current device: CD_WIDE where such a cluster can be placed, else
+// CD_PORTABLE; a context may ask for either.  Looked up once a device.
+struct ClusterOptIn {
+  SmemOptIn smem;
+  int blocks[SMEM_MAX_DEVICES];   // accessed atomically
+};
+inline kx_status cluster_opt_in(kx_ctx* c, ClusterOptIn& rec, const void* kernel, size_t smem, int* blocks) {
+  const kx_status so = smem_opt_in(c, rec.smem, kernel, smem);
+  if (so != KX_OK) return so;
+  int dev = 0;
+  cudaGetDevice(&dev);   // checked by smem_opt_in
+  int n = __atomic_load_n(&rec.blocks[dev], __ATOMIC_ACQUIRE);
+  if (n == 0) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(CD_WIDE);
+    cfg.blockDim = dim3(CD_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = CD_WIDE;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int fit = 0;
+    const bool wide = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+                      cudaOccupancyMaxActiveClusters(&fit, kernel, &cfg) == cudaSuccess && fit >= 1;
+    if (!wide) cudaGetLastError();
+    n = wide ? CD_WIDE : CD_PORTABLE;
+    __atomic_store_n(&rec.blocks[dev], n, __ATOMIC_RELEASE);
+  }
+  *blocks = c->cluster_blocks > 0 ? std::min(c->cluster_blocks, n) : n;
+  return KX_OK;
+}
+
+// Launch of a cluster kernel: `clusters` clusters of `blocks` blocks.
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_cluster(void (*kern)(KArgs...), int clusters, size_t smem, cudaStream_t st, Args... args) {
+inline cudaError_t launch_cluster(void (*kern)(KArgs...), int blocks, int clusters, size_t smem, cudaStream_t st,
+                                  Args... args) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(clusters * CD_CTAS);
+  cfg.gridDim = dim3(clusters * blocks);
   cfg.blockDim = dim3(CD_THREADS);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute at[1];
-  cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = CD_CTAS;
+  at[0].val.clusterDim.x = blocks;
   at[0].val.clusterDim.y = 1;
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;

@@ -247,6 +247,7 @@ struct kx_ctx {
   int side_ctas = 0;        // long-lived CTAs of other kernels sharing the SMs meanwhile
   int side_steps = 1 << 30; // leading steps of each Arnoldi process that the side CTAs may overlap
   unsigned wait_polls = KX_BARRIER_MAX_POLLS;   // polls of one grid-barrier wait (coop.cu)
+  int cluster_blocks = 0;   // most blocks a cluster of the projected work (0: by the device)
   int sharers = 1;          // contexts that the threaded driver runs at once, this one among them
   int pdl = 0;              // launch the Arnoldi chain with programmatic dependent launch
   // single-sweep Arnoldi workspace (per slot, and one shared vector)

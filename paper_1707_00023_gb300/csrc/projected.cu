@@ -22,18 +22,19 @@ namespace kx {
 // One cluster a slot: the exponential of one step of the table as in
 // kx_cdense.cuh, then the table itself, each block multiplying its rows (16
 // lanes a row: four products and four sums of the slow double-precision pipe
-// in each of four warps) and storing its entries of u into every block's
+// in each of two warps) and storing its entries of u into every block's
 // shared memory, one cluster barrier a step.  Every block follows the same
 // values, so all take the same decisions; block 0 records them.
 constexpr int TAB_LANES = 16;
-constexpr int TAB_ROWS = MMAX / CD_CTAS;   // rows of a block at the largest m
+constexpr int TAB_ROWS = MMAX / CD_PORTABLE;   // most rows of a block
 constexpr int TAB_STEPS = 32;              // K: steps of the table, one a lane in the check
-static_assert(TAB_ROWS * TAB_LANES <= CD_THREADS && TAB_ROWS * TAB_LANES % 32 == 0, "whole warps");
+static_assert(TAB_ROWS * TAB_LANES <= CD_THREADS && MMAX / CD_WIDE * TAB_LANES % 32 == 0, "whole warps");
+static_assert(CD_WIDE <= TAB_LANES, "a lane stores to each block");
 static_assert((TAB_STEPS + 1) * MMAX <= CD_MAT, "the table fits the right operand's place");
 
 __global__ void __launch_bounds__(CD_THREADS) k_substep(SlotSet<float> ss, int ldh, double* ws) {
   constexpr int K = TAB_STEPS;
-  const int slot = blockIdx.x / CD_CTAS, rank = cl_rank();
+  const int C = cl_size(), slot = blockIdx.x / C, rank = cl_rank();
   const Slot<float> sl = slot_at(ss, slot);
   const double* H = sl.H;
   SlotState* st = sl.st;
@@ -88,14 +89,14 @@ __global__ void __launch_bounds__(CD_THREADS) k_substep(SlotSet<float> ss, int l
     cl_sync();   // every block past its exponential before another one's stores arrive
     const int row = tid / TAB_LANES, lane = tid % TAB_LANES;
     for (int k = 1; k <= K; ++k) {
-      if (tid < TAB_ROWS * TAB_LANES) {
+      if (tid < MMAX / C * TAB_LANES) {
         const double* u = U + (k - 1) * MMAX;
         double x = 0.0;
         if (row < w.R)
           for (int c = lane; c < m; c += TAB_LANES) x = fma(E[row * CD_LD + c], u[c], x);
 #pragma unroll
         for (int o = TAB_LANES / 2; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-        if (row < w.R && lane < CD_CTAS) cl_store(&U[k * MMAX + w.r0 + row], lane, x);
+        if (row < w.R && lane < C) cl_store(&U[k * MMAX + w.r0 + row], lane, x);
       }
       cl_sync();
     }
@@ -158,11 +159,12 @@ __global__ void __launch_bounds__(CD_THREADS) k_substep(SlotSet<float> ss, int l
 
 kx_status launch_substep_control(kx_ctx* c, int slot, int ns) {
   const int m = c->m;
-  static SmemOptIn attr{};
-  const kx_status so = smem_opt_in(c, attr, (const void*)k_substep, CD_SMEM);
+  static ClusterOptIn attr{};
+  int blocks = 0;
+  const kx_status so = cluster_opt_in(c, attr, (const void*)k_substep, CD_SMEM, &blocks);
   if (so != KX_OK) return so;
   time_begin(c);
-  launch_cluster(k_substep, ns, CD_SMEM, c->stream, make_slotset<float>(c, slot), m + 1, c->d_cd_ws);
+  launch_cluster(k_substep, blocks, ns, CD_SMEM, c->stream, make_slotset<float>(c, slot), m + 1, c->d_cd_ws);
   time_end(c, KX_K_PROJ, 0.0);
   KX_CHECK_LAUNCH(c);
   return KX_OK;
@@ -386,12 +388,13 @@ __global__ void __launch_bounds__(CD_THREADS) k_expm_project(const double* H, in
 
 kx_status launch_expm_project(kx_ctx* c, const double* dH, int ldh, int m, double beta, double tau,
                               const double* d_om, int nfreq, double* d_u) {
-  static SmemOptIn attr{};
-  const kx_status so = smem_opt_in(c, attr, (const void*)k_expm_project, PHI_SMEM);
+  static ClusterOptIn attr{};
+  int blocks = 0;
+  const kx_status so = cluster_opt_in(c, attr, (const void*)k_expm_project, PHI_SMEM, &blocks);
   if (so != KX_OK) return so;
   int* status = reinterpret_cast<int*>(c->d_small + 64);
   time_begin(c);
-  launch_cluster(k_expm_project, 1, PHI_SMEM, c->stream, dH, ldh, m, beta, tau, d_om, nfreq, d_u, status,
+  launch_cluster(k_expm_project, blocks, 1, PHI_SMEM, c->stream, dH, ldh, m, beta, tau, d_om, nfreq, d_u, status,
                  c->d_cd_ws);
   time_end(c, KX_K_PROJ, 0.0);
   KX_CHECK_LAUNCH(c);

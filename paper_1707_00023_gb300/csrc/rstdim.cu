@@ -92,13 +92,13 @@ constexpr int RST_ZC = RST_L * RST_P;                   // columns of [Z_0 .. Z_
 constexpr int RST_O = 3 * RST_L;                        // sampled values of a chunk
 constexpr int RST_SMEM = CD_SMEM + MMAX * CD_LD * (int)sizeof(double);
 static_assert(RST_L == 16, "four doublings");
-static_assert(RST_ZC / 2 <= CD_LD && RST_O <= MMAX, "the half-filled tables fit the shared operands");
+static_assert(RST_ZC / 2 <= CD_LD && RST_O <= MMAX && RST_O / 2 <= CD_RMAX * CD_PORTABLE, "the half-filled tables fit the shared operands");
 
 __global__ void __launch_bounds__(CD_THREADS) k_rst_setup(const double* __restrict__ H, int ldh, const SlotState* st,
                                                           double d, double* mats, double* ws, int* status) {
   extern __shared__ __align__(16) double sm[];
   __shared__ double red[32];
-  const int rank = cl_rank(), tid = threadIdx.x;
+  const int C = cl_size(), rank = cl_rank(), tid = threadIdx.x;
   const int md = st->m_done;
   const int n = md + RST_P;
   // (m+6)-square [[-d H_m, e_1 e_1^T], [0, J]], J the shift
@@ -163,7 +163,7 @@ __global__ void __launch_bounds__(CD_THREADS) k_rst_setup(const double* __restri
       *reinterpret_cast<double2*>(Zs + r * CD_LD + c) = __ldcg(reinterpret_cast<const double2*>(gZ + r * RST_ZC + c));
     }
     // this block's share of the sampling rows
-    const int per = (3 * half + CD_CTAS - 1) / CD_CTAS;
+    const int per = (3 * half + C - 1) / C;
     const int s0 = min(3 * half, rank * per), ns = min(3 * half, s0 + per) - s0;
     for (int o = tid; o < ns * md; o += CD_THREADS) {
       const int r = o / md, c = o - r * md;
@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(CD_THREADS) k_rst_setup(const double* __restri
   }
   // the tables of the marching kernels, zero past the basis' size
   const double* EL = gE;                       // E^16 after four doublings
-  const int t0 = rank * CD_THREADS + tid, nt = CD_CTAS * CD_THREADS;
+  const int t0 = rank * CD_THREADS + tid, nt = C * CD_THREADS;
   for (int o = t0; o < MMAX * MMAX; o += nt) {
     const int r = o / MMAX, c = o % MMAX;
     mats[o] = r < md && c < md ? __ldcg(EL + r * CD_LD + c) : 0.0;
@@ -217,11 +217,12 @@ __global__ void __launch_bounds__(CD_THREADS) k_rst_setup(const double* __restri
 kx_status launch_rst_setup(kx_ctx* c, cudaStream_t st, int slot, double d) {
   Slot<float> s = make_slot<float>(c, slot);
   int* status = reinterpret_cast<int*>(c->d_small + 64);
-  static SmemOptIn attr{};
-  const kx_status so = smem_opt_in(c, attr, (const void*)k_rst_setup, RST_SMEM);
+  static ClusterOptIn attr{};
+  int blocks = 0;
+  const kx_status so = cluster_opt_in(c, attr, (const void*)k_rst_setup, RST_SMEM, &blocks);
   if (so != KX_OK) return so;
   time_begin(c);
-  launch_cluster(k_rst_setup, 1, RST_SMEM, st, (const double*)s.H, c->m + 1, (const SlotState*)s.st, d, c->d_rst_mats,
+  launch_cluster(k_rst_setup, blocks, 1, RST_SMEM, st, (const double*)s.H, c->m + 1, (const SlotState*)s.st, d, c->d_rst_mats,
                  c->d_cd_ws, status);
   time_end(c, KX_K_PROJ, 0.0);
   KX_CHECK_LAUNCH(c);
