@@ -49,7 +49,9 @@ constexpr size_t CO_SMEM = 195 * 1024;
 // (blocks times the barriers so far; zeroed by the kernel that normalises
 // column 0).  False when the wait runs out: after `limit` polls (a cooperative
 // grid starts all its blocks or none, so other kernels' blocks are never
-// waited for here).  The release on the arrival covers
+// waited for here).  Four polls a round of the loop: with one the double-
+// precision process, three barriers a step, took 1.3 % longer (32^3 2845 us,
+// 2811).  The release on the arrival covers
 // the writes of the whole block (ordered before it by the block barrier), and
 // the acquire on the poll the reads after it.
 __device__ __forceinline__ bool grid_barrier(unsigned* cnt, unsigned target, unsigned limit) {
@@ -58,6 +60,7 @@ __device__ __forceinline__ bool grid_barrier(unsigned* cnt, unsigned target, uns
   if (threadIdx.x == 0) {
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(cnt) : "memory");
     int good = 0;
+#pragma unroll 4
     for (unsigned k = 0; k < limit; ++k) {
       unsigned v;
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(cnt) : "memory");
