@@ -188,8 +188,10 @@ kx_status arnoldi(kx_ctx* ctx, const void* d_v0, int m, void* d_V, double* H,
  *   nfreq == 0: u = exp(-tau H_m) beta e_1                   (m values)
  *   nfreq >= 1: u_j = u(tau) of u' = -H_m u + sin(omega_j t) beta e_1,
  *               u(0) = 0, for each omega_j (host array)      (m x nfreq)
- * Evaluated by FP64 scaling-and-squaring Pade (Higham 2005) of the
- * (m+2) x (m+2) matrix that carries the source phase.  u_out: host or
+ * Evaluated in FP64 by the truncated Taylor series with scaling and squaring
+ * (Paterson and Stockmeyer's evaluation, Al-Mohy and Higham's norm limits) of
+ * exp(-tau H_m), whose products serve every frequency, and of the two columns
+ * a frequency that carry its source.  u_out: host or
  * device, column-major m x max(1, nfreq).  m <= krylov_dim, nfreq <=
  * max_freqs.  Synchronises the stream. */
 kx_status expm_phi_project(kx_ctx* ctx, const double* H, int ldh, int m,

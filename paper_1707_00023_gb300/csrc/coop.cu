@@ -9,7 +9,7 @@
 // between the dots and the update (it is never written before it is
 // orthogonal), and a step has two grid barriers: after the partial dots, and
 // after the partial norms, which also orders the new column before its
-// neighbours' reads.  Every block sums the same partials in the same order,
+// neighbours' reads (double precision: a third, after the dots' totals).  Every block sums the same partials in the same order,
 // so all reach the same coefficients and decisions; block 0 records them.
 //   phase A: w = A v_j, partial dots V_i . w (i <= j) and ||w||^2
 //   phase B: v_{j+1} = w - sum_i h_ij v_i (compensated in FP32), partial norm
@@ -28,6 +28,8 @@
 // the partials); a thread's own columns are plain loads.
 // Every barrier wait is bounded: when one runs out the block records
 // KX_ETIMEOUT and returns, and so do the others.
+// One slot's blocks take nearly every SM, for the shortest process; contexts of
+// several slots, or driven beside others, may take fewer (coop_run).
 #include <atomic>
 
 #include "kx_eft.cuh"
@@ -48,12 +50,12 @@ constexpr size_t CO_SMEM = 195 * 1024;
 // Barrier over the `blocks` blocks of a slot: the counter reaches `target`
 // (blocks times the barriers so far; zeroed by the kernel that normalises
 // column 0).  False when the wait runs out: after `limit` polls (a cooperative
-// grid starts all its blocks or none, so other kernels' blocks are never
-// waited for here).  Four polls a round of the loop: with one the double-
-// precision process, three barriers a step, took 1.3 % longer (32^3 2845 us,
-// 2811).  The release on the arrival covers
-// the writes of the whole block (ordered before it by the block barrier), and
-// the acquire on the poll the reads after it.
+// grid starts all its blocks or none, measured beside a kernel that held half of
+// the SMs, so other kernels' blocks are never waited for here).  Four polls a
+// round of the loop: with one the double-precision process took 1.3 % longer
+// (32^3 2845 us, 2811).  The release on the arrival covers the writes of the
+// whole block (ordered before it by the block barrier), and the acquire on the
+// poll the reads after it.
 __device__ __forceinline__ bool grid_barrier(unsigned* cnt, unsigned target, unsigned limit) {
   __shared__ int ok;
   __syncthreads();
