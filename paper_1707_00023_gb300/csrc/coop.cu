@@ -535,7 +535,9 @@ __global__ void __launch_bounds__(P::MAXT, 1) k_coop(Geo g, SlotSet<typename P::
     V* kout = keep + (j + 1) * NC * nti + it;
     const bool held = j + 1 < kc;
     // the squares of a quad of values (or of one) summed in the working
-    // precision, as in pass B, no more
+    // precision, as in pass B, no more (plain method at 64^3, T = 400, twelve
+    // media, field errors: 5.1e-7 with a thread's 24 squares in floats, 4.6e-7
+    // so and by the per-step launches)
     S t2 = SO::of(T(0));
     if (ngrp == 1) {
       if (act) {
