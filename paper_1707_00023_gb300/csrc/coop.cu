@@ -737,12 +737,19 @@ kx_status coop_run(kx_ctx* c, int slot0, int ns, int want, int m, const void* g_
     cfg.numAttrs = 1;
     const double vb = (double)c->n * c->esize;
     time_begin(c);
-    cudaLaunchKernelEx(&cfg, k_coop<P, AUG>, c->geo, make_slotset<T>(c, slot0 + q), m, c->ld,
+    const cudaError_t e =
+        cudaLaunchKernelEx(&cfg, k_coop<P, AUG>, c->geo, make_slotset<T>(c, slot0 + q), m, c->ld,
                        (const T*)c->d_inv_eps, (const T*)c->d_sig2, (const T*)g_aug, c->m + 1,
                        sizeof(T) == 8 ? 1e-12 : 1e-6, p.nti, p.keep, c->wait_polls);
     // algorithmic bytes: per step v_j, V_0 .. V_{j-1} twice, v_{j+1}, 1/eps (and g)
     time_end(c, KX_K_PASS_A,
              nq * m * ((m + 2.0) * vb + (double)c->geo.ne * c->geo.ncell * c->esize + (g_aug ? vb : 0.0)));
+    if (e == cudaErrorCooperativeLaunchTooLarge && q == 0) {
+      // fewer multiprocessors than the device reports (a partition of it)
+      cudaGetLastError();
+      *ran = false;
+      return KX_OK;
+    }
     KX_CHECK_LAUNCH(c);
   }
   return KX_OK;
