@@ -534,18 +534,24 @@ __global__ void __launch_bounds__(P::MAXT, 1) k_coop(Geo g, SlotSet<typename P::
     T* out = Vc + (int64_t)(j + 1) * ld;
     V* kout = keep + (j + 1) * NC * nti + it;
     const bool held = j + 1 < kc;
-    // the squares of a quad of values (or of one) summed in the working
-    // precision, as in pass B, no more (plain method at 64^3, T = 400, twelve
+    // at most four squares (a quad's, or of three components of a cell) summed in
+    // the working precision, as in pass B (plain method at 64^3, T = 400, twelve
     // media, field errors: 5.1e-7 with a thread's 24 squares in floats, 4.6e-7
     // so and by the per-step launches)
+    constexpr int SQ = sizeof(V) > sizeof(T) ? 1 : 3;
     S t2 = SO::of(T(0));
+    T sq = T(0);
     if (ngrp == 1) {
       if (act) {
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
           o[c] = P::fold(o[c], lo[c]);
           P::store(out + c * nc, o[c]);
-          t2 = add(t2, P::dot(o[c], o[c]));
+          sq += P::dot(o[c], o[c]);
+          if (c % SQ == SQ - 1 || c == NC - 1) {
+            t2 = add(t2, sq);
+            sq = T(0);
+          }
         }
       }
       if (held) {
@@ -570,8 +576,13 @@ __global__ void __launch_bounds__(P::MAXT, 1) k_coop(Geo g, SlotSet<typename P::
           h = P::fold(h, l);
           P::store(out + c * nc, h);
           if (held) kout[c * nti] = h;
-          t2 = add(t2, P::dot(h, h));
+          sq += P::dot(h, h);   // cells: three components at most
+          if (SQ == 1) {
+            t2 = add(t2, sq);
+            sq = T(0);
+          }
         }
+      if (SQ > 1) t2 = add(t2, sq);
     }
     const S n2 = warp_total(t2);
     if (lane == 0) red[warp] = n2;
