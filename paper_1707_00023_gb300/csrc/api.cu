@@ -578,12 +578,12 @@ kx_status create_impl(const kx_desc* desc, const double* eps_cell, const uint8_t
     };
     for (const Alloc& a : rst) allocs[nalloc++] = a;
   }
-  // arrays of a mebibyte or more start on 2 MB boundaries, as allocations of
+  // arrays that L2 does not hold start on 2 MB boundaries, as allocations of
   // their own would: with the basis at a 256-byte offset the two passes of a
   // 96^3 process read it 2 % slower (pass B 7.40 against 7.24 ms, pass A 8.16
   // against 8.06; 72^3 3.32 against 3.27 and 4.12 against 4.09)
   auto place = [](size_t at, size_t bytes) {
-    const size_t a = bytes >= ((size_t)1 << 20) ? (size_t)1 << 21 : 256;
+    const size_t a = bytes >= ((size_t)128 << 20) ? (size_t)1 << 21 : 256;
     return (at + a - 1) / a * a;
   };
   size_t total = 0;
